@@ -103,16 +103,15 @@ typedef struct {
     double inf_rho, inf_U[3], inf_T; /* far-field state */
     int32_t precision;      /* UGKS_FP64 or UGKS_FP32 */
     const double *prim_init;/* [n_cells][dim+2] initial (rho, U, T), or NULL: far-field state */
-    int32_t patch_cells;    /* gather tiling: cells per patch (0: autotuned by timing the gather
-                               kernel on this case, cached per case shape) */
-    int32_t vtile;          /* gather tiling: velocities per tile, 32, 64 or 128 (0: automatic) */
-    int32_t gather_threads; /* gather tiling: threads per CTA, 256 or 512 (512 only for UGKS_FP32 with
+    int32_t patch_cells;    /* tiling of the flux pass: cells per CTA (0: autotuned by timing the pass on
+                               this case, cached per case shape) */
+    int32_t vtile;          /* velocities per warp of the flux pass, 32, 64 or 128 (0: automatic) */
+    int32_t gather_threads; /* threads per CTA of the flux pass, 256 or 512 (512 only for UGKS_FP32 with
                                vtile <= 64; 0: automatic, 256 unless the autotuner picks 512) */
-    int32_t gather_tile_group; /* gather grid order: the grid sweeps the patches once per group of this
-                               many velocity tiles, the tiles of a patch adjacent, so that a patch's
-                               face data are read once per group (1 .. 1024, larger values are
-                               clamped to the number of tiles; 0: chosen by the autotuner when
-                               patch_cells is 0, else 1) */
+    int32_t gather_tile_group; /* velocity tiles per moment group of stage 1: the moments of a cell's flux
+                               residual are summed over groups of this many tiles, the groups in FP64
+                               (1 .. 1024, larger values are clamped to the number of tiles, and to what
+                               the flux buffer may hold; 0: chosen from the sizes of the case) */
     int32_t w0_analytic;    /* interface equilibrium W0 (Sec. 2.4) from: 0 the discrete half-range
                                sums over the velocity set (default), 1 the analytic half-range
                                moments of the face-state Maxwellians over the continuous velocity
@@ -121,9 +120,8 @@ typedef struct {
 
 /* Device allocator.  alloc returns a device pointer of at least `bytes`
  * (256-byte aligned) usable on `stream`, or NULL; free releases it.  Blocks
- * are freed by ugks_destroy and by ugks_create when the autotuner replaces a
- * tiling's patch arrays, in both cases after the case stream has finished the
- * work that reads them. */
+ * are freed by ugks_destroy (and by ugks_halo_set, which replaces a list) after
+ * the case stream has finished the work that reads them. */
 typedef struct {
     void *ctx;
     void *(*alloc)(void *ctx, size_t bytes, void *stream);
@@ -139,15 +137,15 @@ typedef struct {
     int64_t step;              /* steps taken so far */
     size_t device_bytes;       /* device memory held by the case */
     size_t f_bytes;            /* bytes of one copy of f */
-    int32_t n_patches, patch_cells, vtile;  /* gather tiling in use */
+    int32_t n_patches, patch_cells, vtile;  /* tiling of the flux pass in use */
     int64_t kernel_launches_per_step;
     int64_t n_wall_faces;               /* faces of type UGKS_FACE_WALL */
-    int32_t gather_threads;             /* threads per CTA of the gather pass in use */
-    int32_t gather_tile_group;          /* velocity tiles per group of the gather grid in use */
+    int32_t gather_threads;             /* threads per CTA of the flux pass in use */
+    int32_t gather_tile_group;          /* velocity tiles per moment group of stage 1 in use */
 } ugks_info_t;
 
 /* Create a case: validates and copies the inputs, orders cells for locality,
- * builds least-squares coefficients and gather patches, allocates device state
+ * builds least-squares coefficients and face entries, allocates device state
  * and initialises f^0 = Maxwellian(W^0) (Sec. 3.1).  `stream` is a cudaStream_t
  * (NULL: the legacy default stream).  On success *out owns the device memory. */
 ugks_status ugks_create(const ugks_mesh *mesh, const ugks_vgrid *vgrid, const ugks_params *params,
@@ -239,10 +237,9 @@ ugks_status ugks_profile_begin(ugks_case *c, int32_t max_steps);
 ugks_status ugks_profile_end(ugks_case *c, double *ms, int32_t n, int32_t *steps);
 
 /* Batched stepping of several cases (one GPU).  The cases must share the
- * dimension and precision.  Each batch step runs every case's gather pass in
- * one persistent kernel per (velocity-tile width, block size) present in the
- * batch, which walks a (case, patch, velocity tile) work list, and each of the
- * step's other kernels once for all cases (block offsets per case), so a
+ * dimension and precision.  Each batch step runs every kernel once for all cases
+ * (block offsets per case), the flux and stage-1 kernels once per velocity chunk
+ * and per (velocity tile, block size, faces per cell) present in the batch, so a
  * step is about a dozen launches whatever the number of cases.  The whole
  * step is captured once as a CUDA graph on `stream` (cudaStream_t, NULL: a
  * stream of the batch's own) and replayed.  Results are bit-identical to
@@ -257,7 +254,7 @@ void ugks_batch_destroy(ugks_batch *b);
 /* ---- Serving loop (continuous batching of independent cases) ----
  * Requests arrive (at a time on the server clock); every ugks_server_tick
  * admits arrived requests, first fit in arrival order, while a slot is free
- * and the request's estimated device footprint (two copies of f plus the
+ * and the request's estimated device footprint (f, the flux buffer and the
  * O(cells + faces) arrays) fits the remaining budget; steps every running case
  * steps_per_tick times in batches (ugks_batch: one launch per kernel of the step
  * for all cases, CUDA-graph replay); then reads each running case's residual and retires

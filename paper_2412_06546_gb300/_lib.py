@@ -366,9 +366,8 @@ class Case:
 
 
 class Batch:
-    """Several cases stepped together: one persistent gather launch over a
-    (case, patch, velocity tile) work list per step, the whole step captured
-    once as a CUDA graph (``ugks_batch_*``)."""
+    """Several cases stepped together: every kernel of a step launched once over
+    all cases, the whole step captured once as a CUDA graph (``ugks_batch_*``)."""
 
     def __init__(self, cases, stream=None):
         L = load()

@@ -2,7 +2,7 @@
 // of the GB300 UGKS library (internal; not part of the C ABI).
 //
 // Layout in HBM (internal cell order = Morton order of the centroids):
-//   f      [C][NC][nvp]  T   distribution, NC = 2 (h, b) in 2D, 1 (h) in 3D,
+//   f      [C][NC][nvp]  T   distribution, updated in place, NC = 2 (h, b) in 2D, 1 (h) in 3D,
 //                            velocity contiguous, padded to a multiple of the
 //                            velocity tile (padded velocities have u = 0, w = 0)
 //   W      [C][D+2]      f64 conserved variables
@@ -29,36 +29,42 @@ enum { GR_U = 0, GR_LAM = 3, GR_PREF = 4, GR_NB = 5, GR_NL2 = 6, GREC = 8 };
 enum { FR_U = 0, FR_LAM = 3, FR_PREF = 4, FR_KQ = 5, FR_QS = 8, FR_NB = 13, FR_XB = 14,
        FR_BETA = 15, FR_NL2 = 39, FREC = 40 };
 
-// flux record read by the gather pass: the equilibrium part of the
+// flux record read by the flux pass: the equilibrium part of the
 // time-integrated interface distribution, q3 (g0 + g0+) + q4 u.grad g0 +
-// q5 dg0/dt, is H0(c) P_m(c) with c = u - U0 and, per stored component m,
-// P_m(c) = a0 + a.c + sum_{e<=f} B_ef c_e c_f + (gamma.c)|c|^2
-enum { XR_U = 0, XR_PREF = 3, XR_NL2 = 4, XR_LAM = 5, XR_Q1 = 6, XR_Q2 = 7, XR_POLY = 8, XREC = 24 };
+// q5 dg0/dt, is H0(c) P_m(c) with c = u - U0, H0 = PREF e^{-lam |c|^2} and, per
+// stored component m, P_m(c) = a0 + a.c + sum_{e<=f} B_ef c_e c_f + (gamma.c)|c|^2.
+// U = -U0; EX = the coefficient gauss_ex() takes (-lam, or -lam log2 e in FP32)
 template <int D> struct Poly {
     static constexpr int NB = D * (D + 1) / 2;
     static constexpr int N = 1 + D + NB + D;   // a0, a, B (packed upper, off-diagonal doubled), gamma
 };
+template <int D> struct XRec {
+    static constexpr int U = 0, EX = D, Q1 = D + 1, Q2 = D + 2, PREF = D + 3, POLY = D + 4;
+    static constexpr int LEN = (POLY + (4 - D) * Poly<D>::N + 3) / 4 * 4;   // 24 in 2D, 20 in 3D
+};
 
-enum { FT_INTERIOR = 0, FT_WALL = 1, FT_FARFIELD = 2, FT_PERIODIC = 3 };
+// FT_NONE: an entry that pads a cell to the entry count of the mesh
+enum { FT_INTERIOR = 0, FT_WALL = 1, FT_FARFIELD = 2, FT_PERIODIC = 3, FT_NONE = 4 };
 
 // nodes of the last velocity axis the separable half-range sums hold in shared memory
 constexpr int SUM1_SEP_MAX_NL = 512;
 
-// layout of the values of one gather entry (cell c, face f): a = LSQ
-// coefficient of the neighbour across f (0 for a wall), rs = x_f - x_c,
-// n = unit normal of f pointing out of c, ro = x_f - x_other (periodic image;
-// 0 for far-field ghosts), cs = -S_f / |Omega_c|.  Grouped in 16-byte vectors
-// so that each pass loads only the vectors it reads: the slopes' first face
-// loop the first SLOPE1 values (a, rs), their limiter loop the first vector
-// (rs), the flux loop everything but the vectors in [SKIP0, SKIP1) (a, in 3D).
+// largest face count the entries are padded to (hexahedra)
+constexpr int MAX_NF = 6;
+
+// layout of the values of one entry (cell c, face f): a = LSQ coefficient of
+// the neighbour across f (0 for a wall), rs = x_f - x_c, n = unit normal of f
+// pointing out of its owner, cs = -sigma S_f / |Omega_c| with sigma = 1 for the
+// owner and -1 for the neighbour, so that the flux F of f in the owner's
+// orientation enters c as cs F.  Grouped in 16-byte vectors so that each pass
+// loads only what it reads: a and rs by the slopes, rs and n by the fluxes, cs
+// by stage 1.
 template <int D> struct GEnt;
 template <> struct GEnt<2> {
-    static constexpr int A = 0, RS = 2, N = 4, RO = 6, CS = 8, LEN = 12;
-    static constexpr int SLOPE1 = 4, LIMIT = 4, SKIP0 = 0, SKIP1 = 0;
+    static constexpr int A = 0, RS = 2, N = 4, CS = 6, LEN = 8;
 };
 template <> struct GEnt<3> {
-    static constexpr int RS = 0, CS = 3, A = 4, N = 8, RO = 12, LEN = 16;
-    static constexpr int SLOPE1 = 8, LIMIT = 4, SKIP0 = 4, SKIP1 = 8;
+    static constexpr int RS = 0, CS = 3, A = 4, N = 8, LEN = 12;
 };
 
 // Everything a kernel needs, by value.  Geometry used inside velocity loops is
@@ -75,8 +81,11 @@ struct DevCase {
     const double *ud[3], *wd;
     const T *u[3], *w;
     const T *uw;                  // [nvp][4] (u_x, u_y, u_z or 0, w) packed for one vector load
-    // distribution: f_cur = f^n, f_nxt = f~ written by the gather pass
-    T *f_cur, *f_nxt;
+    // distribution, updated in place: f^n, then f~ (stage 1), then f^{n+1}
+    T *f_cur;
+    // time-integrated flux of every face in its owner's orientation for one
+    // chunk of velocities: [F][NC][chunk]
+    T *flux;
     // macroscopic state
     double *W, *q, *gradW, *vol;
     double *prim, *primg, *gradprim;  // primitive (rho, U, T) of cells / ghosts, limited gradient
@@ -90,13 +99,14 @@ struct DevCase {
     const double *cf_r_d;
     const T *cf_r;                // x_f - x_c (periodic image on the neighbour side)
     const T *cf_coef;             // -sigma S_f / |Omega_c|
-    // gather entries, one per (cell, face) in cf order, in the cell's own
-    // orientation: gi = {other, face, type, patch slot of other}, where other
-    // is the neighbour cell (interior, periodic), the ghost slot (far field) or
-    // the wall slot (wall); gf = GEnt<D> values (LSQ coefficient, offsets,
-    // outward normal, -S_f/|Omega_c|)
+    // entries, one per (cell, face) in cf order: gi = {row, face, type + 256
+    // (cell owns the face), ghost or wall slot} with row the neighbour cell
+    // (interior, periodic) or the cell itself; gf = GEnt<D> values.  nf > 0:
+    // every cell has nf entries (the largest face count of the mesh, if at most
+    // MAX_NF), padded with FT_NONE; nf = 0: the cells' own counts (cf_ptr)
     const int4 *gi;
     const T *gf;
+    int nf;
     const double *eps2_d;
     const T *eps2;
     // faces
@@ -105,6 +115,7 @@ struct DevCase {
     const double *fn_d, *frL_d, *frR_d;
     const T *fn, *frL, *frR;      // T copies used inside velocity loops
     T dtT;                        // dt in the arithmetic type
+    T one;                        // 1 (see psum)
     // ghosts (one per far-field face)
     const int *gface;
     double *Wg;                   // [G][D+2]
@@ -129,7 +140,7 @@ struct DevCase {
     double *fsum1, *fsum2;        // [F][S1], [F][S2]
     double *fprim0;               // [F][D+2] rho0, U0, lam0
     double *fqs;                  // [F][5] time integrals q1..q5 of the interface
-    double *dW_part;              // [C][n_groups][D+2] moments of the flux residual over a tile group
+    double *dW_part;              // [C][n_groups][D+2] moments of the flux residual over gvel velocities
     double *res_part;             // [n_res_blocks][2(D+2)]
     const unsigned char *owned;   // [C] 1 for cells whose residual counts (a subdomain's own cells),
                                   // nullptr: every cell
@@ -139,12 +150,11 @@ struct DevCase {
     int sep1;                     // sep with the last axis strictly ascending and at most
                                   // SUM1_SEP_MAX_NL nodes (separable half-range sums)
     const T *axis[3], *axw[3];
-    // gather tiling
-    int P, n_patches, n_vt, vtile;
-    int nth;                      // threads per gather CTA (256, or 512 for FP32 at TV <= 2)
-    int vt_group;                 // velocity tiles per gather CTA (see k_gather)
-    int n_groups;                 // tile groups: ceil(n_vt / vt_group)
-    const int *ring_ptr, *ring_cells;
+    // tiling of the flux and stage-1 passes
+    int P, n_patches, vtile;      // cells per CTA and velocities per warp of the flux pass
+    int nth;                      // threads per CTA of the flux pass (256, or 512 for FP32 at vtile <= 64)
+    int chunk, n_chunks;          // velocities per chunk (a multiple of gvel), chunks
+    int gvel, n_groups;           // velocities of a cell per warp of stage 1 (a multiple of vtile), groups per cell
 };
 
 // ------------------------------------------------------------------ math
@@ -378,20 +388,6 @@ __device__ __forceinline__ void ldv(const T *__restrict__ p, T (&x)[TV])
         for (int j = 0; j < CH; ++j) x[i * CH + j] = e[j];
     }
 }
-// the same from and to shared memory
-template <typename T, int TV>
-__device__ __forceinline__ void ldv_s(const T *p, T (&x)[TV])
-{
-    constexpr int CH = vec_chunk<T, TV>();
-    using V = typename VecOf<T, CH>::type;
-#pragma unroll
-    for (int i = 0; i < TV / CH; ++i) {
-        const V v = reinterpret_cast<const V *>(p)[i];
-        const T *e = reinterpret_cast<const T *>(&v);
-#pragma unroll
-        for (int j = 0; j < CH; ++j) x[i * CH + j] = e[j];
-    }
-}
 template <typename T, int TV>
 __device__ __forceinline__ void stv(T *p, const T (&x)[TV])
 {
@@ -453,6 +449,194 @@ __device__ __forceinline__ void load_uw(const double *__restrict__ uw, int k, do
     w = b.y;
 }
 
+// ------------------------------------------------------------ packs
+// The velocities of a lane are held in packs: pairs of FP32 values worked on by
+// the packed instructions (fma/add/mul .f32x2: the arithmetic of two velocities
+// per issued instruction at the rounding of the scalar ones; measured on GB300
+// at 1.87 packed against 3.6 scalar instructions per cycle and SM, so the
+// arithmetic rate is the same but half of the issue slots are free for loads,
+// compares and selects), single values otherwise.  Every contraction is
+// explicit, so all instantiations of a formula round alike.
+template <typename T, int TV> struct Pk {
+    static constexpr int W = 1, NP = TV;
+    using P = T;
+};
+template <> struct Pk<float, 2> {
+    static constexpr int W = 2, NP = 1;
+    using P = float2;
+};
+template <> struct Pk<float, 4> {
+    static constexpr int W = 2, NP = 2;
+    using P = float2;
+};
+
+__device__ __forceinline__ float pfma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ float pmul(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ float padd(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ double pfma(double a, double b, double c) { return __fma_rn(a, b, c); }
+__device__ __forceinline__ double pmul(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ double padd(double a, double b) { return __dadd_rn(a, b); }
+__device__ __forceinline__ float2 pfma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float2 pmul(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 padd(float2 a, float2 b) { return __fadd2_rn(a, b); }
+
+// the same value in every element
+template <typename P> __device__ __forceinline__ P pbc(double v);
+template <> __device__ __forceinline__ double pbc<double>(double v) { return v; }
+template <typename P> __device__ __forceinline__ P pbc(float v);
+template <> __device__ __forceinline__ float pbc<float>(float v) { return v; }
+template <> __device__ __forceinline__ float2 pbc<float2>(float v) { return make_float2(v, v); }
+
+// element j of a lane's velocities
+template <int W, typename P> __device__ __forceinline__ auto &pel(P *x, int j)
+{
+    if constexpr (W == 1) return x[j];
+    else return (j & 1) ? x[j >> 1].y : x[j >> 1].x;
+}
+
+// TV consecutive values into packs
+template <typename T, int TV>
+__device__ __forceinline__ void ldp(const T *__restrict__ p, typename Pk<T, TV>::P (&x)[Pk<T, TV>::NP])
+{
+    T v[TV];
+    ldv<T, TV>(p, v);
+#pragma unroll
+    for (int j = 0; j < TV; ++j) pel<Pk<T, TV>::W>(x, j) = v[j];
+}
+
+// a + b where a is a product that must not be contracted into the sum.  ptxas
+// fuses a packed multiplication and addition even where both carry .rn (the
+// scalar ones it leaves alone; measured: mul.rn.f32x2 + add.rn.f32x2 rounds
+// once), so the packed sum is an fma with a factor of 1 that the compiler does
+// not see, one = DevCase::one.
+__device__ __forceinline__ float psum(float a, float b, float) { return __fadd_rn(a, b); }
+__device__ __forceinline__ double psum(double a, double b, double) { return __dadd_rn(a, b); }
+__device__ __forceinline__ float2 psum(float2 a, float2 b, float one) { return __ffma2_rn(a, make_float2(one, one), b); }
+
+// u . n without contraction, as normal_velocity
+template <typename T, int D, typename P>
+__device__ __forceinline__ P pnormal(const P (&u)[D], const T *n, T one)
+{
+    P s = psum(pmul(u[0], pbc<P>(n[0])), pmul(u[1], pbc<P>(n[1])), one);
+    if constexpr (D == 3) s = psum(pmul(u[D - 1], pbc<P>(n[D - 1])), s, one);
+    return s;
+}
+
+// exp(-lam c2) from the record's coefficient (-lam; -lam log2 e in FP32)
+__device__ __forceinline__ float gauss_ex(float ex, float c2) { return ex2_approx(__fmul_rn(ex, c2)); }
+__device__ __forceinline__ double gauss_ex(double ex, double c2) { return exp(ex * c2); }
+
+// Sign tests and running extrema.  A double compare costs as much as an FP64
+// multiply (an SM retires 1.6 of either per cycle), so FP64 values are compared
+// as integers: the bits of a double order as its value for non-negative ones,
+// and for all after the magnitude bits of the negative ones are inverted.
+__device__ __forceinline__ bool gt0(float x) { return x > 0.f; }
+__device__ __forceinline__ bool lt0(float x) { return x < 0.f; }
+__device__ __forceinline__ bool gt0(double x) { return __double_as_longlong(x) > 0; }
+__device__ __forceinline__ bool lt0(double x)
+{
+    const long long b = __double_as_longlong(x);
+    return b < 0 && b != (long long)0x8000000000000000ull;
+}
+
+template <typename T> struct Extrema;
+template <> struct Extrema<float> {
+    float hi, lo;
+    __device__ __forceinline__ void set(float x) { hi = lo = x; }
+    __device__ __forceinline__ void add(float x)
+    {
+        hi = fmaxf(hi, x);
+        lo = fminf(lo, x);
+    }
+    // two values with one three-input instruction per extremum
+    __device__ __forceinline__ void add(float x, float y)
+    {
+        asm("max.f32 %0, %0, %1, %2;" : "+f"(hi) : "f"(x), "f"(y));
+        asm("min.f32 %0, %0, %1, %2;" : "+f"(lo) : "f"(x), "f"(y));
+    }
+    __device__ __forceinline__ float top() const { return hi; }
+    __device__ __forceinline__ float bottom() const { return lo; }
+};
+template <> struct Extrema<double> {
+    long long hi, lo;
+    static __device__ __forceinline__ long long key(double x)
+    {
+        const long long b = __double_as_longlong(x);
+        return b ^ ((b >> 63) & 0x7fffffffffffffffll);
+    }
+    static __device__ __forceinline__ double value(long long k)
+    {
+        return __longlong_as_double(k ^ ((k >> 63) & 0x7fffffffffffffffll));
+    }
+    __device__ __forceinline__ void set(double x) { hi = lo = key(x); }
+    __device__ __forceinline__ void add(double x)
+    {
+        const long long k = key(x);
+        hi = k > hi ? k : hi;
+        lo = k < lo ? k : lo;
+    }
+    __device__ __forceinline__ void add(double x, double y)
+    {
+        add(x);
+        add(y);
+    }
+    __device__ __forceinline__ double top() const { return value(hi); }
+    __device__ __forceinline__ double bottom() const { return value(lo); }
+};
+
+// a / b by the approximate reciprocal; b below the normal range counts as 0
+// (the callers discard or bound the quotient there)
+__device__ __forceinline__ float fdiv_ftz(float a, float b)
+{
+    float q;
+    asm("div.approx.ftz.f32 %0, %1, %2;" : "=f"(q) : "f"(a), "f"(b));
+    return q;
+}
+
+// min(1, n1 / d1, n2 / d2) of non-negative numerators and denominators; a
+// quotient 0 / 0 counts as 1.  FP32: fmin ignores the NaN of 0 / 0.  FP64: the
+// smaller quotient is found by cross products, so that one division is left.
+__device__ __forceinline__ float min_ratio(float n1, float d1, float n2, float d2)
+{
+    float r;
+    asm("min.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(fdiv_ftz(n1, d1)), "f"(fdiv_ftz(n2, d2)), "f"(1.f));
+    return r;
+}
+__device__ __forceinline__ double min_ratio(double n1, double d1, double n2, double d2)
+{
+    if (!gt0(d1)) n1 = d1 = 1.0;
+    if (!gt0(d2)) n2 = d2 = 1.0;
+    const bool first = __double_as_longlong(n1 * d2) < __double_as_longlong(n2 * d1);
+    const double n = first ? n1 : n2, d = first ? d1 : d2;
+    return __double_as_longlong(n) < __double_as_longlong(d) ? n / d : 1.0;
+}
+
+// phi theta of the positivity scaling: theta = f / (f - v) if v < 0 (0 if f <= 0;
+// FP32: or below the normal range, where fdiv_ftz would see 0 / 0)
+__device__ __forceinline__ float positive_scale(float phi, float f, float v)
+{
+    const float th = f >= 1.17549435e-38f ? fdiv_ftz(f, __fsub_rn(f, v)) : 0.f;
+    return v < 0.f ? phi * th : phi;
+}
+__device__ __forceinline__ double positive_scale(double phi, double f, double v)
+{
+    if (!lt0(v)) return phi;
+    return gt0(f) ? phi * (f / (f - v)) : 0.0;
+}
+
+// entries of cell c
+template <typename T>
+__device__ __forceinline__ void entry_range(const DevCase<T> &dc, int c, int &e0, int &ne)
+{
+    if (dc.nf > 0) {
+        e0 = c * dc.nf;
+        ne = dc.nf;
+    } else {
+        e0 = __ldg(dc.cf_ptr + c);
+        ne = __ldg(dc.cf_ptr + c + 1) - e0;
+    }
+}
+
 // Micro reconstruction of cell c (Sec. 3.1 Step 2) for the TV consecutive
 // velocities of this lane: least-squares slope grad = sum_j a_cj (f_j - f_c),
 // Venkatakrishnan factor phi = min over the faces of c of (D1^2 + eps^2 +
@@ -460,175 +644,207 @@ __device__ __forceinline__ void load_uw(const double *__restrict__ uw, int k, do
 // so that the reconstruction is non-negative at every face centre and at the
 // foot of the characteristic after one step: with dmin = min(0, min_f D2_f),
 // v = f_c + phi (dmin + min(0, -dt u.grad)); theta = f_c / (f_c - v) if v < 0.
-// Every face entry is read once for all TV velocities.  fl points at f_cur +
-// the lane's first velocity; fi returns f_c.  The face loops are unrolled so
-// that the entry and neighbour loads of several faces are in flight together
-// (the pass is bound by their latency).
-template <typename T, int D, int NC, int TV>
-__device__ __forceinline__ void cell_slope_tv(const DevCase<T> &dc, const T *__restrict__ fl, int c,
-                                              const T (&u)[3][TV], T (&g)[NC][D][TV], T (&fi)[NC][TV])
+// fl points at f_cur + the lane's first velocity; fi returns f_c, g the scaled
+// slope, ug = u . g.  NF > 0: ne == NF entries, their rows all requested before
+// the first is used; NF = 0: any number.  A wall or padding entry reads the
+// cell itself (no difference, no extremum).
+template <typename T, int D, int NC, int TV, int NF>
+__device__ __forceinline__ void cell_slope(const DevCase<T> &dc, const T *__restrict__ fl, const int c, const int e0,
+                                           const int ne, const typename Pk<T, TV>::P (&u)[Pk<T, TV>::NP][D],
+                                           typename Pk<T, TV>::P (&fi)[NC][Pk<T, TV>::NP],
+                                           typename Pk<T, TV>::P (&g)[NC][Pk<T, TV>::NP][D],
+                                           typename Pk<T, TV>::P (&ug)[NC][Pk<T, TV>::NP])
 {
     using E = GEnt<D>;
-    constexpr int HA = E::SLOPE1;                 // a and rs, in whole vector loads
+    using K = Pk<T, TV>;
+    using P = typename K::P;
+    constexpr int W = K::W, NP = K::NP;
     const int nvp = dc.nvp;
     const size_t rs = (size_t)NC * nvp;
-    T vmax[NC][TV], vmin[NC][TV];
     const T *fc = fl + (size_t)c * rs;
+    P nfi[NC][NP];
+    Extrema<T> ex[NC][TV];
 #pragma unroll
     for (int m = 0; m < NC; ++m) {
-        ldv<T, TV>(fc + (size_t)m * nvp, fi[m]);
+        ldp<T, TV>(fc + (size_t)m * nvp, fi[m]);
 #pragma unroll
-        for (int j = 0; j < TV; ++j) {
-            vmax[m][j] = vmin[m][j] = fi[m][j];
+        for (int i = 0; i < NP; ++i) {
+            nfi[m][i] = pmul(fi[m][i], pbc<P>(T(-1)));
 #pragma unroll
-            for (int d = 0; d < D; ++d) g[m][d][j] = 0;
+            for (int d = 0; d < D; ++d) g[m][i][d] = pbc<P>(T(0));
         }
+#pragma unroll
+        for (int j = 0; j < TV; ++j) ex[m][j].set(pel<W>(fi[m], j));
     }
-    const int e0 = __ldg(dc.cf_ptr + c), e1 = __ldg(dc.cf_ptr + c + 1);
-#pragma unroll 4
-    for (int e = e0; e < e1; ++e) {
-        const int4 gi = __ldg(dc.gi + e);
-        if (gi.z == FT_WALL) continue;
-        T ge[HA];
-        load_rec<HA>(dc.gf + (size_t)e * E::LEN, ge);
-        T fj[NC][TV];
-        if (gi.z == FT_FARFIELD) {
+    // f of the cell across an entry
+    auto across = [&](const int4 gi, P (&fj)[NC][NP]) {
+        const T *fo = fl + (size_t)gi.x * rs;
+#pragma unroll
+        for (int m = 0; m < NC; ++m) ldp<T, TV>(fo + (size_t)m * nvp, fj[m]);
+        if ((gi.z & 255) == FT_FARFIELD) {
             T gr[GREC];
-            load_rec<GREC>(dc.grec + (size_t)gi.x * GREC, gr);
+            load_rec<GREC>(dc.grec + (size_t)gi.w * GREC, gr);
 #pragma unroll
             for (int j = 0; j < TV; ++j) {
-                const T uj[3] = {u[0][j], u[1][j], u[2][j]};
-                const T H = maxwell_h<T, D>(gr, uj);
-                fj[0][j] = H;
-                if (NC == 2) fj[NC - 1][j] = gr[GR_NB] * H;
-            }
-        } else {
-            const T *fo = fl + (size_t)gi.x * rs;
+                T uj[3] = {T(0), T(0), T(0)};
 #pragma unroll
-            for (int m = 0; m < NC; ++m) ldv<T, TV>(fo + (size_t)m * nvp, fj[m]);
+                for (int d = 0; d < D; ++d) {
+                    P t[NP];
+#pragma unroll
+                    for (int i = 0; i < NP; ++i) t[i] = u[i][d];
+                    uj[d] = pel<W>(t, j);
+                }
+                const T H = maxwell_h<T, D>(gr, uj);
+                pel<W>(fj[0], j) = H;
+                if (NC == 2) pel<W>(fj[NC - 1], j) = gr[GR_NB] * H;
+            }
         }
+    };
+    auto slope_term = [&](const int e, P (&fj)[NC][NP]) {
+        T a[4];
+        load_rec<4>(dc.gf + (size_t)e * E::LEN + (E::A / 4) * 4, a);
+#pragma unroll
+        for (int m = 0; m < NC; ++m)
+#pragma unroll
+            for (int i = 0; i < NP; ++i) {
+                const P df = padd(fj[m][i], nfi[m][i]);
+#pragma unroll
+                for (int d = 0; d < D; ++d) g[m][i][d] = pfma(pbc<P>(a[E::A % 4 + d]), df, g[m][i][d]);
+            }
+    };
+    auto extrema = [&](P (&x)[NC][NP], P (&y)[NC][NP], bool both, auto &q) {
 #pragma unroll
         for (int m = 0; m < NC; ++m)
 #pragma unroll
             for (int j = 0; j < TV; ++j) {
-                const T df = fj[m][j] - fi[m][j];
-#pragma unroll
-                for (int d = 0; d < D; ++d) g[m][d][j] += ge[E::A + d] * df;
-                vmax[m][j] = fj[m][j] > vmax[m][j] ? fj[m][j] : vmax[m][j];
-                vmin[m][j] = fj[m][j] < vmin[m][j] ? fj[m][j] : vmin[m][j];
+                if (both) q[m][j].add(pel<W>(x[m], j), pel<W>(y[m], j));
+                else q[m][j].add(pel<W>(x[m], j));
             }
+    };
+    if constexpr (NF > 0) {
+        P fj[NF][NC][NP];
+#pragma unroll
+        for (int e = 0; e < NF; ++e) across(__ldg(dc.gi + e0 + e), fj[e]);
+#pragma unroll
+        for (int e = 0; e < NF; ++e) slope_term(e0 + e, fj[e]);
+#pragma unroll
+        for (int e = 0; e < NF; e += 2) extrema(fj[e], fj[e + 1 < NF ? e + 1 : e], e + 1 < NF, ex);
+    } else {
+        for (int e = 0; e < ne; ++e) {
+            P fj[NC][NP];
+            across(__ldg(dc.gi + e0 + e), fj);
+            slope_term(e0 + e, fj);
+            extrema(fj, fj, false, ex);
+        }
     }
-    const T e2 = __ldg(dc.eps2 + c);
     // Venkatakrishnan's factor at a face, phi(d2) = (a2 + 2 d1 d2) / (a2 + d2 (2 d2 + d1))
     // with a2 = d1^2 + eps^2 and d1 of the sign of d2, is at least 1 for
     // 0 <= d2/d1 <= 1/2 and strictly decreasing in |d2| beyond.  Its minimum over
     // the faces (clipped at 1) is therefore taken at the largest and at the most
     // negative d2, so the face loop only tracks those two, and phi is evaluated
     // twice per velocity instead of once per face.
-    T dmax[NC][TV], dmin[NC][TV];
+    Extrema<T> d2x[NC][TV];
 #pragma unroll
     for (int m = 0; m < NC; ++m)
 #pragma unroll
-        for (int j = 0; j < TV; ++j) dmax[m][j] = dmin[m][j] = T(0);
-#pragma unroll 4
-    for (int e = e0; e < e1; ++e) {
-        T ge[E::LIMIT];
-        load_rec<E::LIMIT>(dc.gf + (size_t)e * E::LEN, ge);
+        for (int j = 0; j < TV; ++j) d2x[m][j].set(T(0));
+    auto offset = [&](const int e, P (&d2)[NC][NP]) {
+        T r[4];
+        load_rec<4>(dc.gf + (size_t)e * E::LEN + (E::RS / 4) * 4, r);
 #pragma unroll
         for (int m = 0; m < NC; ++m)
 #pragma unroll
-            for (int j = 0; j < TV; ++j) {
-                T d2 = 0;
+            for (int i = 0; i < NP; ++i) {
+                P s = pmul(g[m][i][0], pbc<P>(r[E::RS % 4]));
 #pragma unroll
-                for (int d = 0; d < D; ++d) d2 += g[m][d][j] * ge[E::RS + d];
-                dmin[m][j] = d2 < dmin[m][j] ? d2 : dmin[m][j];
-                dmax[m][j] = d2 > dmax[m][j] ? d2 : dmax[m][j];
+                for (int d = 1; d < D; ++d) s = pfma(g[m][i][d], pbc<P>(r[E::RS % 4 + d]), s);
+                d2[m][i] = s;
             }
-    }
-    T phi[NC][TV];
+    };
+    if constexpr (NF > 0) {
 #pragma unroll
-    for (int m = 0; m < NC; ++m)
-#pragma unroll
-        for (int j = 0; j < TV; ++j) {
-            phi[m][j] = T(1);
-            if (dc.limiter) {
-                auto venk = [&](T d1, T d2) {
-                    const T a2 = d1 * d1 + e2;
-                    const T num = a2 + T(2) * d1 * d2;
-                    const T den = a2 + d2 * (T(2) * d2 + d1);
-                    return den > T(0) ? fdiv(num, den) : T(1);
-                };
-                if (dmax[m][j] > T(0)) {
-                    const T ph = venk(vmax[m][j] - fi[m][j], dmax[m][j]);
-                    phi[m][j] = ph < phi[m][j] ? ph : phi[m][j];
-                }
-                if (dmin[m][j] < T(0)) {
-                    const T ph = venk(vmin[m][j] - fi[m][j], dmin[m][j]);
-                    phi[m][j] = ph < phi[m][j] ? ph : phi[m][j];
-                }
-            }
+        for (int e = 0; e < NF; e += 2) {
+            P x[NC][NP], y[NC][NP];
+            offset(e0 + e, x);
+            if (e + 1 < NF) offset(e0 + e + 1, y);
+            extrema(x, y, e + 1 < NF, d2x);
         }
-    const T dt = dc.dtT;
+    } else {
+        for (int e = 0; e < ne; ++e) {
+            P x[NC][NP];
+            offset(e0 + e, x);
+            extrema(x, x, false, d2x);
+        }
+    }
+    const P e2 = pbc<P>(__ldg(dc.eps2 + c)), ndt = pbc<P>(-dc.dtT);
 #pragma unroll
     for (int m = 0; m < NC; ++m)
 #pragma unroll
-        for (int j = 0; j < TV; ++j) {
-            T ug = 0;
+        for (int i = 0; i < NP; ++i) {
+            P phi = pbc<P>(T(1)), dn, dp, low;
 #pragma unroll
-            for (int d = 0; d < D; ++d) ug += u[d][j] * g[m][d][j];
-            const T foot = -dt * ug;
-            const T v = fi[m][j] + phi[m][j] * (dmin[m][j] + (foot < T(0) ? foot : T(0)));
-            T sc = phi[m][j];
-            if (v < T(0)) sc *= fi[m][j] > T(0) ? fdiv(fi[m][j], fi[m][j] - v) : T(0);
+            for (int w = 0; w < W; ++w) {
+                pel<W>(&dp, w) = d2x[m][i * W + w].top();
+                pel<W>(&dn, w) = d2x[m][i * W + w].bottom();
+            }
+            if (dc.limiter) {
+                P hi, lo, num[2], den[2];
 #pragma unroll
-            for (int d = 0; d < D; ++d) g[m][d][j] *= sc;
+                for (int w = 0; w < W; ++w) {
+                    pel<W>(&hi, w) = ex[m][i * W + w].top();
+                    pel<W>(&lo, w) = ex[m][i * W + w].bottom();
+                }
+#pragma unroll
+                for (int s = 0; s < 2; ++s) {
+                    const P d1 = padd(s ? lo : hi, nfi[m][i]), d2 = s ? dn : dp;
+                    const P a2 = pfma(d1, d1, e2);
+                    num[s] = pfma(padd(d1, d1), d2, a2);
+                    den[s] = pfma(d2, pfma(pbc<P>(T(2)), d2, d1), a2);
+                }
+#pragma unroll
+                for (int w = 0; w < W; ++w)
+                    pel<W>(&phi, w) =
+                        min_ratio(pel<W>(num, w), pel<W>(den, w), pel<W>(num + 1, w), pel<W>(den + 1, w));
+            }
+            P s = pmul(u[i][0], g[m][i][0]);
+#pragma unroll
+            for (int d = 1; d < D; ++d) s = pfma(u[i][d], g[m][i][d], s);
+            const P foot = pmul(s, ndt);
+#pragma unroll
+            for (int w = 0; w < W; ++w) {
+                const T ft = pel<W>(const_cast<P *>(&foot), w);
+                pel<W>(&low, w) = lt0(ft) ? ft : T(0);
+            }
+            low = padd(dn, low);
+            P v = pfma(phi, low, fi[m][i]);
+#pragma unroll
+            for (int w = 0; w < W; ++w)
+                pel<W>(&phi, w) = positive_scale(pel<W>(&phi, w), pel<W>(&fi[m][i], w), pel<W>(&v, w));
+#pragma unroll
+            for (int d = 0; d < D; ++d) g[m][i][d] = pmul(g[m][i][d], phi);
+            s = pmul(u[i][0], g[m][i][0]);
+#pragma unroll
+            for (int d = 1; d < D; ++d) s = pfma(u[i][d], g[m][i][d], s);
+            ug[m][i] = s;
         }
 }
 
-// Interface flux of Eq. microscopicFlux with the distribution of Eq.
-// fullSolution integrated over the step (q1..q5):
-// F = u_n [q1 f_up + q2 u.grad f_up + H0(c) P(c)], the equilibrium part
-// q3 (g0 + g0+) + q4 u.grad g0 + q5 dg0/dt expanded into P (see XR_POLY).
-template <typename T, int D>
-__device__ __forceinline__ T poly_eval(const T *__restrict__ a, const T c[D], T c2)
+// P_m(c) of the flux record (see XRec)
+template <typename T, int D, typename P>
+__device__ __forceinline__ P poly_eval(const T *__restrict__ a, const P (&c)[D], const P c2)
 {
     constexpr int NB = Poly<D>::NB;
-    T p = a[0];
-#pragma unroll
-    for (int e = 0; e < D; ++e) p += a[1 + e] * c[e];
-    int t = 1 + D;
-    T q = 0;
+    P p = pbc<P>(a[0]), q, g;
 #pragma unroll
     for (int e = 0; e < D; ++e) {
-        T r = 0;
+        p = pfma(pbc<P>(a[1 + e]), c[e], p);
+        P r = pmul(pbc<P>(a[1 + D + (e * (2 * D - e + 1)) / 2]), c[e]);
 #pragma unroll
-        for (int f = e; f < D; ++f) r += a[t + (e * (2 * D - e + 1)) / 2 + (f - e)] * c[f];
-        q += r * c[e];
+        for (int f = e + 1; f < D; ++f) r = pfma(pbc<P>(a[1 + D + (e * (2 * D - e + 1)) / 2 + (f - e)]), c[f], r);
+        q = e == 0 ? pmul(r, c[0]) : pfma(r, c[e], q);
+        g = e == 0 ? pmul(pbc<P>(a[1 + D + NB]), c[0]) : pfma(pbc<P>(a[1 + D + NB + e]), c[e], g);
     }
-    p += q;
-    T g = 0;
-#pragma unroll
-    for (int e = 0; e < D; ++e) g += a[t + NB + e] * c[e];
-    return p + g * c2;
-}
-
-template <typename T, int D, int NC>
-__device__ __forceinline__ void interface_flux(const T *__restrict__ xr, const T u[3], T un,
-                                               const T fup[NC], const T ugf[NC], T F[NC])
-{
-    T c[D], c2 = 0;
-#pragma unroll
-    for (int d = 0; d < D; ++d) {
-        c[d] = u[d] - xr[XR_U + d];
-        c2 += c[d] * c[d];
-    }
-    const T H0 = xr[XR_PREF] * gauss<T>(xr[XR_LAM], xr[XR_NL2], c2);
-    const T q1 = xr[XR_Q1], q2 = xr[XR_Q2];
-#pragma unroll
-    for (int m = 0; m < NC; ++m) {
-        const T P = poly_eval<T, D>(xr + XR_POLY + m * Poly<D>::N, c, c2);
-        F[m] = un * (q1 * fup[m] + q2 * ugf[m] + H0 * P);
-    }
+    return pfma(g, c2, padd(p, q));
 }
 
 }  // namespace ugks

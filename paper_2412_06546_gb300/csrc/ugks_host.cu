@@ -56,11 +56,11 @@ struct ugks_case {
     bool user_alloc = false;
     std::vector<std::pair<void *, size_t>> blocks;
     size_t device_bytes = 0, f_bytes = 0;
-    size_t stage_bytes = 0;        // bytes of f_nxt, the staging area of state I/O (>= f_bytes)
+    size_t stage_bytes = 0;        // bytes of the flux buffer, the staging area of state I/O between steps
     ugks::DevCase<double> d64{};
     ugks::DevCase<float> d32{};
-    ugks::StepConfig cfg{};
-    int P = 0, vtile = 0, nth = 256, n_patches = 0, n_vt = 0, vt_group = 1, n_groups = 1;
+    int P = 0, vtile = 0, nth = 256, n_patches = 0, vt_group = 1;
+    int nf = 0, gvel = 0, n_groups = 1, chunk = 0, n_chunks = 1;
     long long *perm_d = nullptr;   // caller cell i -> internal cell
     std::vector<long long> perm_h; // the same on the host
     std::vector<long long> wall_face_h;   // face id of every wall slot
@@ -185,15 +185,14 @@ struct Host {
     std::vector<int> cf_ptr, cf_face;
     std::vector<signed char> cf_side;
     std::vector<double> cf_r, cf_coef;
-    std::vector<double> gf;          // gather entry values [ncf][GEnt<D>::LEN]
-    std::vector<int> gi;             // gather entry ids [ncf][4] (patch slots: build_patches)
+    std::vector<double> gf;          // entry values, GEnt<D>::LEN each
+    std::vector<int> gi;             // entry ids, 4 each
+    int nf = 0;                      // entries per cell (0: the cells' own counts)
     std::vector<int> nb_ptr, nb_id;
     std::vector<double> nb_a, eps2, vol;
     std::vector<int> fL, fR, faux, ftag, gface, wface;
     std::vector<signed char> ftype;
     std::vector<double> fn, frL, frR;
-    std::vector<int> ring_ptr, ring_cells;
-    int max_slope = 0;
 };
 
 // CFL time step of Algorithm 1 over the first n cells of the mesh:
@@ -315,9 +314,7 @@ bool invert_small(int D, const double *A, double *Ainv)
     return true;
 }
 
-void build_patches(Host &h, int C, int P);
-
-void preprocess(const ugks_mesh *m, const ugks_params *p, int P, Host &h)
+void preprocess(const ugks_mesh *m, const ugks_params *p, Host &h)
 {
     const int D = m->dim;
     const int C = (int)m->n_cells, F = (int)m->n_faces;
@@ -465,87 +462,48 @@ void preprocess(const ugks_mesh *m, const ugks_params *p, int P, Host &h)
         h.eps2[c] = Kh * Kh * Kh;
     }
 
-    // ---- gather entry values of every (cell, face), in the cell's own
-    //      orientation: LSQ coefficient, x_f - x_c, outward normal,
-    //      x_f - x_other, -S_f / |Omega_c|
+    // ---- entries of every (cell, face) (GEnt, DevCase::gi), padded to the same
+    //      count in every cell where that is at most MAX_NF
+    int most = 0;
+    for (int c = 0; c < C; ++c) most = std::max(most, h.cf_ptr[c + 1] - h.cf_ptr[c]);
+    // counts with kernels of their own: 3 and 4 in 2D, 4 and 6 in 3D
+    h.nf = most == 0 || most > ugks::MAX_NF ? 0 : D == 2 ? (most <= 3 ? 3 : most <= 4 ? 4 : 0) : (most <= 4 ? 4 : 6);
     const int GL = D == 2 ? ugks::GEnt<2>::LEN : ugks::GEnt<3>::LEN;
-    h.gf.assign((size_t)ncf * GL, 0.0);
+    const int oA = D == 2 ? ugks::GEnt<2>::A : ugks::GEnt<3>::A;
+    const int oRS = D == 2 ? ugks::GEnt<2>::RS : ugks::GEnt<3>::RS;
+    const int oN = D == 2 ? ugks::GEnt<2>::N : ugks::GEnt<3>::N;
+    const int oCS = D == 2 ? ugks::GEnt<2>::CS : ugks::GEnt<3>::CS;
+    const size_t n_ent = h.nf > 0 ? (size_t)C * h.nf : (size_t)ncf;
+    h.gf.assign(n_ent * GL, 0.0);
+    h.gi.assign(n_ent * 4, 0);
     for (int c = 0; c < C; ++c) {
         int q = h.nb_ptr[c];
-        for (int e = h.cf_ptr[c]; e < h.cf_ptr[c + 1]; ++e) {
+        size_t at = h.nf > 0 ? (size_t)c * h.nf : (size_t)h.cf_ptr[c];
+        const size_t end = h.nf > 0 ? at + h.nf : (size_t)h.cf_ptr[c + 1];
+        for (int e = h.cf_ptr[c]; e < h.cf_ptr[c + 1]; ++e, ++at) {
             const int f = h.cf_face[e], t = h.ftype[f];
-            const bool own = h.cf_side[e] == 0;
-            double *g = &h.gf[(size_t)e * GL];
-            const int oA = D == 2 ? ugks::GEnt<2>::A : ugks::GEnt<3>::A;
-            const int oRS = D == 2 ? ugks::GEnt<2>::RS : ugks::GEnt<3>::RS;
-            const int oN = D == 2 ? ugks::GEnt<2>::N : ugks::GEnt<3>::N;
-            const int oRO = D == 2 ? ugks::GEnt<2>::RO : ugks::GEnt<3>::RO;
-            const int oCS = D == 2 ? ugks::GEnt<2>::CS : ugks::GEnt<3>::CS;
+            const bool own = h.cf_side[e] == 0, inner = t == UGKS_FACE_INTERIOR || t == UGKS_FACE_PERIODIC;
+            double *g = &h.gf[at * GL];
+            int *gi = &h.gi[at * 4];
+            gi[0] = inner ? (own ? h.fR[f] : h.fL[f]) : c;
+            gi[1] = f;
+            gi[2] = t + (own ? 256 : 0);
+            gi[3] = inner ? 0 : h.faux[f];
             if (t != UGKS_FACE_WALL) {
                 for (int d = 0; d < D; ++d) g[oA + d] = h.nb_a[(size_t)q * D + d];
                 ++q;
             }
             for (int d = 0; d < D; ++d) {
                 g[oRS + d] = h.cf_r[(size_t)e * D + d];
-                g[oN + d] = own ? h.fn[(size_t)f * D + d] : -h.fn[(size_t)f * D + d];
-                if (t == UGKS_FACE_INTERIOR || t == UGKS_FACE_PERIODIC)
-                    g[oRO + d] = own ? h.frR[(size_t)f * D + d] : h.frL[(size_t)f * D + d];
+                g[oN + d] = h.fn[(size_t)f * D + d];
             }
-            g[oCS] = -m->face_S[f] / h.vol[c];
+            g[oCS] = (own ? -1.0 : 1.0) * m->face_S[f] / h.vol[c];
+        }
+        for (; at < end; ++at) {
+            h.gi[at * 4] = c;
+            h.gi[at * 4 + 2] = ugks::FT_NONE;
         }
     }
-
-    build_patches(h, C, P);
-}
-
-// gather patches: P consecutive cells (Morton order) and their face neighbours
-// (ring); slot indices of every face entry's owner / neighbour in its patch
-void build_patches(Host &h, int C, int P)
-{
-    const int ncf = h.cf_ptr[C];
-    h.ring_ptr.clear();
-    h.ring_cells.clear();
-    h.max_slope = 0;
-    const int np = (C + P - 1) / P;
-    h.ring_ptr.assign(np + 1, 0);
-    h.gi.assign((size_t)ncf * 4, -1);
-    std::vector<int> slot_of(C, -1);
-    for (int pi = 0; pi < np; ++pi) {
-        const int cb = pi * P, ce = std::min(C, cb + P);
-        for (int c = cb; c < ce; ++c) slot_of[c] = c - cb;
-        int ns = ce - cb;
-        std::vector<int> ring;
-        for (int c = cb; c < ce; ++c)
-            for (int e = h.cf_ptr[c]; e < h.cf_ptr[c + 1]; ++e) {
-                const int f = h.cf_face[e];
-                for (int o : {h.fL[f], h.fR[f]})
-                    if (o >= 0 && slot_of[o] < 0) {
-                        slot_of[o] = ns++;
-                        ring.push_back(o);
-                    }
-            }
-        // gather entries of the patch cells: {other, face, type, slot of other}
-        for (int c = cb; c < ce; ++c)
-            for (int e = h.cf_ptr[c]; e < h.cf_ptr[c + 1]; ++e) {
-                const int f = h.cf_face[e], t = h.ftype[f];
-                int *g = &h.gi[(size_t)e * 4];
-                if (t == UGKS_FACE_INTERIOR || t == UGKS_FACE_PERIODIC) {
-                    const int o = h.cf_side[e] == 0 ? h.fR[f] : h.fL[f];
-                    g[0] = o;
-                    g[3] = slot_of[o];
-                } else {
-                    g[0] = h.faux[f];
-                }
-                g[1] = f;
-                g[2] = t;
-            }
-        h.max_slope = std::max(h.max_slope, ns);
-        h.ring_cells.insert(h.ring_cells.end(), ring.begin(), ring.end());
-        h.ring_ptr[pi + 1] = (int)h.ring_cells.size();
-        for (int c = cb; c < ce; ++c) slot_of[c] = -1;
-        for (int o : ring) slot_of[o] = -1;
-    }
-    if (h.max_slope > 32767) fail(UGKS_EINVAL, "patch too large");
 }
 
 template <typename T>
@@ -661,11 +619,10 @@ void fill_case(ugks_case *c, ugks::DevCase<T> &dc, const ugks_mesh *m, const ugk
     // state
     const size_t fcount = (size_t)c->C * c->NC * c->nvp;
     dc.f_cur = (T *)c->dalloc(fcount * sizeof(T));
-    // f_nxt also stages state I/O, in host rows of up to FP64: room for at
-    // least two cells' FP64 rows (one per upload slot), even on tiny meshes
-    c->stage_bytes = std::max(fcount * sizeof(T), (size_t)2 * c->NC * c->nvp * sizeof(double));
-    dc.f_nxt = (T *)c->dalloc(c->stage_bytes);
-    c->f_bytes = fcount * sizeof(T);
+    // the flux buffer also stages state I/O, in host rows of up to FP64: room
+    // for at least two cells' FP64 rows (one per upload slot), even on tiny meshes
+    c->stage_bytes = std::max((size_t)c->F * c->NC * c->chunk * sizeof(T), (size_t)2 * c->NC * c->nvp * sizeof(double));
+    dc.flux = (T *)c->dalloc(c->stage_bytes);
     std::vector<double> W((size_t)c->C * M);
     for (int64_t i = 0; i < c->C; ++i) {
         const int ci = h.perm_u2i[i];
@@ -704,6 +661,7 @@ void fill_case(ugks_case *c, ugks::DevCase<T> &dc, const ugks_mesh *m, const ugk
     dc.cf_coef = c->upload(cast<T>(h.cf_coef));
     dc.gi = reinterpret_cast<const int4 *>(c->upload(h.gi));
     dc.gf = c->upload(cast<T>(h.gf));
+    dc.nf = h.nf;
     dc.eps2_d = c->upload(h.eps2);
     dc.eps2 = c->upload(cast<T>(h.eps2));
     dc.fL = c->upload(h.fL);
@@ -718,6 +676,7 @@ void fill_case(ugks_case *c, ugks::DevCase<T> &dc, const ugks_mesh *m, const ugk
     dc.frL = c->upload(cast<T>(h.frL));
     dc.frR = c->upload(cast<T>(h.frR));
     dc.dtT = (T)c->dt;
+    dc.one = T(1);
     dc.gface = c->upload(h.gface);
     dc.Wg = (double *)c->dalloc((size_t)std::max(c->G, 1) * M * sizeof(double));
     dc.grec = (T *)c->dalloc((size_t)std::max(c->G, 1) * ugks::GREC * sizeof(T));
@@ -750,7 +709,7 @@ void fill_case(ugks_case *c, ugks::DevCase<T> &dc, const ugks_mesh *m, const ugk
     dc.krec = (T *)c->dalloc((size_t)c->C * ugks::CREC * sizeof(T));
     const size_t Fm = (size_t)std::max<int64_t>(c->F, 1);
     dc.frec = (T *)c->dalloc(Fm * ugks::FREC * sizeof(T));
-    dc.xrec = (T *)c->dalloc(Fm * ugks::XREC * sizeof(T));
+    dc.xrec = (T *)c->dalloc(Fm * (D == 2 ? ugks::XRec<2>::LEN : ugks::XRec<3>::LEN) * sizeof(T));
     dc.fside = (T *)c->dalloc(Fm * 2 * ugks::GREC * sizeof(T));
     dc.fdW0 = (double *)c->dalloc(Fm * D * M * sizeof(double));
     dc.fq0 = (double *)c->dalloc(Fm * D * sizeof(double));
@@ -760,85 +719,84 @@ void fill_case(ugks_case *c, ugks::DevCase<T> &dc, const ugks_mesh *m, const ugk
     dc.fsum2 = (double *)c->dalloc(Fm * NS * (D + 1) * sizeof(double));
     dc.fprim0 = (double *)c->dalloc(Fm * M * sizeof(double));
     dc.fqs = (double *)c->dalloc(Fm * 5 * sizeof(double));
-    // sized for the smallest velocity tile, so that the autotuner may retile
-    dc.dW_part = (double *)c->dalloc((size_t)c->C * (c->nvp / 32) * M * sizeof(double));
+    dc.dW_part = (double *)c->dalloc((size_t)c->C * c->n_groups * M * sizeof(double));
     dc.res_part = (double *)c->dalloc((size_t)c->n_res_blocks * 2 * M * sizeof(double));
     dc.flags = c->flags_d;
     dc.owned = nullptr;
+    dc.gvel = c->gvel;
+    dc.n_groups = c->n_groups;
+    dc.chunk = c->chunk;
+    dc.n_chunks = c->n_chunks;
     dc.P = c->P;
     dc.nth = c->nth;
-    dc.vt_group = c->vt_group;
-    dc.n_groups = c->n_groups;
     dc.n_patches = c->n_patches;
-    dc.n_vt = c->n_vt;
     dc.vtile = c->vtile;
-    dc.ring_ptr = c->upload(h.ring_ptr);
-    dc.ring_cells = c->upload(h.ring_cells);
 }
 
 }  // namespace
 
 namespace {
 
-// Autotuner of the gather tiling: the patch size, the velocity tile and the
-// threads per CTA are chosen by timing the gather kernel itself on this case (it writes only f~
-// and scratch, so the state is untouched), and the choice is cached per
-// (dimension, precision, velocity count, mesh-size bucket) for later cases of
-// the same shape.
+// velocity tile used when neither the caller nor the autotuner sets one
+int kDefaultVtile(int prec) { return prec == UGKS_FP64 ? 32 : 64; }
+
+// Velocities per warp of stage 1 (gvel) and per chunk of the flux buffer.
+// A warp of stage 1 ends its group of velocities with a reduction over its lanes
+// that costs as much as about 250 velocities of the pass itself: groups of 1024,
+// fewer where the mesh has too few cells to fill the chip with one warp per cell
+// and group, or where the flux buffer of a group would exceed a copy of f.  (The
+// 107k-cell tetrahedral mesh x 4,568 velocities in FP32, flux and stage-1 passes:
+// 9.10, 8.30 and 7.95 ms at 256, 512 and 1024.)  The buffer holds as many
+// groups as fit 64 MB or a copy of f, whichever is smaller (4 MB are always
+// taken): fewer launches for small cases, little memory for large ones.
+void set_chunks(ugks_case *c, int tile_group)
+{
+    const int nvp = (int)c->nvp;
+    const size_t per_vel = (size_t)std::max<int64_t>(c->F, 1) * c->NC * (c->prec == UGKS_FP64 ? 8 : 4);
+    const size_t most = std::max((size_t)c->f_bytes, (size_t)4 << 20);
+    const int64_t warps = 152 * 32;
+    int groups = (nvp + 1023) / 1024, step = 128;
+    auto vel = [&] { return ((nvp + groups - 1) / groups + step - 1) / step * step; };
+    while (vel() > step && (c->C * groups < warps || vel() * per_vel > most)) ++groups;
+    c->gvel = std::min(vel(), nvp);
+    if (tile_group > 0) {
+        // the caller's group, as far as the buffer may hold it
+        const int64_t fit = std::max<int64_t>(1, (int64_t)(most / (per_vel * c->vtile)));
+        c->gvel = (int)std::min<int64_t>(std::min(tile_group, nvp / c->vtile), fit) * c->vtile;
+    }
+    c->n_groups = (nvp + c->gvel - 1) / c->gvel;
+    const size_t in = std::max<size_t>(1, std::min(most, (size_t)64 << 20) / (per_vel * c->gvel));
+    c->n_chunks = (int)((c->n_groups + in - 1) / in);
+    c->chunk = std::min((c->n_groups + c->n_chunks - 1) / c->n_chunks * c->gvel, nvp);
+    c->n_chunks = (nvp + c->chunk - 1) / c->chunk;
+}
+
+// Autotuner of the flux pass: cells per CTA, velocities per warp and threads per
+// CTA are chosen by timing the flux and stage-1 passes themselves on this case
+// (before the state is initialised for the caller), and the choice is cached
+// per (dimension, precision, velocity count, mesh-size bucket) for later cases
+// of the same shape.
 struct Tiling {
-    int P = 0, vtile = 0, nth = 256, G = 1;
+    int P = 0, vtile = 0, nth = 256;
 };
 std::mutex g_tune_mutex;
 std::map<std::string, Tiling> g_tune_cache;
 
-// dynamic shared memory of the gather: the moment accumulators (P x 16
-// values) and the slope buffer ((patch + ring) x NC x D x vtile values)
-size_t gather_smem(int max_slope, int NC, int D, int vtile, int P, size_t esz)
-{
-    return ((size_t)P * 16 + (size_t)max_slope * NC * D * vtile) * esz;
-}
-
-// velocity tile used when neither the caller nor the autotuner sets one
-int kDefaultVtile(int prec) { return prec == UGKS_FP64 ? 32 : 64; }
-
 template <typename T>
-void set_tiling(ugks_case *c, ugks::DevCase<T> &dc, const Host &h, int P, int vtile, int nth, int G, size_t smem)
+void set_tiling(ugks_case *c, ugks::DevCase<T> &dc, int P, int vtile, int nth)
 {
-    c->P = P;
-    c->n_patches = (int)((c->C + P - 1) / P);
-    c->vtile = vtile;
-    c->nth = nth;
-    c->n_vt = (int)(c->nvp / vtile);
-    c->vt_group = std::max(1, std::min(G, c->n_vt));
-    c->n_groups = (c->n_vt + c->vt_group - 1) / c->vt_group;
-    c->cfg.smem = smem;
-    dc.P = P;
-    dc.n_patches = c->n_patches;
-    dc.vtile = vtile;
-    dc.nth = nth;
-    dc.n_vt = c->n_vt;
-    dc.vt_group = c->vt_group;
-    dc.n_groups = c->n_groups;
-    // the old patch arrays may still be read by queued kernels: drain the
-    // stream first, so that any allocator may reuse them at once
-    if (dc.ring_ptr || dc.ring_cells || dc.gi)
-        cuda_ok(c->stream ? cudaStreamSynchronize(c->stream) : cudaDeviceSynchronize(), "retile sync");
-    c->dfree(dc.ring_ptr);
-    c->dfree(dc.ring_cells);
-    c->dfree(dc.gi);
-    dc.ring_ptr = c->upload(h.ring_ptr);
-    dc.ring_cells = c->upload(h.ring_cells);
-    dc.gi = reinterpret_cast<const int4 *>(c->upload(h.gi));
+    dc.P = c->P = P;
+    dc.n_patches = c->n_patches = (int)((c->C + P - 1) / P);
+    dc.vtile = c->vtile = vtile;
+    dc.nth = c->nth = nth;
 }
 
 template <typename T>
-void autotune(ugks_case *c, ugks::DevCase<T> &dc, Host &h, int smem_max, bool tune_vtile, bool tune_threads,
-              bool tune_group)
+void autotune(ugks_case *c, ugks::DevCase<T> &dc, bool tune_vtile, bool tune_threads)
 {
-    const size_t esz = sizeof(T);
     char key[160];
-    snprintf(key, sizeof(key), "D%d_nc%d_p%d_vt%d_t%d_g%d_nv%lld_c%d", c->D, c->NC, c->prec,
-             tune_vtile ? 0 : c->vtile, tune_threads ? 0 : c->nth, tune_group ? 0 : c->vt_group, (long long)c->Nv,
+    snprintf(key, sizeof(key), "D%d_nf%d_p%d_vt%d_t%d_g%d_nv%lld_c%d", c->D, c->nf, c->prec,
+             tune_vtile ? 0 : c->vtile, tune_threads ? 0 : c->nth, c->gvel, (long long)c->Nv,
              (int)std::lround(std::log2((double)c->C)));
     Tiling best;
     {
@@ -846,84 +804,41 @@ void autotune(ugks_case *c, ugks::DevCase<T> &dc, Host &h, int smem_max, bool tu
         auto it = g_tune_cache.find(key);
         if (it != g_tune_cache.end()) best = it->second;
     }
-    const int C = (int)c->C;
-    auto smem_of = [&](const Host &hh, int vt, int P) { return gather_smem(hh.max_slope, c->NC, c->D, vt, P, esz); };
     if (best.P == 0) {
-        // tetrahedra have more faces and larger rings than triangles, and one
-        // stored component per velocity: smaller patches and wider velocity tiles
-        const std::vector<int> pc = c->prec == UGKS_FP64 ? std::vector<int>{16, 24, 32, 48}
-                                    : c->D == 3          ? std::vector<int>{16, 24, 32, 48, 64, 96}
-                                                         : std::vector<int>{24, 32, 48, 64, 96};
-        std::vector<int> vc = {c->vtile};
-        if (tune_vtile) vc = c->D == 3 ? std::vector<int>{32, 64, 128} : std::vector<int>{32, 64};
-        // 512-thread CTAs (64 registers, two per SM) for FP32 at up to 64 velocities
-        std::vector<int> tc = {c->nth};
-        if (tune_threads) tc = c->prec == UGKS_FP32 ? std::vector<int>{256, 512} : std::vector<int>{256};
+        std::vector<int> vc = {c->vtile}, tc = {c->nth};
+        if (tune_vtile) vc = c->prec == UGKS_FP64 ? std::vector<int>{32, 64} : std::vector<int>{64, 128};
+        if (tune_threads && c->prec == UGKS_FP32) tc = {256, 512};
         cuda_ok(ugks::launch_pre_gather(dc, c->stream), "autotune prep");
         cudaEvent_t e0, e1;
         cuda_ok(cudaEventCreate(&e0), "event");
         cuda_ok(cudaEventCreate(&e1), "event");
-        auto time_gather = [&](size_t smem) {
-            cuda_ok(ugks::launch_gather(dc, smem, c->stream), "autotune gather");
-            cuda_ok(cudaEventRecord(e0, c->stream), "event");
-            for (int r = 0; r < 2; ++r) cuda_ok(ugks::launch_gather(dc, smem, c->stream), "autotune gather");
-            cuda_ok(cudaEventRecord(e1, c->stream), "event");
-            cuda_ok(cudaEventSynchronize(e1), "event");
-            float ms = 0.f;
-            cuda_ok(cudaEventElapsedTime(&ms, e0, e1), "event");
-            return ms;
-        };
-        const int G0 = c->vt_group;
         float best_ms = 0.f;
         for (int nth : tc)
             for (int vt : vc) {
-                if (c->nvp % vt || (nth == 512 && vt > 64)) continue;
-                for (int P : pc) {
-                    if (P > C && P != pc.front()) continue;
-                    if (nth == 512 && P < 32) continue;          // 16 warps need work
-                    build_patches(h, C, P);
-                    const size_t smem = smem_of(h, vt, P);
-                    if (smem > (size_t)smem_max) continue;
-                    set_tiling(c, dc, h, P, vt, nth, G0, smem);
-                    const float ms = time_gather(smem);
+                if ((c->chunk % vt && c->n_chunks > 1) || (nth == 512 && vt > 64)) continue;
+                for (int P : {8, 16, 32, 64}) {
+                    if (P < nth / 32) continue;          // a warp per cell
+                    if (P > 16 && P > c->C / 64) continue;
+                    set_tiling(c, dc, P, vt, nth);
+                    cuda_ok(ugks::launch_gather(dc, c->stream), "autotune gather");
+                    cuda_ok(cudaEventRecord(e0, c->stream), "event");
+                    for (int r = 0; r < 2; ++r) cuda_ok(ugks::launch_gather(dc, c->stream), "autotune gather");
+                    cuda_ok(cudaEventRecord(e1, c->stream), "event");
+                    cuda_ok(cudaEventSynchronize(e1), "event");
+                    float ms = 0.f;
+                    cuda_ok(cudaEventElapsedTime(&ms, e0, e1), "event");
                     if (best.P == 0 || ms < best_ms) {
-                        best = {P, vt, nth, G0};
+                        best = {P, vt, nth};
                         best_ms = ms;
                     }
                 }
             }
-        // then the grid order at the chosen tiling: groups of G velocity tiles
-        if (best.P != 0 && tune_group) {
-            build_patches(h, C, best.P);
-            const size_t smem = smem_of(h, best.vtile, best.P);
-            set_tiling(c, dc, h, best.P, best.vtile, best.nth, G0, smem);
-            for (int G : {1, 2, 4, 8, 16, 32, 64}) {
-                if (G == G0 || G > c->n_vt) continue;
-                dc.vt_group = G;
-                dc.n_groups = (c->n_vt + G - 1) / G;
-                const float ms = time_gather(smem);
-                if (ms < best_ms) {
-                    best.G = G;
-                    best_ms = ms;
-                }
-            }
-            dc.vt_group = c->vt_group;
-            dc.n_groups = c->n_groups;
-        }
         cudaEventDestroy(e0);
         cudaEventDestroy(e1);
-        if (best.P == 0) return;                 // keep the default tiling
         std::lock_guard<std::mutex> lock(g_tune_mutex);
         g_tune_cache[key] = best;
     }
-    if (best.P != c->P || best.vtile != c->vtile || best.nth != c->nth) {
-        build_patches(h, C, best.P);
-        const size_t smem = smem_of(h, best.vtile, best.P);
-        if (smem <= (size_t)smem_max) set_tiling(c, dc, h, best.P, best.vtile, best.nth, best.G, smem);
-    } else if (best.G != c->vt_group) {
-        c->vt_group = dc.vt_group = best.G;
-        c->n_groups = dc.n_groups = (c->n_vt + best.G - 1) / best.G;
-    }
+    set_tiling(c, dc, best.P, best.vtile, best.nth);
 }
 
 ugks_status guard(const std::function<void()> &fn)
@@ -955,7 +870,7 @@ auto with_dc(ugks_case *c, Fn &&fn)
 }
 
 // f of the case into host memory, f[C][ncomp][nv] of element type S in caller
-// cell order, staged through the f_nxt buffer in chunks of cells
+// cell order, staged through the flux buffer in chunks of cells
 template <typename S>
 void export_f(ugks_case *c, S *f)
 {
@@ -965,7 +880,7 @@ void export_f(ugks_case *c, S *f)
     for (int c0 = 0; c0 < (int)c->C; c0 += chunk) {
         const int nc = (int)std::min<int64_t>(chunk, c->C - c0);
         with_dc(c, [&](auto &dc) {
-            S *stg = (S *)dc.f_nxt;
+            S *stg = (S *)dc.flux;
             cuda_ok(ugks::launch_f_export(dc, c->perm_d, c0, nc, stg, c->stream), "f export");
             cuda_ok(cudaMemcpyAsync(f + (size_t)c0 * per, stg, (size_t)nc * per * sizeof(S), cudaMemcpyDeviceToHost,
                                     c->stream),
@@ -975,12 +890,12 @@ void export_f(ugks_case *c, S *f)
     }
 }
 
-// f from host memory (layout of export_f) into the case.  The f_nxt buffer is
+// f from host memory (layout of export_f) into the case.  The flux buffer is
 // split into two staging slots; chunks of cells alternate between them.  The
 // copy of a chunk runs on the case's copy stream while the case stream imports
 // (reorders and converts) the chunk before it; a slot is refilled only after
 // its previous import.  The first copy waits for the work already queued on
-// the case stream, which may still use f_nxt.
+// the case stream, which may still use the buffer.
 template <typename S>
 void import_f(ugks_case *c, const S *f)
 {
@@ -1001,7 +916,7 @@ void import_f(ugks_case *c, const S *f)
         const int sl = k & 1;
         if (k >= 2) cuda_ok(cudaStreamWaitEvent(c->copy_stream, consumed[sl], 0), "event wait");
         with_dc(c, [&](auto &dc) {
-            S *stg = (S *)dc.f_nxt + (size_t)sl * slot;
+            S *stg = (S *)dc.flux + (size_t)sl * slot;
             cuda_ok(cudaMemcpyAsync(stg, f + (size_t)c0 * per, (size_t)nc * per * sizeof(S), cudaMemcpyHostToDevice,
                                     c->copy_stream),
                     "f upload");
@@ -1088,42 +1003,24 @@ ugks_status ugks_create(const ugks_mesh *mesh, const ugks_vgrid *vgrid, const ug
             c->alloc = *alloc;
             c->user_alloc = true;
         }
-        const size_t esz = c->prec == UGKS_FP64 ? 8 : 4;
-        // tiling: velocity tile of 32*TV, patch of P cells sized to shared memory
         // velocity rows are padded to a multiple of the widest tile the autotuner
         // may choose (64 in 2D, 128 in 3D) unless the tile is fixed
         c->vtile = params->vtile > 0 ? params->vtile : kDefaultVtile(c->prec);
         c->nth = params->gather_threads > 0 ? params->gather_threads : 256;
         const int vpad = params->vtile > 0 ? params->vtile : (c->D == 3 ? 128 : 64);
-        int P = params->patch_cells > 0 ? params->patch_cells : (c->prec == UGKS_FP64 ? 32 : 48);
+        c->P = params->patch_cells > 0 ? params->patch_cells : 16;
         Host h;
-        int dev = 0;
-        cuda_ok(cudaGetDevice(&dev), "cudaGetDevice");
-        int smem_max = 0;
-        cuda_ok(cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev), "smem attr");
-        for (;;) {
-            h = Host();
-            preprocess(mesh, params, P, h);
-            const size_t smem = gather_smem(h.max_slope, c->NC, c->D, c->vtile, P, esz);
-            if (smem <= (size_t)smem_max || P <= 4) {
-                if (smem > (size_t)smem_max) fail(UGKS_EINVAL, "mesh stencil too large for shared memory");
-                c->cfg.smem = smem;
-                break;
-            }
-            P = std::max(4, P / 2);
-        }
-        c->P = P;
-        c->n_patches = (int)((c->C + P - 1) / P);
+        preprocess(mesh, params, h);
+        c->nf = h.nf;
+        c->n_patches = (int)((c->C + c->P - 1) / c->P);
         c->nvp = (c->Nv + vpad - 1) / vpad * vpad;
-        c->n_vt = (int)(c->nvp / c->vtile);
-        c->vt_group = std::max(1, std::min(params->gather_tile_group > 0 ? params->gather_tile_group : 1, c->n_vt));
-        c->n_groups = (c->n_vt + c->vt_group - 1) / c->vt_group;
+        c->f_bytes = (size_t)c->C * c->NC * c->nvp * (c->prec == UGKS_FP64 ? 8 : 4);
+        set_chunks(c.get(), params->gather_tile_group);
         c->G = (int)h.gface.size();
         c->NW = (int)h.wface.size();
         // upwind CFL bound (the CFL step of Algorithm 1)
         c->dt = params->dt > 0.0 ? params->dt : cfl_dt_of(mesh, vgrid, params->cfl, mesh->n_cells);
         c->n_res_blocks = (int)((c->C + 255) / 256);
-        c->cfg.n_res_blocks = c->n_res_blocks;
         c->flags_d = (int *)c->dalloc(sizeof(int));
         cuda_ok(cudaMemsetAsync(c->flags_d, 0, sizeof(int), c->stream), "memset");
         c->range_d = (unsigned long long *)c->dalloc(2 * sizeof(unsigned long long));
@@ -1131,19 +1028,18 @@ ugks_status ugks_create(const ugks_mesh *mesh, const ugks_vgrid *vgrid, const ug
         cuda_ok(cudaMemsetAsync(c->res_d, 0, 8 * sizeof(double), c->stream), "memset");
         c->perm_h.assign(h.perm_u2i.begin(), h.perm_u2i.end());
         c->perm_d = c->upload(c->perm_h);
-        if (c->prec == UGKS_FP64) {
-            fill_case<double>(c.get(), c->d64, mesh, vgrid, params, h);
-            cuda_ok(ugks::launch_init(c->d64, c->stream), "init");
-            if (params->patch_cells == 0)
-                autotune<double>(c.get(), c->d64, h, smem_max, params->vtile == 0, params->gather_threads == 0,
-                                 params->gather_tile_group == 0);
-        } else {
-            fill_case<float>(c.get(), c->d32, mesh, vgrid, params, h);
-            cuda_ok(ugks::launch_init(c->d32, c->stream), "init");
-            if (params->patch_cells == 0)
-                autotune<float>(c.get(), c->d32, h, smem_max, params->vtile == 0, params->gather_threads == 0,
-                                params->gather_tile_group == 0);
-        }
+        with_dc(c.get(), [&](auto &dc) {
+            fill_case(c.get(), dc, mesh, vgrid, params, h);
+            cuda_ok(ugks::launch_init(dc, c->stream), "init");
+            if (params->patch_cells == 0) {
+                // the trial passes overwrite f in place: initialise it again
+                autotune(c.get(), dc, params->vtile == 0, params->gather_threads == 0);
+                cuda_ok(ugks::launch_init(dc, c->stream), "init");
+            }
+            c->vt_group = params->gather_tile_group > 0
+                              ? (int)std::min<int64_t>(params->gather_tile_group, c->nvp / c->vtile)
+                              : std::max(1, c->gvel / c->vtile);
+        });
         cuda_ok(c->stream ? cudaStreamSynchronize(c->stream) : cudaDeviceSynchronize(), "create sync");
     });
     if (st != UGKS_OK) {
@@ -1164,7 +1060,7 @@ ugks_status ugks_step(ugks_case *c, int32_t nsteps)
         for (int32_t s = 0; s < nsteps; ++s) {
             cudaEvent_t *ev = nullptr;
             if (c->prof_used < c->prof_max) ev = &c->prof_ev[(size_t)c->prof_used++ * (ugks::N_GROUPS + 1)];
-            with_dc(c, [&](auto &dc) { cuda_ok(ugks::launch_step(dc, c->cfg, c->stream, ev), "step launch"); });
+            with_dc(c, [&](auto &dc) { cuda_ok(ugks::launch_step(dc, c->stream, ev), "step launch"); });
             ++c->step;
             c->stepped = true;
         }
@@ -1289,7 +1185,7 @@ ugks_status ugks_get_cells(ugks_case *c, const int64_t *cells, int64_t n, double
             ids[(size_t)i] = c->perm_h[(size_t)cells[i]];
         }
         // staging in the gradient scratch (C*D*M doubles >= n*(1 + M)): the
-        // internal ids, then W; f goes through the f~ buffer in chunks
+        // internal ids, then W; f goes through the flux buffer in chunks
         double *gW = c->prec == UGKS_FP64 ? c->d64.gradW : c->d32.gradW;
         long long *ids_d = reinterpret_cast<long long *>(gW);
         double *wst = gW + n;
@@ -1308,7 +1204,7 @@ ugks_status ugks_get_cells(ugks_case *c, const int64_t *cells, int64_t n, double
             for (int c0 = 0; c0 < (int)n; c0 += chunk) {
                 const int nc = (int)std::min<int64_t>(chunk, n - c0);
                 with_dc(c, [&](auto &dc) {
-                    double *stg = (double *)dc.f_nxt;
+                    double *stg = (double *)dc.flux;
                     cuda_ok(ugks::launch_f_export(dc, ids_d, c0, nc, stg, c->stream), "f gather");
                     cuda_ok(cudaMemcpyAsync(f + (size_t)c0 * per, stg, (size_t)nc * per * sizeof(double),
                                             cudaMemcpyDeviceToHost, c->stream),
@@ -1377,7 +1273,7 @@ ugks_status ugks_info(const ugks_case *c, ugks_info_t *info)
         info->vtile = c->vtile;
         info->gather_threads = c->nth;
         info->gather_tile_group = c->vt_group;
-        info->kernel_launches_per_step = 5 + (c->F > 0 ? 5 : 0) + (c->NW > 0 ? 1 : 0);
+        info->kernel_launches_per_step = 4 + 2 * c->n_chunks + (c->F > 0 ? 5 : 0) + (c->NW > 0 ? 1 : 0);
         info->n_wall_faces = c->NW;
     });
 }
@@ -1496,11 +1392,13 @@ struct ugks_batch {
     cudaStream_t stream = nullptr;
     bool own_stream = false;
     void *dcases = nullptr;         // device array of DevCase<T>
-    // one persistent gather launch per (velocity tile, threads per CTA) in the batch
+    // the flux and stage-1 passes, one launch each per chunk over the cases of a
+    // group (same velocity tile, threads per CTA and entry count): per chunk
+    // the block offsets of both kernels over all cases of the batch
     struct Group {
-        int vtile = 0, nth = 256, nwork = 0, grid = 0;
-        int4 *work = nullptr;
-        size_t smem = 0;
+        int vtile = 0, nth = 256, nf = 0, n_chunks = 0;
+        int *off = nullptr;                  // [n_chunks][2][n + 1]
+        std::vector<int> blocks;             // [n_chunks][2]
     };
     std::vector<Group> groups;
     // the other kernels of a step, one launch each over all cases: block offsets
@@ -1546,36 +1444,32 @@ void batch_build(ugks_batch *b)
     }
     cuda_ok(cudaMalloc((void **)&b->small_off, off.size() * sizeof(int)), "batch alloc");
     cuda_ok(cudaMemcpy(b->small_off, off.data(), off.size() * sizeof(int), cudaMemcpyHostToDevice), "batch upload");
-    // one persistent launch per (velocity tile, threads per CTA) in the batch
-    std::vector<std::pair<int, int>> tiles;
-    for (auto *c : b->cases)
-        if (std::find(tiles.begin(), tiles.end(), std::make_pair(c->vtile, c->nth)) == tiles.end())
-            tiles.push_back({c->vtile, c->nth});
-    for (const auto &tt : tiles) {
-        const int vtile = tt.first, nth = tt.second;
-        auto in_group = [&](const ugks_case *c) { return c->vtile == vtile && c->nth == nth; };
+    for (auto *first : b->cases) {
+        auto in_group = [&](const ugks_case *c) {
+            return c->vtile == first->vtile && c->nth == first->nth && c->nf == first->nf;
+        };
+        if (first != *std::find_if(b->cases.begin(), b->cases.end(), in_group)) continue;   // its group is there
         ugks_batch::Group g;
-        g.vtile = vtile;
-        g.nth = nth;
-        std::vector<int4> work;
-        int max_grp = 0;
-        for (int i = 0; i < n; ++i)
-            if (in_group(b->cases[i])) {
-                g.smem = std::max(g.smem, b->cases[i]->cfg.smem);
-                max_grp = std::max(max_grp, b->cases[i]->n_groups);
+        g.vtile = first->vtile;
+        g.nth = first->nth;
+        g.nf = first->nf;
+        for (auto *c : b->cases)
+            if (in_group(c)) g.n_chunks = std::max(g.n_chunks, c->n_chunks);
+        std::vector<int> goff((size_t)g.n_chunks * 2 * (n + 1), 0);
+        for (int r = 0; r < g.n_chunks; ++r)
+            for (int k = 0; k < 2; ++k) {
+                int *o = &goff[((size_t)r * 2 + k) * (n + 1)];
+                for (int i = 0; i < n; ++i) {
+                    long long nb = o[i];
+                    if (in_group(b->cases[i])) nb += k == 0 ? ugks::flux_blocks<T>(h[i], r) : ugks::stage1_blocks<T>(h[i], r);
+                    if (nb > INT32_MAX) fail(UGKS_EINVAL, "batch too large for one launch of the flux pass");
+                    o[i + 1] = (int)nb;
+                }
+                g.blocks.push_back(o[n]);
             }
-        // tile group outer, case, then patch innermost: consecutive CTAs work
-        // on neighbouring patches of one case and group, as in the single-case grid
-        for (int gr = 0; gr < max_grp; ++gr)
-            for (int i = 0; i < n; ++i) {
-                if (!in_group(b->cases[i]) || gr >= b->cases[i]->n_groups) continue;
-                for (int pi = 0; pi < b->cases[i]->n_patches; ++pi) work.push_back(make_int4(i, pi, gr, 0));
-            }
-        cuda_ok(cudaMalloc((void **)&g.work, sizeof(int4) * std::max<size_t>(1, work.size())), "batch alloc");
+        cuda_ok(cudaMalloc((void **)&g.off, goff.size() * sizeof(int)), "batch alloc");
         b->groups.push_back(g);      // owned by the batch from here on
-        cuda_ok(cudaMemcpy(g.work, work.data(), sizeof(int4) * work.size(), cudaMemcpyHostToDevice), "batch upload");
-        b->groups.back().nwork = (int)work.size();
-        b->groups.back().grid = std::min((int)work.size(), ugks::gather_resident_ctas<T>(b->D, vtile, nth, g.smem));
+        cuda_ok(cudaMemcpy(g.off, goff.data(), goff.size() * sizeof(int), cudaMemcpyHostToDevice), "batch upload");
     }
 }
 
@@ -1593,9 +1487,13 @@ void batch_capture(ugks_batch *b)
     cuda_ok(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal), "begin capture");
     for (int k = ugks::SK_PREP; k <= ugks::SK_WALL_SUM; ++k) small(k);
     for (const auto &g : b->groups)
-        cuda_ok(ugks::launch_gather_batch<T>(b->D, g.vtile, g.nth, (const ugks::DevCase<T> *)b->dcases, g.work,
-                                             g.nwork, g.grid, g.smem, st),
-                "batched gather");
+        for (int r = 0; r < g.n_chunks; ++r) {
+            const int *off = g.off + (size_t)r * 2 * (n + 1);
+            cuda_ok(ugks::launch_flux<T>(b->D, g.nf, g.vtile, g.nth, g.blocks[2 * r], r, st, nullptr, dcs, off, n),
+                    "batched flux pass");
+            cuda_ok(ugks::launch_stage1<T>(b->D, g.nf, g.blocks[2 * r + 1], r, st, nullptr, dcs, off + n + 1, n),
+                    "batched stage 1");
+        }
     small(ugks::SK_UPDATE_W);
     small(ugks::SK_COLLIDE);
     cuda_ok(cudaStreamEndCapture(st, &b->graph), "end capture");
@@ -1609,7 +1507,7 @@ void batch_free(ugks_batch *b)
     if (b->graph) cudaGraphDestroy(b->graph);
     if (b->dcases) cudaFree(b->dcases);
     for (auto &g : b->groups)
-        if (g.work) cudaFree(g.work);
+        if (g.off) cudaFree(g.off);
     if (b->small_off) cudaFree(b->small_off);
     for (auto e : b->case_ev)
         if (e) cudaEventDestroy(e);

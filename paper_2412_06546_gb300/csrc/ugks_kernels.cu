@@ -9,8 +9,8 @@
 //   k_face_sum2   moments of g0 for the slope systems                    (Sec. 2.4)
 //   k_face_fin2   spatial and time slopes of g0                          (Sec. 2.4)
 //   k_wall_sum    wall density from zero net mass flux                   (Eq. maxWalldes)
-//   k_gather      per (cell patch, velocity tile): micro slopes, face fluxes, stage 1,
-//                 moments of the flux residual                           (velocity loop, Eq. microS1)
+//   k_flux        micro slopes and the outgoing face fluxes               (velocity loop)
+//   k_stage1      flux balance, stage 1, moments of the flux residual     (velocity loop, Eq. microS1)
 //   k_update_W    W^{n+1} and stage-2 coefficients                       (Eq. macroscopicUpdata)
 //   k_collide     stage 2 and the heat flux of f^{n+1}                   (Eq. microS2)
 // All per-velocity arithmetic is in T (double or float).  Velocity-moment sums
@@ -18,7 +18,7 @@
 // sums are accumulated in FP64: the face sums from FP32 block partials of at
 // most SUM_BLOCK terms per lane (see block_to_fp64), the wall density and the
 // heat flux from Kahan-compensated lane sums, the moments of the flux residual
-// from double-float lane and warp sums.  Macroscopic scalars (W, the
+// from double-float lane and warp sums (k_stage1).  Macroscopic scalars (W, the
 // equilibrium parameters, the heat flux, the collision coefficients) are
 // formed in FP64.
 #include "ugks_device.cuh"
@@ -1218,13 +1218,13 @@ __device__ __forceinline__ void face_fin2_body(const DevCase<T> &dc, const int b
     double kq[D];
     for (int d = 0; d < D; ++d) kq[d] = kappa * dc.fq0[(size_t)f * D + d];
     const double *qs = dc.fqs + (size_t)f * 5;   // time integrals of k_face_fin1
-    T *x = dc.xrec + (size_t)f * XREC;
-    for (int d = 0; d < 3; ++d) x[XR_U + d] = d < D ? (T)U0[d] : T(0);
-    x[XR_PREF] = (T)pref_of(rho0, lam0, D);
-    x[XR_NL2] = (T)(-lam0 * LOG2E);
-    x[XR_LAM] = (T)lam0;
-    x[XR_Q1] = (T)qs[0];
-    x[XR_Q2] = (T)qs[1];
+    using X = XRec<D>;
+    T *x = dc.xrec + (size_t)f * X::LEN;
+    for (int d = 0; d < D; ++d) x[X::U + d] = (T)-U0[d];
+    x[X::EX] = (T)(std::is_same<T, float>::value ? -lam0 * LOG2E : -lam0);
+    x[X::Q1] = (T)qs[0];
+    x[X::Q2] = (T)qs[1];
+    x[X::PREF] = (T)pref_of(rho0, lam0, D);
     constexpr int NB = Poly<D>::NB, NP = Poly<D>::N;
     for (int m = 0; m < NC; ++m) {
         const double sm = m == 0 ? 1.0 : nb;            // scale of the b moments
@@ -1254,7 +1254,7 @@ __device__ __forceinline__ void face_fin2_body(const DevCase<T> &dc, const int b
         a0 += qs[4] * alphaA;
         for (int e = 0; e < D; ++e) a[e] += qs[4] * sm * xa[1 + e];
         diag += qs[4] * 0.5 * sm * xa[D + 1];
-        T *pm = x + XR_POLY + m * NP;
+        T *pm = x + X::POLY + m * NP;
         pm[0] = (T)a0;
         for (int e = 0; e < D; ++e) pm[1 + e] = (T)a[e];
         int t = 1 + D;
@@ -1317,8 +1317,12 @@ __device__ __forceinline__ void wall_sum_body(const DevCase<T> &dc, const int bx
     // unit-density wall Maxwellian over the step, so that F_w = A + rho_w B
     CSum<T> v[NR];
     // TW consecutive velocities per thread: the wall cell's limited slope
-    // (the gather's slope routine) reads each face entry once for all of them
+    // (cell_slope) reads each face entry once for all of them
     constexpr int TW = 4;
+    using K = Pk<T, TW>;
+    using P = typename K::P;
+    int e0, ne;
+    entry_range(dc, c, e0, ne);
     for (int k0 = TW * threadIdx.x; k0 < dc.nvp; k0 += TW * blockDim.x) {
         T u[3][TW], wk[TW], un[TW];
         ldv<T, TW>(dc.u[0] + k0, u[0]);
@@ -1335,30 +1339,29 @@ __device__ __forceinline__ void wall_sum_body(const DevCase<T> &dc, const int bx
             un[j] = normal_velocity<T, D>(uj, n);
             out = out || un[j] > T(0);
         }
-        T g[NC][D][TW], fi[NC][TW];
-        if (out) cell_slope_tv<T, D, NC, TW>(dc, dc.f_cur + k0, c, u, g, fi);
+        P up[K::NP][D], g[NC][K::NP][D], fi[NC][K::NP], ug[NC][K::NP];
+#pragma unroll
+        for (int j = 0; j < TW; ++j)
+#pragma unroll
+            for (int d = 0; d < D; ++d) pel<K::W>(&up[j / K::W][d], j % K::W) = u[d][j];
+        if (out) cell_slope<T, D, NC, TW, 0>(dc, dc.f_cur + k0, c, e0, ne, up, fi, g, ug);
 #pragma unroll
         for (int j = 0; j < TW; ++j) {
             const T uj[3] = {u[0][j], u[1][j], u[2][j]};
             T Fh = 0, Fb = 0;
             int off = -1;
             if (un[j] > T(0)) {
-                T hin = fi[0][j], ug = 0;
+                T hin = pel<K::W>(fi[0], j);
 #pragma unroll
-                for (int d = 0; d < D; ++d) {
-                    hin += g[0][d][j] * r[d];
-                    ug += uj[d] * g[0][d][j];
-                }
-                v[0].add(wk[j] * un[j] * (hin - hdt * ug));
-                Fh = dt * un[j] * (hin - hdt * ug);
+                for (int d = 0; d < D; ++d) hin += pel<K::W>(&g[0][j / K::W][d], j % K::W) * r[d];
+                const T uga = pel<K::W>(ug[0], j);
+                v[0].add(wk[j] * un[j] * (hin - hdt * uga));
+                Fh = dt * un[j] * (hin - hdt * uga);
                 if (NC == 2) {
-                    T bin = fi[NC - 1][j], ugb = 0;
+                    T bin = pel<K::W>(fi[NC - 1], j);
 #pragma unroll
-                    for (int d = 0; d < D; ++d) {
-                        bin += g[NC - 1][d][j] * r[d];
-                        ugb += uj[d] * g[NC - 1][d][j];
-                    }
-                    Fb = dt * un[j] * (bin - hdt * ugb);
+                    for (int d = 0; d < D; ++d) bin += pel<K::W>(&g[NC - 1][j / K::W][d], j % K::W) * r[d];
+                    Fb = dt * un[j] * (bin - hdt * pel<K::W>(ug[NC - 1], j));
                 }
                 off = 2;
             } else if (un[j] < T(0)) {
@@ -1421,321 +1424,384 @@ __global__ void __launch_bounds__(256) k_wall_sum_batch(const DevCase<T> *__rest
 }
 
 // ------------------------------------------------------------ gather pass
-// One CTA per (patch of P consecutive cells, group of G = vt_group consecutive
-// velocity tiles of V = 32*TV velocities); the CTA takes the group's tiles one
-// after the other, and in a tile lane l handles the TV consecutive velocities
-// V*tile + TV*l + j.  Per tile:
-// Phase A: limited slopes of the patch cells and their face neighbours (ring)
-//          into shared memory, each computed once.
-// Phase B: per patch cell, the flux of every face (Eq. microscopicFlux with
-//          Eq. fullSolution; walls per Sec. 2.5) in the cell's own
-//          orientation, stage 1 (Eq. microS1) written to f_nxt, and the moments
-//          sum_k w psi_k R_k of the flux residual for the W update (Eq.
-//          macroscopicUpdata / macroscopicFlux).  The cell's own f and slopes
-//          stay in registers; every face entry is read once for all TV
-//          velocities of the lane.
-// The moments of a cell accumulate over the group's tiles in shared memory
-// (the warp that owns a cell is the same for every tile) and are written once
-// per (cell, group).  Consecutive tiles of a patch re-read its face entries
-// and records from the SM's cache.
-//
-// Shared memory: the moment accumulators, P x 16 values of T (FP32: the
-// double-float pair of each of up to 8 moments; FP64: the moments), then the
-// slope buffer, (patch + ring) x NC x D x V values of T.
-template <typename T>
-__host__ __device__ constexpr int gather_acc_values(int P) { return P * 16; }
+// The velocity loop of Algorithm 1 in two passes over a chunk of velocities,
+// with the chunk's face fluxes in between:
+//   k_flux    every cell's limited slopes (each once), and from the registers
+//             that hold them the time-integrated flux (Eq. microscopicFlux with
+//             Eq. fullSolution; walls per Sec. 2.5) of those velocities that
+//             leave the cell, through each of its faces.  A velocity crosses a
+//             face from one side, so every flux is evaluated and stored once,
+//             by the cell it comes from; a boundary face's cell stores both
+//             directions.
+//   k_stage1  per cell the sum of its faces' fluxes, stage 1 (Eq. microS1) in
+//             place, and the moments sum_k w psi_k R_k of the flux residual for
+//             the W update (Eq. macroscopicUpdata / macroscopicFlux).
+// One pass over patches of cells that kept the slopes in shared memory spent
+// most of its instructions on slopes recomputed for the neighbours of a patch
+// (2.2 evaluations per cell of 48-cell patches), on fluxes evaluated from both
+// sides of a face and on selects between the sides: 897 thread instructions
+// per cell-velocity for tetrahedra against 286 of the two kernels here
+// (k_flux 194, k_stage1 92 at 256-velocity groups).  The price is the flux
+// buffer, F/C values per cell and velocity written once and read twice, which
+// L2 and HBM have room for.  107k-cell tetrahedral mesh x 4,568 velocities,
+// FP32: 17.2 -> 7.95 ms; 24k cells x 28^3: 18.4 -> 8.2 ms; 30k triangles x
+// 60x50: 3.18 -> 1.55 ms; FP64, 8k triangles x 60x50: 21.0 -> 13.4 ms.
+// A chunk bounds the buffer; velocities of different chunks do not meet, so
+// the update is in place.
 
-template <typename T, int D, int NC, int TV>
-__device__ __forceinline__ void gather_item(const DevCase<T> &dc, const int p, const int grp, T *sg)
+// One warp per cell and tile of 32 TV velocities, TV consecutive ones per lane;
+// the warps of a CTA take the P cells of a patch in turn.  Bound: instruction
+// issue and the latency of the neighbours' rows (16 warps per SM; DRAM at 9 % of
+// its peak).  TV = 4 reads an entry or a record for twice the velocities of
+// TV = 2 (107k-cell tetrahedral mesh: 9.1 against 12.4 ms of both kernels).
+template <typename T, int D, int NC, int TV, int NF>
+__device__ __forceinline__ void flux_body(const DevCase<T> &dc, const int bx, const int chunk)
 {
-    constexpr int V = 32 * TV;
-    constexpr int M = D + 2;
-    // velocities per lane of the slope pass: twice TV in the FP32 form with one
-    // stored component (a half-warp per slope cell), else TV (registers)
-    constexpr int TVA = std::is_same<T, float>::value && NC == 1 && TV <= 2 ? 2 * TV : TV;
     using E = GEnt<D>;
+    using X = XRec<D>;
+    using K = Pk<T, TV>;
+    using P = typename K::P;
+    constexpr int W = K::W, NP = K::NP, V = 32 * TV;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-    const int cb = p * dc.P;
-    const int npc = min(dc.P, dc.C - cb);
-    const int rb = dc.ring_ptr[p], re = dc.ring_ptr[p + 1];
-    const int nslope = npc + (re - rb);
-    const int nvp = dc.nvp;
-    const size_t rs = (size_t)NC * nvp;
-    T *const sacc = sg;                         // moment accumulators [P][16]
-    T *const sl = sg + gather_acc_values<T>(dc.P) + TV * lane;   // this lane's column of the slope buffer
-    for (int i = threadIdx.x; i < gather_acc_values<T>(dc.P); i += blockDim.x) sacc[i] = T(0);
-    const int vt0 = grp * dc.vt_group, vt1 = min(dc.n_vt, vt0 + dc.vt_group);
-    for (int vt = vt0; vt < vt1; ++vt) {
-        const int kl = vt * V + TV * lane;
-        const T *__restrict__ fl = dc.f_cur + kl;
-
-        T u[3][TV];
-        auto load_u = [&](int k, auto &uu) {
-            constexpr int N = sizeof(uu[0]) / sizeof(T);
-            ldv<T, N>(dc.u[0] + k, uu[0]);
-            ldv<T, N>(dc.u[1] + k, uu[1]);
-            if (D == 3) ldv<T, N>(dc.u[2] + k, uu[2]);
-            else
+    // patches fastest: the CTAs in flight cover neighbouring patches of one
+    // tile, so that the rows of f and of the flux buffer they share stay in L2
+    const int tile = bx / dc.n_patches, p = bx - tile * dc.n_patches;
+    const int kc = tile * V + TV * lane, k = chunk * dc.chunk + kc;   // in the chunk, of all
+    if (kc >= dc.chunk || k >= dc.nvp) return;                        // the last tile may be short
+    const int cb = p * dc.P, ce = min(dc.C, cb + dc.P);
+    const T *__restrict__ fl = dc.f_cur + k;
+    P u[NP][D];
 #pragma unroll
-                for (int j = 0; j < N; ++j) uu[2][j] = T(0);
-        };
-
-        // ---- phase A: slopes (micro reconstruction of the velocity loop, Algorithm 1)
-        if constexpr (TVA == TV) {
-            load_u(kl, u);
-            for (int s = warp; s < nslope; s += nwarps) {
-                const int c = s < npc ? cb + s : dc.ring_cells[rb + s - npc];
-                T g[NC][D][TV], fi[NC][TV];
-                cell_slope_tv<T, D, NC, TV>(dc, fl, c, u, g, fi);
+    for (int d = 0; d < D; ++d) {
+        P t[NP];
+        ldp<T, TV>(dc.u[d] + k, t);
 #pragma unroll
-                for (int m = 0; m < NC; ++m)
+        for (int i = 0; i < NP; ++i) u[i][d] = t[i];
+    }
+    const T dt = dc.dtT, hdt2 = T(0.5) * dc.dtT * dc.dtT;
+    for (int c = cb + warp; c < ce; c += nwarps) {
+        int e0 = c * NF, ne = NF;
+        if (NF == 0) entry_range(dc, c, e0, ne);
+        P fi[NC][NP], g[NC][NP][D], ug[NC][NP];
+        cell_slope<T, D, NC, TV, NF>(dc, fl, c, e0, ne, u, fi, g, ug);
+        auto face = [&](const int e) {
+            const int4 gi = __ldg(dc.gi + e);
+            const int type = gi.z & 255;
+            if (type == FT_NONE) return;
+            T rsv[4], nv[4];
+            load_rec<4>(dc.gf + (size_t)e * E::LEN + (E::RS / 4) * 4, rsv);
+            load_rec<4>(dc.gf + (size_t)e * E::LEN + E::N, nv);
+            const T *r = rsv + E::RS % 4;
+            P un[NP];
 #pragma unroll
-                    for (int d = 0; d < D; ++d) stv<T, TV>(sl + ((s * NC + m) * D + d) * V, g[m][d]);
-            }
-        } else {
-            // each half-warp takes a slope cell, TVA velocities per lane: the
-            // face entries are read once for twice the velocities
-            const int hl = lane & 15;
-            const int klA = vt * V + TVA * hl;
-            T ua[3][TVA];
-            load_u(klA, ua);
-            const T *__restrict__ fla = dc.f_cur + klA;
-            T *const sla = sg + gather_acc_values<T>(dc.P) + TVA * hl;
-            for (int s = 2 * warp + (lane >> 4); s < nslope; s += 2 * nwarps) {
-                const int c = s < npc ? cb + s : dc.ring_cells[rb + s - npc];
-                T g[NC][D][TVA], fi[NC][TVA];
-                cell_slope_tv<T, D, NC, TVA>(dc, fla, c, ua, g, fi);
+            for (int i = 0; i < NP; ++i) un[i] = pnormal<T, D, P>(u[i], nv, dc.one);
+            // the velocities this cell evaluates: those that leave it (u.n = 0,
+            // no flux, falls to the neighbour); all of a boundary face
+            const bool own = (gi.z >> 8) != 0;
+            unsigned on = 0;
 #pragma unroll
-                for (int m = 0; m < NC; ++m)
+            for (int j = 0; j < TV; ++j) on |= (gt0(pel<W>(un, j)) == own ? 1u : 0u) << j;
+            P F[NC][NP];
+            // value of the cell at the face centre
+            auto at_face = [&](int m, int i) {
+                P s = fi[m][i];
 #pragma unroll
-                    for (int d = 0; d < D; ++d) stv<T, TVA>(sla + ((s * NC + m) * D + d) * V, g[m][d]);
-            }
-            load_u(kl, u);
-        }
-        __syncthreads();
-
-        // ---- phase B: fluxes, stage 1, moments (velocity loop and wall flux, Algorithm 1)
-        const T dt = dc.dtT;
-        const T hdt2 = T(0.5) * dc.dtT * dc.dtT;
-        for (int s = warp; s < npc; s += nwarps) {
-            const int c = cb + s;
-            T fs[NC][TV], gs[NC][D][TV], R[NC][TV];
-#pragma unroll
-            for (int m = 0; m < NC; ++m) {
-                ldv<T, TV>(fl + (size_t)c * rs + (size_t)m * nvp, fs[m]);
-#pragma unroll
-                for (int d = 0; d < D; ++d) ldv_s<T, TV>(sl + ((s * NC + m) * D + d) * V, gs[m][d]);
-#pragma unroll
-                for (int j = 0; j < TV; ++j) R[m][j] = 0;
-            }
-            const int e0 = __ldg(dc.cf_ptr + c), e1 = __ldg(dc.cf_ptr + c + 1);
-#pragma unroll 4
-            for (int e = e0; e < e1; ++e) {
-                const int4 gi = __ldg(dc.gi + e);
-                T ge[E::LEN];
-                if constexpr (E::SKIP1 > E::SKIP0) {
-                    load_rec<E::SKIP0>(dc.gf + (size_t)e * E::LEN, *reinterpret_cast<T (*)[E::SKIP0]>(ge));
-                    load_rec<E::LEN - E::SKIP1>(dc.gf + (size_t)e * E::LEN + E::SKIP1,
-                                                *reinterpret_cast<T (*)[E::LEN - E::SKIP1]>(ge + E::SKIP1));
-                } else {
-                    load_rec<E::LEN>(dc.gf + (size_t)e * E::LEN, ge);
-                }
-                const T cs = ge[E::CS];
-                T un[TV];
+                for (int d = 0; d < D; ++d) s = pfma(g[m][i][d], pbc<P>(r[d]), s);
+                return s;
+            };
+            if (type == FT_WALL) {
+                T wr[GREC];
+                load_rec<GREC>(dc.wrec + (size_t)gi.w * GREC, wr);
 #pragma unroll
                 for (int j = 0; j < TV; ++j) {
-                    const T uj[3] = {u[0][j], u[1][j], u[2][j]};
-                    un[j] = normal_velocity<T, D>(uj, ge + E::N);
-                }
-                if (gi.z == FT_WALL) {
-                    T wr[GREC];
-                    load_rec<GREC>(dc.wrec + (size_t)gi.x * GREC, wr);
+                    const int i = j / W;
+                    T uj[3] = {T(0), T(0), T(0)};
 #pragma unroll
-                    for (int j = 0; j < TV; ++j) {
-                        const T uj[3] = {u[0][j], u[1][j], u[2][j]};
-                        T F[NC];
-                        if (un[j] > T(0)) {
-#pragma unroll
-                            for (int m = 0; m < NC; ++m) {
-                                T fin = fs[m][j], ug = 0;
-#pragma unroll
-                                for (int d = 0; d < D; ++d) {
-                                    fin += gs[m][d][j] * ge[E::RS + d];
-                                    ug += uj[d] * gs[m][d][j];
-                                }
-                                F[m] = un[j] * (dt * fin - hdt2 * ug);
-                            }
-                        } else {
-                            const T H = maxwell_h<T, D>(wr, uj);
-                            F[0] = un[j] * dt * H;
-                            if (NC == 2) F[NC - 1] = un[j] * dt * wr[GR_NB] * H;
-                        }
-#pragma unroll
-                        for (int m = 0; m < NC; ++m) R[m][j] += cs * F[m];
-                    }
-                    continue;
-                }
-                T fr[XREC];
-                load_rec<XREC>(dc.xrec + (size_t)gi.y * XREC, fr);
-                if (gi.z == FT_FARFIELD) {
-                    T gr[GREC];
-                    load_rec<GREC>(dc.grec + (size_t)gi.x * GREC, gr);
-#pragma unroll
-                    for (int j = 0; j < TV; ++j) {
-                        const T uj[3] = {u[0][j], u[1][j], u[2][j]};
-                        T fup[NC], ugf[NC], F[NC];
-                        if (un[j] > T(0)) {
-#pragma unroll
-                            for (int m = 0; m < NC; ++m) {
-                                T v = fs[m][j], ug = 0;
-#pragma unroll
-                                for (int d = 0; d < D; ++d) {
-                                    v += gs[m][d][j] * ge[E::RS + d];
-                                    ug += uj[d] * gs[m][d][j];
-                                }
-                                fup[m] = v;
-                                ugf[m] = ug;
-                            }
-                        } else {
-                            const T H = maxwell_h<T, D>(gr, uj);
-                            fup[0] = H;
-                            if (NC == 2) fup[NC - 1] = gr[GR_NB] * H;
-#pragma unroll
-                            for (int m = 0; m < NC; ++m) ugf[m] = 0;
-                        }
-                        interface_flux<T, D, NC>(fr, uj, un[j], fup, ugf, F);
-#pragma unroll
-                        for (int m = 0; m < NC; ++m) R[m][j] += cs * F[m];
-                    }
-                    continue;
-                }
-                // interior or periodic: the neighbour's f and slopes
-                T fo[NC][TV], go[NC][D][TV];
-                const T *so = sl + (size_t)gi.w * NC * D * V;
-#pragma unroll
-                for (int m = 0; m < NC; ++m) {
-                    ldv<T, TV>(fl + (size_t)gi.x * rs + (size_t)m * nvp, fo[m]);
-#pragma unroll
-                    for (int d = 0; d < D; ++d) ldv_s<T, TV>(so + (m * D + d) * V, go[m][d]);
-                }
-#pragma unroll
-                for (int j = 0; j < TV; ++j) {
-                    const T uj[3] = {u[0][j], u[1][j], u[2][j]};
-                    const bool self = un[j] > T(0);
-                    T fup[NC], ugf[NC], F[NC];
+                    for (int d = 0; d < D; ++d) uj[d] = pel<W>(&u[i][d], j % W);
+                    const T H = maxwell_h<T, D>(wr, uj), unj = pel<W>(un, j);
 #pragma unroll
                     for (int m = 0; m < NC; ++m) {
-                        T v = self ? fs[m][j] : fo[m][j], ug = 0;
-#pragma unroll
-                        for (int d = 0; d < D; ++d) {
-                            const T gd = self ? gs[m][d][j] : go[m][d][j];
-                            v += gd * (self ? ge[E::RS + d] : ge[E::RO + d]);
-                            ug += uj[d] * gd;
-                        }
-                        fup[m] = v;
-                        ugf[m] = ug;
-                    }
-                    interface_flux<T, D, NC>(fr, uj, un[j], fup, ugf, F);
-#pragma unroll
-                    for (int m = 0; m < NC; ++m) R[m][j] += cs * F[m];
-                }
-            }
-            // stage 1 and the moments of R
-            T cr[CREC];
-            load_rec<CREC>(dc.crec + (size_t)c * CREC, cr);
-            const T cc = cr[CR_C];
-            T wk[TV];
-            ldv<T, TV>(dc.w + kl, wk);
-            // moments sum_k w psi_k R_k of this tile: FP64 sums in the FP64 form;
-            // in the FP32 form each term is an FP32 product, and the sums over the
-            // lane's velocities and across the warp are double-float (error-free
-            // additions), widened to FP64 for the W update
-            constexpr int NR = M <= 4 ? 4 : 8;
-            T mh[NR], ml[NR];
-#pragma unroll
-            for (int i = 0; i < NR; ++i) mh[i] = ml[i] = T(0);
-            T out[NC][TV];
-#pragma unroll
-            for (int j = 0; j < TV; ++j) {
-                const T uj[3] = {u[0][j], u[1][j], u[2][j]};
-                T fp[NC];
-                shakhov_fplus<T, D, NC>(cr, uj, fp);
-#pragma unroll
-                for (int m = 0; m < NC; ++m) out[m][j] = fs[m][j] + R[m][j] + cc * (fp[m] - fs[m][j]);
-                T u2 = 0;
-#pragma unroll
-                for (int d = 0; d < D; ++d) u2 += uj[d] * uj[d];
-                const T wr0 = wk[j] * R[0][j];
-                T x[M];
-                x[0] = wr0;
-#pragma unroll
-                for (int d = 0; d < D; ++d) x[1 + d] = uj[d] * wr0;
-                x[D + 1] = T(0.5) * (u2 * wr0 + (NC == 2 ? wk[j] * R[NC - 1][j] : T(0)));
-#pragma unroll
-                for (int i = 0; i < M; ++i) {
-                    if constexpr (std::is_same<T, float>::value) {
-                        if (j == 0) mh[i] = x[i];
-                        else ff_add(mh[i], ml[i], x[i], 0.f);
-                    } else {
-                        mh[i] += x[i];
+                        P s = at_face(m, i);
+                        const T out = dt * pel<W>(&s, j % W) - hdt2 * pel<W>(ug[m], j);
+                        pel<W>(F[m], j) = (on >> j & 1) ? unj * out : (m == 0 ? unj * dt : unj * dt * wr[GR_NB]) * H;
                     }
                 }
-            }
-#pragma unroll
-            for (int m = 0; m < NC; ++m) stv<T, TV>(dc.f_nxt + kl + (size_t)c * rs + (size_t)m * nvp, out[m]);
-            const int vi = lane >> (NR == 4 ? 3 : 2);
-            const bool holder = (lane & (NR == 4 ? 7 : 3)) == 0 && vi < M;
-            if constexpr (std::is_same<T, float>::value) {
-                float oh, ol;
-                warp_transpose_sum_ff2<NR>(mh, ml, oh, ol);
-                if (holder) ff_add(sacc[s * 16 + vi], sacc[s * 16 + 8 + vi], oh, ol);
+                on = (1u << TV) - 1;
             } else {
-                const T sm = warp_transpose_sum<T, NR>(mh);
-                if (holder) sacc[s * 16 + vi] += sm;
+                T x[X::LEN];
+                load_rec<X::LEN>(dc.xrec + (size_t)gi.y * X::LEN, x);
+                P fup[NC][NP], ugf[NC][NP];
+#pragma unroll
+                for (int m = 0; m < NC; ++m)
+#pragma unroll
+                    for (int i = 0; i < NP; ++i) {
+                        fup[m][i] = at_face(m, i);
+                        ugf[m][i] = ug[m][i];
+                    }
+                if (type == FT_FARFIELD) {                 // the ghost's Maxwellian comes in
+                    T gr[GREC];
+                    load_rec<GREC>(dc.grec + (size_t)gi.w * GREC, gr);
+#pragma unroll
+                    for (int j = 0; j < TV; ++j) {
+                        if (on >> j & 1) continue;
+                        T uj[3] = {T(0), T(0), T(0)};
+#pragma unroll
+                        for (int d = 0; d < D; ++d) uj[d] = pel<W>(&u[j / W][d], j % W);
+                        const T H = maxwell_h<T, D>(gr, uj);
+#pragma unroll
+                        for (int m = 0; m < NC; ++m) {
+                            pel<W>(fup[m], j) = m == 0 ? H : gr[GR_NB] * H;
+                            pel<W>(ugf[m], j) = T(0);
+                        }
+                    }
+                    on = (1u << TV) - 1;
+                }
+                const P q1 = pbc<P>(x[X::Q1]), q2 = pbc<P>(x[X::Q2]);
+#pragma unroll
+                for (int i = 0; i < NP; ++i) {
+                    P cv[D], c2, h;
+#pragma unroll
+                    for (int d = 0; d < D; ++d) {
+                        cv[d] = padd(u[i][d], pbc<P>(x[X::U + d]));
+                        c2 = d == 0 ? pmul(cv[0], cv[0]) : pfma(cv[d], cv[d], c2);
+                    }
+#pragma unroll
+                    for (int w = 0; w < W; ++w) pel<W>(&h, w) = gauss_ex(x[X::EX], pel<W>(&c2, w));
+                    h = pmul(h, pbc<P>(x[X::PREF]));
+#pragma unroll
+                    for (int m = 0; m < NC; ++m) {
+                        const P eq = poly_eval<T, D, P>(x + X::POLY + m * Poly<D>::N, cv, c2);
+                        F[m][i] = pmul(un[i], pfma(h, eq, pfma(q1, fup[m][i], pmul(q2, ugf[m][i]))));
+                    }
+                }
+            }
+            T *Fr = dc.flux + (size_t)gi.y * NC * dc.chunk + kc;
+            if (on == (1u << TV) - 1) {
+#pragma unroll
+                for (int m = 0; m < NC; ++m) {
+                    T v[TV];
+#pragma unroll
+                    for (int j = 0; j < TV; ++j) v[j] = pel<W>(F[m], j);
+                    stv<T, TV>(Fr + (size_t)m * dc.chunk, v);
+                }
+            } else if (on) {
+#pragma unroll
+                for (int m = 0; m < NC; ++m)
+#pragma unroll
+                    for (int j = 0; j < TV; ++j)
+                        if (on >> j & 1) Fr[(size_t)m * dc.chunk + j] = pel<W>(F[m], j);
+            }
+        };
+        if constexpr (NF > 0) {
+#pragma unroll
+            for (int e = 0; e < NF; ++e) face(e0 + e);
+        } else {
+            for (int e = 0; e < ne; ++e) face(e0 + e);
+        }
+    }
+}
+
+// 512-thread CTAs are held to 64 registers so that two fit an SM; 256-thread
+// CTAs take what ptxas chooses (118 registers for tetrahedra at TV = 4, two CTAs
+// per SM): held to 80 registers, three CTAs spill and measure 8.00 against
+// 8.30 ms on the 107k-cell tetrahedral mesh but 9.02 against 8.77 ms on 24k
+// cells x 28^3 and 1.81 against 1.74 ms on the 30k-cell triangulation.
+template <typename T, int D, int NC, int TV, int NF, int NTH>
+__global__ void __launch_bounds__(NTH, NTH >= 512 ? 2 : 0) k_flux(DevCase<T> dc, int chunk)
+{
+    flux_body<T, D, NC, TV, NF>(dc, blockIdx.x, chunk);
+}
+
+template <typename T, int D, int NC, int TV, int NF, int NTH>
+__global__ void __launch_bounds__(NTH, NTH >= 512 ? 2 : 0)
+    k_flux_batch(const DevCase<T> *__restrict__ cases, const int *__restrict__ off, int n, int chunk)
+{
+    int bx;
+    const DevCase<T> &dc = batch_case(cases, off, n, bx);
+    flux_body<T, D, NC, TV, NF>(dc, bx, chunk);
+}
+
+// Moment sums of stage 1: a lane adds its terms two velocities at a time into
+// double-float pairs in the FP32 form (TwoSum, the errors summed in the low
+// part), plainly in the FP64 form.
+template <typename P> struct MomentSum;
+template <> struct MomentSum<double> {
+    double s;
+    __device__ __forceinline__ void zero() { s = 0.0; }
+    __device__ __forceinline__ void add(double x, double) { s = __dadd_rn(s, x); }
+};
+template <> struct MomentSum<float2> {
+    float2 h, l;
+    __device__ __forceinline__ void zero() { h = l = make_float2(0.f, 0.f); }
+    // every addition rounds by itself (see psum)
+    __device__ __forceinline__ void add(float2 x, float one)
+    {
+        const float2 m1 = make_float2(-one, -one);
+        const float2 s = psum(x, h, one), v = pfma(h, m1, s);     // s - h
+        l = padd(l, padd(pfma(pfma(v, m1, s), m1, h), pfma(v, m1, x)));   // (h - (s - v)) + (x - v)
+        h = s;
+    }
+};
+
+// One warp per cell and group of gvel velocities of the chunk, four consecutive
+// velocities per lane.  Bound: the latency of its row loads (nf rows of the flux
+// buffer and f, which is written in place); the reduction at a group's end costs
+// as much as 250 velocities (see set_chunks in ugks_host.cu).
+template <typename T, int D, int NC, int NF>
+__device__ __forceinline__ void stage1_body(const DevCase<T> &dc, const int bx, const int chunk)
+{
+    using E = GEnt<D>;
+    using K = Pk<T, 4>;
+    using P = typename K::P;
+    constexpr int M = D + 2, W = K::W, NP = K::NP;
+    const int lane = threadIdx.x & 31;
+    const int ncb = (dc.C + 7) >> 3, grp = bx / ncb;
+    const int c = (bx - grp * ncb) * 8 + (threadIdx.x >> 5);
+    if (c >= dc.C) return;
+    const int kb = chunk * dc.chunk, kg = grp * dc.gvel;              // chunk start; group start in the chunk
+    const int kn = min(min(dc.chunk, dc.nvp - kb), kg + dc.gvel);     // end in the chunk
+    if (kg >= kn) return;                                              // the last chunk may be short
+    int e0 = c * NF, ne = NF;
+    if (NF == 0) entry_range(dc, c, e0, ne);
+    T cs[NF > 0 ? NF : 1];
+    const T *Fr[NF > 0 ? NF : 1];
+    if constexpr (NF > 0) {
+        // a padding entry reads the first face's row with coefficient 0
+        const int f0 = __ldg(dc.gi + e0).y;
+#pragma unroll
+        for (int e = 0; e < NF; ++e) {
+            const int4 gi = __ldg(dc.gi + e0 + e);
+            cs[e] = __ldg(dc.gf + (size_t)(e0 + e) * E::LEN + E::CS);
+            Fr[e] = dc.flux + (size_t)(gi.z == FT_NONE ? f0 : gi.y) * NC * dc.chunk;
+        }
+    }
+    T cr[CREC];
+    load_rec<CREC>(dc.crec + (size_t)c * CREC, cr);
+    const P ccol = pbc<P>(cr[CR_C]), kl2 = pbc<P>(T(2) * cr[CR_LAM]);
+    MomentSum<P> acc[M];
+#pragma unroll
+    for (int i = 0; i < M; ++i) acc[i].zero();
+    T *frow = dc.f_cur + (size_t)c * NC * dc.nvp + kb;
+    for (int kc = kg + 4 * lane; kc < kn; kc += 128) {
+        P fs[NC][NP], R[NC][NP];
+#pragma unroll
+        for (int m = 0; m < NC; ++m) {
+            using V4 = typename VecOf<T, vec_chunk<T, 4>()>::type;
+            constexpr int CH = vec_chunk<T, 4>();
+#pragma unroll
+            for (int q = 0; q < 4 / CH; ++q) {                        // f is written below: ordinary loads
+                const V4 v = reinterpret_cast<const V4 *>(frow + (size_t)m * dc.nvp + kc)[q];
+                const T *ev = reinterpret_cast<const T *>(&v);
+#pragma unroll
+                for (int j = 0; j < CH; ++j) pel<W>(fs[m], q * CH + j) = ev[j];
+            }
+#pragma unroll
+            for (int i = 0; i < NP; ++i) R[m][i] = pbc<P>(T(0));
+        }
+        if constexpr (NF > 0) {
+            P Fv[NF][NC][NP];
+#pragma unroll
+            for (int e = 0; e < NF; ++e)
+#pragma unroll
+                for (int m = 0; m < NC; ++m) ldp<T, 4>(Fr[e] + (size_t)m * dc.chunk + kc, Fv[e][m]);
+#pragma unroll
+            for (int e = 0; e < NF; ++e)
+#pragma unroll
+                for (int m = 0; m < NC; ++m)
+#pragma unroll
+                    for (int i = 0; i < NP; ++i) R[m][i] = pfma(pbc<P>(cs[e]), Fv[e][m][i], R[m][i]);
+        } else {
+            for (int e = 0; e < ne; ++e) {
+                const int4 gi = __ldg(dc.gi + e0 + e);
+                const P ce = pbc<P>(__ldg(dc.gf + (size_t)(e0 + e) * E::LEN + E::CS));
+#pragma unroll
+                for (int m = 0; m < NC; ++m) {
+                    P Fv[NP];
+                    ldp<T, 4>(dc.flux + ((size_t)gi.y * NC + m) * dc.chunk + kc, Fv);
+#pragma unroll
+                    for (int i = 0; i < NP; ++i) R[m][i] = pfma(ce, Fv[i], R[m][i]);
+                }
             }
         }
-        __syncthreads();                        // the next tile's slopes overwrite the buffer
-    }
-    // the moments of the group, once per (cell, group), by the warp that owns the cell
-    for (int s = warp; s < npc; s += nwarps) {
-        const int vi = lane >> (M <= 4 ? 3 : 2);
-        if ((lane & (M <= 4 ? 7 : 3)) == 0 && vi < M) {
-            double v = (double)sacc[s * 16 + vi];
-            if constexpr (std::is_same<T, float>::value) v += (double)sacc[s * 16 + 8 + vi];
-            dc.dW_part[((size_t)(cb + s) * dc.n_groups + grp) * M + vi] = v;
+        P u[D][NP], wk[NP];
+#pragma unroll
+        for (int d = 0; d < D; ++d) ldp<T, 4>(dc.u[d] + kb + kc, u[d]);
+        ldp<T, 4>(dc.w + kb + kc, wk);
+#pragma unroll
+        for (int i = 0; i < NP; ++i) {
+            // f+ of the cell (shakhov_fplus), stage 1
+            P cv[D], c2, kqc, u2, h;
+#pragma unroll
+            for (int d = 0; d < D; ++d) {
+                cv[d] = padd(u[d][i], pbc<P>(-cr[CR_U + d]));
+                c2 = d == 0 ? pmul(cv[0], cv[0]) : pfma(cv[d], cv[d], c2);
+                kqc = d == 0 ? pmul(cv[0], pbc<P>(cr[CR_KQ])) : pfma(cv[d], pbc<P>(cr[CR_KQ + d]), kqc);
+                u2 = d == 0 ? pmul(u[0][i], u[0][i]) : pfma(u[d][i], u[d][i], u2);
+            }
+#pragma unroll
+            for (int w = 0; w < W; ++w)
+                pel<W>(&h, w) = cr[CR_PREF] * gauss<T>(cr[CR_LAM], cr[CR_NL2], pel<W>(&c2, w));
+#pragma unroll
+            for (int m = 0; m < NC; ++m) {
+                const P X = pfma(kqc, pfma(kl2, c2, pbc<P>(T(m == 0 ? -(D + 2) : -D))), pbc<P>(T(1)));
+                const P df = pfma(m == 0 ? h : pmul(h, pbc<P>(cr[CR_NB])), X, pmul(fs[m][i], pbc<P>(T(-1))));
+                fs[m][i] = pfma(ccol, df, padd(fs[m][i], R[m][i]));
+            }
+            const P wr = pmul(wk[i], R[0][i]);
+            acc[0].add(wr, dc.one);
+#pragma unroll
+            for (int d = 0; d < D; ++d) acc[1 + d].add(pmul(u[d][i], wr), dc.one);
+            const P en = NC == 2 ? pfma(u2, wr, pmul(wk[i], R[NC - 1][i])) : pmul(u2, wr);
+            acc[D + 1].add(pmul(pbc<P>(T(0.5)), en), dc.one);
+        }
+#pragma unroll
+        for (int m = 0; m < NC; ++m) {
+            T v[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) v[j] = pel<W>(fs[m], j);
+            stv<T, 4>(frow + (size_t)m * dc.nvp + kc, v);
         }
     }
-}
-
-// NTH threads per CTA; 512-thread CTAs are held to 64 registers so that two
-// fit an SM (32 resident warps, against 24 for 256-thread CTAs at 80).  A
-// minimum of 0 blocks leaves 256-thread CTAs to ptxas's own register choice:
-// an explicit 1 lets it take 113 registers in the 2D FP32 kernel, which
-// drops the SM to two CTAs and costs about 20 %.
-template <typename T, int D, int NC, int TV, int NTH>
-__global__ void __launch_bounds__(NTH, NTH >= 512 ? 2 : 0) k_gather(DevCase<T> dc)
-{
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    // One-dimensional grid of n_patches x n_groups blocks, patches fastest:
-    // the CTAs in flight cover neighbouring patches in the same tile group,
-    // so the rows of f they share (ring cells) are read from L2.
-    const int grp = blockIdx.x / dc.n_patches;
-    gather_item<T, D, NC, TV>(dc, blockIdx.x - grp * dc.n_patches, grp, reinterpret_cast<T *>(smem_raw));
-}
-
-// Persistent gather over many cases: a fixed grid of CTAs walks a work list of
-// (case, patch, tile group) items; each item is exactly the CTA of k_gather
-// for that case, so every case gets bit-identical results alone or batched.
-template <typename T, int D, int NC, int TV, int NTH>
-__global__ void __launch_bounds__(NTH, NTH >= 512 ? 2 : 0) k_gather_batch(const DevCase<T> *__restrict__ cases,
-                                                                          const int4 *__restrict__ work, int nwork)
-{
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    for (int w = blockIdx.x; w < nwork; w += gridDim.x) {
-        const int4 it = work[w];
-        gather_item<T, D, NC, TV>(cases[it.x], it.y, it.z, reinterpret_cast<T *>(smem_raw));
-        __syncthreads();
+    // across the warp
+    constexpr int NR = M <= 4 ? 4 : 8;
+    const int vi = lane >> (NR == 4 ? 3 : 2);
+    double sum;
+    if constexpr (std::is_same<T, float>::value) {
+        float mh[NR], ml[NR], oh, ol;
+#pragma unroll
+        for (int i = 0; i < NR; ++i) {
+            mh[i] = ml[i] = 0.f;
+            if (i < M) {
+                mh[i] = acc[i].h.x;
+                ml[i] = acc[i].l.x;
+                ff_add(mh[i], ml[i], acc[i].h.y, acc[i].l.y);
+            }
+        }
+        warp_transpose_sum_ff2<NR>(mh, ml, oh, ol);
+        sum = (double)oh + (double)ol;
+    } else {
+        T v[NR];
+#pragma unroll
+        for (int i = 0; i < NR; ++i) v[i] = i < M ? acc[i].s : T(0);
+        sum = warp_transpose_sum<T, NR>(v);
     }
+    if ((lane & (NR == 4 ? 7 : 3)) == 0 && vi < M)
+        dc.dW_part[((size_t)c * dc.n_groups + (kb + kg) / dc.gvel) * M + vi] = sum;
+}
+
+template <typename T, int D, int NC, int NF>
+__global__ void __launch_bounds__(256) k_stage1(DevCase<T> dc, int chunk)
+{
+    stage1_body<T, D, NC, NF>(dc, blockIdx.x, chunk);
+}
+
+template <typename T, int D, int NC, int NF>
+__global__ void __launch_bounds__(256) k_stage1_batch(const DevCase<T> *__restrict__ cases,
+                                                      const int *__restrict__ off, int n, int chunk)
+{
+    int bx;
+    const DevCase<T> &dc = batch_case(cases, off, n, bx);
+    stage1_body<T, D, NC, NF>(dc, bx, chunk);
 }
 
 // ------------------------------------------------------------ W update
@@ -1861,7 +1927,7 @@ __device__ __forceinline__ void collide_body(const DevCase<T> &dc, const int bx)
     int nblk = 0;
     // the f~ vectors of the next iteration are loaded before this one's
     // arithmetic, so that a warp keeps a load in flight while it computes
-    const T *frow = dc.f_nxt + (size_t)c * rs;
+    T *frow = dc.f_cur + (size_t)c * rs;
     V4 nxt[NC];
     if (4 * lane < dc.nvp)
 #pragma unroll
@@ -1919,7 +1985,7 @@ __device__ __forceinline__ void collide_body(const DevCase<T> &dc, const int bx)
                 v.y = fn[m][1];
                 v.z = fn[m][2];
                 v.w = fn[m][3];
-                *reinterpret_cast<V4 *>(dc.f_cur + (size_t)c * rs + (size_t)m * dc.nvp + k0) = v;
+                *reinterpret_cast<V4 *>(frow + (size_t)m * dc.nvp + k0) = v;
             }
         }
         if constexpr (F32) {
@@ -2097,35 +2163,101 @@ __global__ void k_halo_unpack(DevCase<T> dc, const int *cells, int n, size_t row
 // ------------------------------------------------------------ launchers
 static inline int cdiv(long long a, int b) { return (int)((a + b - 1) / b); }
 
-template <typename T, int D, int NC, int TV, int NTH>
-static cudaError_t gather_launch(const DevCase<T> &dc, size_t smem, cudaStream_t st)
+// The two kernels of a chunk, for one case (cases == nullptr) or for those of a
+// batch (block offsets off[0..n]).  All cases of a launch share the tiling's
+// velocities per lane tv and threads nth, and the entry count nf.
+template <typename T, int D, int NC, int TV, int NF, int NTH>
+static cudaError_t flux_launch(int blocks, int chunk, cudaStream_t st, const DevCase<T> *dc, const DevCase<T> *cases,
+                               const int *off, int n)
 {
-    auto kern = k_gather<T, D, NC, TV, NTH>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    const int grid = dc.n_patches * dc.n_groups;
-    kern<<<grid, NTH, smem, st>>>(dc);
+    if (cases) k_flux_batch<T, D, NC, TV, NF, NTH><<<blocks, NTH, 0, st>>>(cases, off, n, chunk);
+    else k_flux<T, D, NC, TV, NF, NTH><<<blocks, NTH, 0, st>>>(*dc, chunk);
     return cudaGetLastError();
 }
 
-// the gather kernel of a case: velocities per lane TV = vtile / 32 and
-// threads per CTA (256, or 512 for FP32 at TV <= 2)
-template <typename T, int D, int NC>
-static cudaError_t gather_dispatch(const DevCase<T> &dc, size_t smem, cudaStream_t st)
+template <typename T, int D, int NC, int NF>
+static cudaError_t flux_tiled(int tv, int nth, int blocks, int chunk, cudaStream_t st, const DevCase<T> *dc,
+                              const DevCase<T> *cases, const int *off, int n)
 {
-    const int tv = dc.vtile / 32;
-    if (dc.nth == 512) {
+    if (nth == 512) {
         if constexpr (std::is_same<T, float>::value) {
-            if (tv == 1) return gather_launch<T, D, NC, 1, 512>(dc, smem, st);
-            if (tv == 2) return gather_launch<T, D, NC, 2, 512>(dc, smem, st);
+            if (tv == 1) return flux_launch<T, D, NC, 1, NF, 512>(blocks, chunk, st, dc, cases, off, n);
+            if (tv == 2) return flux_launch<T, D, NC, 2, NF, 512>(blocks, chunk, st, dc, cases, off, n);
         }
         return cudaErrorInvalidValue;
     }
-    if (dc.nth != 256) return cudaErrorInvalidValue;
-    if (tv == 1) return gather_launch<T, D, NC, 1, 256>(dc, smem, st);
-    if (tv == 2) return gather_launch<T, D, NC, 2, 256>(dc, smem, st);
-    if (tv == 4) return gather_launch<T, D, NC, 4, 256>(dc, smem, st);
+    if (tv == 1) return flux_launch<T, D, NC, 1, NF, 256>(blocks, chunk, st, dc, cases, off, n);
+    if (tv == 2) return flux_launch<T, D, NC, 2, NF, 256>(blocks, chunk, st, dc, cases, off, n);
+    if (tv == 4) return flux_launch<T, D, NC, 4, NF, 256>(blocks, chunk, st, dc, cases, off, n);
     return cudaErrorInvalidValue;
+}
+
+// entry counts with kernels of their own: triangles, quadrilaterals and
+// tetrahedra, hexahedra; a mesh with another largest count takes the next one
+// above, one beyond MAX_NF the kernels that loop over the cells' own counts
+template <typename T>
+cudaError_t launch_flux(int D, int nf, int vtile, int nth, int blocks, int chunk, cudaStream_t st,
+                        const DevCase<T> *dc, const DevCase<T> *cases, const int *off, int n)
+{
+    const int tv = vtile / 32;
+    if (blocks <= 0) return cudaSuccess;
+    if (D == 2) {
+        if (nf == 3) return flux_tiled<T, 2, 2, 3>(tv, nth, blocks, chunk, st, dc, cases, off, n);
+        if (nf == 4) return flux_tiled<T, 2, 2, 4>(tv, nth, blocks, chunk, st, dc, cases, off, n);
+        return flux_tiled<T, 2, 2, 0>(tv, nth, blocks, chunk, st, dc, cases, off, n);
+    }
+    if (nf == 4) return flux_tiled<T, 3, 1, 4>(tv, nth, blocks, chunk, st, dc, cases, off, n);
+    if (nf == 6) return flux_tiled<T, 3, 1, 6>(tv, nth, blocks, chunk, st, dc, cases, off, n);
+    return flux_tiled<T, 3, 1, 0>(tv, nth, blocks, chunk, st, dc, cases, off, n);
+}
+
+template <typename T, int D, int NC, int NF>
+static cudaError_t stage1_launch(int blocks, int chunk, cudaStream_t st, const DevCase<T> *dc, const DevCase<T> *cases,
+                                 const int *off, int n)
+{
+    if (cases) k_stage1_batch<T, D, NC, NF><<<blocks, 256, 0, st>>>(cases, off, n, chunk);
+    else k_stage1<T, D, NC, NF><<<blocks, 256, 0, st>>>(*dc, chunk);
+    return cudaGetLastError();
+}
+
+template <typename T>
+cudaError_t launch_stage1(int D, int nf, int blocks, int chunk, cudaStream_t st, const DevCase<T> *dc,
+                          const DevCase<T> *cases, const int *off, int n)
+{
+    if (blocks <= 0) return cudaSuccess;
+    if (D == 2) {
+        if (nf == 3) return stage1_launch<T, 2, 2, 3>(blocks, chunk, st, dc, cases, off, n);
+        if (nf == 4) return stage1_launch<T, 2, 2, 4>(blocks, chunk, st, dc, cases, off, n);
+        return stage1_launch<T, 2, 2, 0>(blocks, chunk, st, dc, cases, off, n);
+    }
+    if (nf == 4) return stage1_launch<T, 3, 1, 4>(blocks, chunk, st, dc, cases, off, n);
+    if (nf == 6) return stage1_launch<T, 3, 1, 6>(blocks, chunk, st, dc, cases, off, n);
+    return stage1_launch<T, 3, 1, 0>(blocks, chunk, st, dc, cases, off, n);
+}
+
+template <typename T> int flux_blocks(const DevCase<T> &dc, int chunk)
+{
+    const int left = dc.nvp - chunk * dc.chunk;
+    return left > 0 ? dc.n_patches * cdiv(std::min(left, dc.chunk), dc.vtile) : 0;
+}
+
+template <typename T> int stage1_blocks(const DevCase<T> &dc, int chunk)
+{
+    const int left = dc.nvp - chunk * dc.chunk;
+    return left > 0 ? cdiv(dc.C, 8) * cdiv(std::min(left, dc.chunk), dc.gvel) : 0;
+}
+
+// the flux and stage-1 passes of one case over its chunks
+template <typename T>
+cudaError_t launch_gather(const DevCase<T> &dc, cudaStream_t st)
+{
+    for (int r = 0; r < dc.n_chunks; ++r) {
+        cudaError_t e = launch_flux<T>(dc.D, dc.nf, dc.vtile, dc.nth, flux_blocks(dc, r), r, st, &dc, nullptr, nullptr, 0);
+        if (e == cudaSuccess)
+            e = launch_stage1<T>(dc.D, dc.nf, stage1_blocks(dc, r), r, st, &dc, nullptr, nullptr, 0);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 // Blocks, threads and dynamic shared memory of the per-case kernels of a step
@@ -2223,7 +2355,7 @@ static void pre_gather(const DevCase<T> &dc, cudaStream_t st, cudaEvent_t *ev)
 }
 
 template <typename T, int D, int NC>
-static void post_gather(const DevCase<T> &dc, const StepConfig &, cudaStream_t st, cudaEvent_t *ev)
+static void post_gather(const DevCase<T> &dc, cudaStream_t st, cudaEvent_t *ev)
 {
     auto mark = [&](int i) {
         if (ev) cudaEventRecord(ev[i], st);
@@ -2236,12 +2368,12 @@ static void post_gather(const DevCase<T> &dc, const StepConfig &, cudaStream_t s
 }
 
 template <typename T, int D, int NC>
-static cudaError_t step_dn(const DevCase<T> &dc, const StepConfig &cfg, cudaStream_t st, cudaEvent_t *ev)
+static cudaError_t step_dn(const DevCase<T> &dc, cudaStream_t st, cudaEvent_t *ev)
 {
     pre_gather<T, D, NC>(dc, st, ev);
-    cudaError_t e = gather_dispatch<T, D, NC>(dc, cfg.smem, st);
+    cudaError_t e = launch_gather(dc, st);
     if (e != cudaSuccess) return e;
-    post_gather<T, D, NC>(dc, cfg, st, ev);
+    post_gather<T, D, NC>(dc, st, ev);
     return cudaGetLastError();
 }
 
@@ -2250,14 +2382,6 @@ cudaError_t launch_pre_gather(const DevCase<T> &dc, cudaStream_t st)
 {
     if (dc.D == 2) pre_gather<T, 2, 2>(dc, st, nullptr);
     else pre_gather<T, 3, 1>(dc, st, nullptr);
-    return cudaGetLastError();
-}
-
-template <typename T>
-cudaError_t launch_post_gather(const DevCase<T> &dc, const StepConfig &cfg, cudaStream_t st)
-{
-    if (dc.D == 2) post_gather<T, 2, 2>(dc, cfg, st, nullptr);
-    else post_gather<T, 3, 1>(dc, cfg, st, nullptr);
     return cudaGetLastError();
 }
 
@@ -2282,81 +2406,9 @@ cudaError_t launch_small_batch(int D, int k, const DevCase<T> *cases, const int 
 }
 
 template <typename T>
-cudaError_t launch_gather(const DevCase<T> &dc, size_t smem, cudaStream_t st)
+cudaError_t launch_step(const DevCase<T> &dc, cudaStream_t st, cudaEvent_t *ev)
 {
-    if (dc.D == 2) return gather_dispatch<T, 2, 2>(dc, smem, st);
-    return gather_dispatch<T, 3, 1>(dc, smem, st);
-}
-
-template <typename T, int D, int NC, int TV, int NTH>
-static cudaError_t gather_batch_launch(const DevCase<T> *cases, const int4 *work, int nwork, int grid, size_t smem,
-                                       cudaStream_t st)
-{
-    auto kern = k_gather_batch<T, D, NC, TV, NTH>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    kern<<<grid, NTH, smem, st>>>(cases, work, nwork);
-    return cudaGetLastError();
-}
-
-template <typename T, int D, int NC>
-static cudaError_t gather_batch_dispatch(int vtile, int nth, const DevCase<T> *cases, const int4 *work, int nwork,
-                                         int grid, size_t smem, cudaStream_t st)
-{
-    const int tv = vtile / 32;
-    if (nth == 512) {
-        if constexpr (std::is_same<T, float>::value) {
-            if (tv == 1) return gather_batch_launch<T, D, NC, 1, 512>(cases, work, nwork, grid, smem, st);
-            if (tv == 2) return gather_batch_launch<T, D, NC, 2, 512>(cases, work, nwork, grid, smem, st);
-        }
-        return cudaErrorInvalidValue;
-    }
-    if (nth != 256) return cudaErrorInvalidValue;
-    if (tv == 1) return gather_batch_launch<T, D, NC, 1, 256>(cases, work, nwork, grid, smem, st);
-    if (tv == 2) return gather_batch_launch<T, D, NC, 2, 256>(cases, work, nwork, grid, smem, st);
-    if (tv == 4) return gather_batch_launch<T, D, NC, 4, 256>(cases, work, nwork, grid, smem, st);
-    return cudaErrorInvalidValue;
-}
-
-template <typename T>
-cudaError_t launch_gather_batch(int D, int vtile, int nth, const DevCase<T> *cases, const int4 *work, int nwork,
-                                int grid, size_t smem, cudaStream_t st)
-{
-    if (D == 2) return gather_batch_dispatch<T, 2, 2>(vtile, nth, cases, work, nwork, grid, smem, st);
-    return gather_batch_dispatch<T, 3, 1>(vtile, nth, cases, work, nwork, grid, smem, st);
-}
-
-// CTAs of the gather kernel that fit on the device at once (persistent grid)
-template <typename T>
-int gather_resident_ctas(int D, int vtile, int nth, size_t smem)
-{
-    int dev = 0, nsm = 0, per = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    const int tv = vtile / 32;
-    const void *fn = nullptr;
-    if (nth == 512 && std::is_same<T, float>::value) {
-        if (D == 2) fn = tv == 1 ? (const void *)k_gather_batch<T, 2, 2, 1, 512> : (const void *)k_gather_batch<T, 2, 2, 2, 512>;
-        else fn = tv == 1 ? (const void *)k_gather_batch<T, 3, 1, 1, 512> : (const void *)k_gather_batch<T, 3, 1, 2, 512>;
-    } else {
-        if (D == 2)
-            fn = tv == 1   ? (const void *)k_gather_batch<T, 2, 2, 1, 256>
-                 : tv == 2 ? (const void *)k_gather_batch<T, 2, 2, 2, 256>
-                           : (const void *)k_gather_batch<T, 2, 2, 4, 256>;
-        else
-            fn = tv == 1   ? (const void *)k_gather_batch<T, 3, 1, 1, 256>
-                 : tv == 2 ? (const void *)k_gather_batch<T, 3, 1, 2, 256>
-                           : (const void *)k_gather_batch<T, 3, 1, 4, 256>;
-    }
-    cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn, nth, smem);
-    return std::max(1, per) * std::max(1, nsm);
-}
-
-template <typename T>
-cudaError_t launch_step(const DevCase<T> &dc, const StepConfig &cfg, cudaStream_t st, cudaEvent_t *ev)
-{
-    return dc.D == 2 ? step_dn<T, 2, 2>(dc, cfg, st, ev) : step_dn<T, 3, 1>(dc, cfg, st, ev);
+    return dc.D == 2 ? step_dn<T, 2, 2>(dc, st, ev) : step_dn<T, 3, 1>(dc, st, ev);
 }
 
 template <typename T>
@@ -2464,8 +2516,6 @@ cudaError_t launch_density_range(const double *W, int C, int M, const unsigned c
 
 template cudaError_t launch_pre_gather<double>(const DevCase<double> &, cudaStream_t);
 template cudaError_t launch_pre_gather<float>(const DevCase<float> &, cudaStream_t);
-template cudaError_t launch_post_gather<double>(const DevCase<double> &, const StepConfig &, cudaStream_t);
-template cudaError_t launch_post_gather<float>(const DevCase<float> &, const StepConfig &, cudaStream_t);
 template int small_kernel_blocks<double>(const DevCase<double> &, int);
 template int small_kernel_blocks<float>(const DevCase<float> &, int);
 template size_t small_kernel_smem<double>(const DevCase<double> &, int);
@@ -2474,16 +2524,18 @@ template cudaError_t launch_small_batch<double>(int, int, const DevCase<double> 
                                                 cudaStream_t);
 template cudaError_t launch_small_batch<float>(int, int, const DevCase<float> *, const int *, int, int, size_t,
                                                cudaStream_t);
-template cudaError_t launch_gather<double>(const DevCase<double> &, size_t, cudaStream_t);
-template cudaError_t launch_gather<float>(const DevCase<float> &, size_t, cudaStream_t);
-template cudaError_t launch_gather_batch<double>(int, int, int, const DevCase<double> *, const int4 *, int, int, size_t,
-                                                 cudaStream_t);
-template cudaError_t launch_gather_batch<float>(int, int, int, const DevCase<float> *, const int4 *, int, int, size_t,
-                                                cudaStream_t);
-template int gather_resident_ctas<double>(int, int, int, size_t);
-template int gather_resident_ctas<float>(int, int, int, size_t);
-template cudaError_t launch_step<double>(const DevCase<double> &, const StepConfig &, cudaStream_t, cudaEvent_t *);
-template cudaError_t launch_step<float>(const DevCase<float> &, const StepConfig &, cudaStream_t, cudaEvent_t *);
+#define UGKS_GATHER(T)                                                                                        \
+    template cudaError_t launch_flux<T>(int, int, int, int, int, int, cudaStream_t, const DevCase<T> *,       \
+                                        const DevCase<T> *, const int *, int);                                \
+    template cudaError_t launch_stage1<T>(int, int, int, int, cudaStream_t, const DevCase<T> *,               \
+                                          const DevCase<T> *, const int *, int);                              \
+    template int flux_blocks<T>(const DevCase<T> &, int);                                                     \
+    template int stage1_blocks<T>(const DevCase<T> &, int);                                                   \
+    template cudaError_t launch_gather<T>(const DevCase<T> &, cudaStream_t);                                  \
+    template cudaError_t launch_step<T>(const DevCase<T> &, cudaStream_t, cudaEvent_t *);
+UGKS_GATHER(double)
+UGKS_GATHER(float)
+#undef UGKS_GATHER
 template cudaError_t launch_init<double>(const DevCase<double> &, cudaStream_t);
 template cudaError_t launch_init<float>(const DevCase<float> &, cudaStream_t);
 template cudaError_t launch_heatflux<double>(const DevCase<double> &, cudaStream_t);

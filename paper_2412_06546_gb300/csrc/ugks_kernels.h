@@ -6,26 +6,27 @@
 
 namespace ugks {
 
-struct StepConfig {
-    size_t smem;        // dynamic shared memory of the gather kernel
-    int n_res_blocks;   // blocks of k_update_W (residual partials)
-};
-
 // kernel groups of one step, in launch order (timed by events when profiling)
 enum { G_PREP = 0, G_FACE = 1, G_WALL = 2, G_GATHER = 3, G_UPDATE = 4, G_COLLIDE = 5, N_GROUPS = 6 };
 template <typename T>
-cudaError_t launch_step(const DevCase<T> &dc, const StepConfig &cfg, cudaStream_t st, cudaEvent_t *ev = nullptr);
+cudaError_t launch_step(const DevCase<T> &dc, cudaStream_t st, cudaEvent_t *ev = nullptr);
 template <typename T> cudaError_t launch_init(const DevCase<T> &dc, cudaStream_t st);
-// the step split around the gather pass, for batched steps
+// the part of a step before the flux pass (autotuner)
 template <typename T> cudaError_t launch_pre_gather(const DevCase<T> &dc, cudaStream_t st);
-template <typename T> cudaError_t launch_post_gather(const DevCase<T> &dc, const StepConfig &cfg, cudaStream_t st);
-template <typename T> cudaError_t launch_gather(const DevCase<T> &dc, size_t smem, cudaStream_t st);
-// persistent gather over a work list of int4 (case, patch, velocity tile, 0) items;
-// cases[] is a device array of DevCase with the same D, vtile and threads per CTA
+// the flux and stage-1 passes over all chunks of a case
+template <typename T> cudaError_t launch_gather(const DevCase<T> &dc, cudaStream_t st);
+// one chunk's flux or stage-1 kernel, for one case (dc) or for n cases in one
+// launch: cases[] a device array of their DevCase with the same D, nf, vtile and
+// threads per CTA, off[0..n] the device prefix sums of their block counts,
+// blocks = off[n]
 template <typename T>
-cudaError_t launch_gather_batch(int D, int vtile, int nth, const DevCase<T> *cases, const int4 *work, int nwork,
-                                int grid, size_t smem, cudaStream_t st);
-template <typename T> int gather_resident_ctas(int D, int vtile, int nth, size_t smem);
+cudaError_t launch_flux(int D, int nf, int vtile, int nth, int blocks, int chunk, cudaStream_t st,
+                        const DevCase<T> *dc, const DevCase<T> *cases, const int *off, int n);
+template <typename T>
+cudaError_t launch_stage1(int D, int nf, int blocks, int chunk, cudaStream_t st, const DevCase<T> *dc,
+                          const DevCase<T> *cases, const int *off, int n);
+template <typename T> int flux_blocks(const DevCase<T> &dc, int chunk);
+template <typename T> int stage1_blocks(const DevCase<T> &dc, int chunk);
 // The per-case kernels of a step, in launch order: pre-gather (SK_PREP ..
 // SK_WALL_SUM), then after the gather SK_UPDATE_W and SK_COLLIDE.
 enum SmallKernel {

@@ -58,19 +58,22 @@ struct Request {
 };
 
 // Device bytes a case will hold, from its sizes (an upper bound of what
-// ugks_create allocates: two copies of f, FP64 cell / face arrays and records).
+// ugks_create allocates: f and the flux buffer, which is at most a copy of f, or
+// up to 4 MB or 128 velocities where that is more, FP64 cell / face arrays and
+// records).
 size_t footprint_estimate(const Request &r)
 {
     const int D = r.D, M = D + 2, NC = D == 2 ? 2 : 1;
     const size_t s = r.params.precision == UGKS_FP64 ? 8 : 4;
     const size_t nvp = (size_t)((r.Nv + 127) / 128 * 128);
     const size_t C = (size_t)r.C, F = (size_t)std::max<int64_t>(r.F, 1);
-    size_t b = 2 * C * NC * nvp * s;                                   // f_cur, f_nxt
+    const size_t f = C * NC * nvp * s, vel = F * NC * s;
+    size_t b = f + std::max({f, std::min<size_t>((size_t)4 << 20, vel * nvp), vel * 128});   // f, fluxes
     b += C * (size_t)(M * 2 + D + D * M * 2 + 8) * 8;                  // W, q, prim, gradients, vol
     b += C * 2 * 12 * s + C * (nvp / 32 + 1) * M * s;                  // records, residual partials
     b += F * (size_t)(40 * s + 24 * s + 16 * s + (D * M + D + D + M + M + 5) * 8 + 60 * 8 + 64);
     b += 2 * F * (size_t)(8 * D + 24) + C * 64 + nvp * 64;             // geometry, LSQ, patches
-    b += 2 * F * (size_t)(16 + 16 * s);                                // gather entries
+    b += 2 * F * (size_t)(16 + 16 * s);                                // entries
     b += (size_t)64 * 256 * 40;                                        // allocation rounding
     return b + b / 8;
 }
