@@ -8,7 +8,7 @@
 //   W      [C][D+2]      f64 conserved variables
 //   q      [C][D]        f64 heat flux of f^n
 //   cell records [C][CREC] T   Maxwellian / Shakhov / collision coefficients
-//   face records [F][FREC] T   interface equilibrium g0, its slopes, q1..q5
+//   flux records [F][XREC] T   interface equilibrium g0, its slopes, q1, q2
 // T is the per-velocity arithmetic type (double or float).
 #pragma once
 #include <cstdint>
@@ -24,10 +24,8 @@ constexpr int MAXM = 5;
 enum { CR_U = 0, CR_LAM = 3, CR_PREF = 4, CR_KQ = 5, CR_C = 8, CR_NB = 9, CR_NL2 = 10, CR_INV = 11, CREC = 12 };
 // ghost / side / wall record: a Maxwellian
 enum { GR_U = 0, GR_LAM = 3, GR_PREF = 4, GR_NB = 5, GR_NL2 = 6, GREC = 8 };
-// face record: g0 of the interface, Shakhov factor, time integrals, slopes in
-// the basis centred at U0: psi_c = (1, c, (|c|^2 + xi^2)/2), c = u - U0
-enum { FR_U = 0, FR_LAM = 3, FR_PREF = 4, FR_KQ = 5, FR_QS = 8, FR_NB = 13, FR_XB = 14,
-       FR_BETA = 15, FR_NL2 = 39, FREC = 40 };
+// face record: the Maxwellian g0 of the interface, read by the sums of k_face_sum2
+enum { FR_U = 0, FR_LAM = 3, FR_PREF = 4, FR_NL2 = 5, FREC = 8 };
 
 // flux record read by the flux pass: the equilibrium part of the
 // time-integrated interface distribution, q3 (g0 + g0+) + q4 u.grad g0 +
@@ -74,7 +72,8 @@ struct DevCase {
     int D, NC;
     int C, F, G, NW;         // cells, faces, far-field ghosts, wall faces
     int nv, nvp;             // velocities, padded count
-    double dt, Pr, omega, mu_ref, nxi;
+    double dt, Pr, omega, nxi;
+    double dt_mu;                 // dt / mu_ref (0: collisionless)
     int limiter;
     int w0_analytic;              // 1: W0 from the analytic half-range moments
     // velocity grid (padded), FP64 and T copies
@@ -141,7 +140,7 @@ struct DevCase {
     double *fprim0;               // [F][D+2] rho0, U0, lam0
     double *fqs;                  // [F][5] time integrals q1..q5 of the interface
     double *dW_part;              // [C][n_groups][D+2] moments of the flux residual over gvel velocities
-    double *res_part;             // [n_res_blocks][2(D+2)]
+    double *res_part;             // [ceil(C / 32)][2(D+2)]
     const unsigned char *owned;   // [C] 1 for cells whose residual counts (a subdomain's own cells),
                                   // nullptr: every cell
     int *flags;                   // [1] numeric failure flag

@@ -68,7 +68,7 @@ struct ugks_case {
     double *res_d = nullptr;       // [M]
     int *flags_d = nullptr;
     unsigned long long *range_d = nullptr;   // [2] bit patterns of the min and max density
-    int n_res_blocks = 0;
+    int n_res_parts = 0;
     bool stepped = false;
     // kernel-group profiling
     std::vector<cudaEvent_t> prof_ev;
@@ -529,9 +529,10 @@ void fill_case(ugks_case *c, ugks::DevCase<T> &dc, const ugks_mesh *m, const ugk
     dc.Pr = p->Pr;
     dc.omega = p->omega;
     dc.nxi = 3.0 - D;
-    dc.mu_ref = std::isinf(p->Kn) ? INFINITY
-                                  : 15.0 * std::sqrt(2.0 * M_PI) * p->Kn * p->L_ref /
-                                        (2.0 * (5.0 - 2.0 * p->omega) * (7.0 - 2.0 * p->omega));
+    // VHS viscosity at the reference state (Bird's mean free path)
+    const double mu_ref = 15.0 * std::sqrt(2.0 * M_PI) * p->Kn * p->L_ref /
+                          (2.0 * (5.0 - 2.0 * p->omega) * (7.0 - 2.0 * p->omega));
+    dc.dt_mu = std::isinf(p->Kn) ? 0.0 : c->dt / mu_ref;
     dc.limiter = p->limiter ? 1 : 0;
     dc.w0_analytic = p->w0_analytic ? 1 : 0;
     // velocities, padded with u = 0, w = 0
@@ -720,7 +721,7 @@ void fill_case(ugks_case *c, ugks::DevCase<T> &dc, const ugks_mesh *m, const ugk
     dc.fprim0 = (double *)c->dalloc(Fm * M * sizeof(double));
     dc.fqs = (double *)c->dalloc(Fm * 5 * sizeof(double));
     dc.dW_part = (double *)c->dalloc((size_t)c->C * c->n_groups * M * sizeof(double));
-    dc.res_part = (double *)c->dalloc((size_t)c->n_res_blocks * 2 * M * sizeof(double));
+    dc.res_part = (double *)c->dalloc((size_t)c->n_res_parts * 2 * M * sizeof(double));
     dc.flags = c->flags_d;
     dc.owned = nullptr;
     dc.gvel = c->gvel;
@@ -1020,7 +1021,7 @@ ugks_status ugks_create(const ugks_mesh *mesh, const ugks_vgrid *vgrid, const ug
         c->NW = (int)h.wface.size();
         // upwind CFL bound (the CFL step of Algorithm 1)
         c->dt = params->dt > 0.0 ? params->dt : cfl_dt_of(mesh, vgrid, params->cfl, mesh->n_cells);
-        c->n_res_blocks = (int)((c->C + 255) / 256);
+        c->n_res_parts = (int)((c->C + 31) / 32);
         c->flags_d = (int *)c->dalloc(sizeof(int));
         cuda_ok(cudaMemsetAsync(c->flags_d, 0, sizeof(int), c->stream), "memset");
         c->range_d = (unsigned long long *)c->dalloc(2 * sizeof(unsigned long long));
@@ -1134,7 +1135,7 @@ ugks_status ugks_residual(ugks_case *c, double *res)
             return;
         }
         const double *rp = c->prec == UGKS_FP64 ? c->d64.res_part : c->d32.res_part;
-        cuda_ok(ugks::launch_residual(rp, c->n_res_blocks, c->D, c->res_d, c->stream), "residual launch");
+        cuda_ok(ugks::launch_residual(rp, c->n_res_parts, c->D, c->res_d, c->stream), "residual launch");
         cuda_ok(cudaMemcpyAsync(res, c->res_d, M * sizeof(double), cudaMemcpyDeviceToHost, c->stream), "residual copy");
         cuda_ok(cudaStreamSynchronize(c->stream), "residual sync");
     });
@@ -1318,12 +1319,12 @@ ugks_status ugks_residual_sums(ugks_case *c, double *sums)
         const int M = c->D + 2;
         for (int i = 0; i < 2 * M; ++i) sums[i] = 0.0;
         if (!c->stepped) return;
-        std::vector<double> part((size_t)c->n_res_blocks * 2 * M);
+        std::vector<double> part((size_t)c->n_res_parts * 2 * M);
         const double *rp = c->prec == UGKS_FP64 ? c->d64.res_part : c->d32.res_part;
         cuda_ok(cudaMemcpyAsync(part.data(), rp, part.size() * sizeof(double), cudaMemcpyDeviceToHost, c->stream),
                 "residual copy");
         cuda_ok(cudaStreamSynchronize(c->stream), "residual sync");
-        for (int b = 0; b < c->n_res_blocks; ++b)
+        for (int b = 0; b < c->n_res_parts; ++b)
             for (int i = 0; i < 2 * M; ++i) sums[i] += part[(size_t)b * 2 * M + i];
     });
 }
@@ -1405,7 +1406,7 @@ struct ugks_batch {
     // off[k][0..n] (device, prefix sums of the cases' block counts), total
     // blocks and dynamic shared memory per kernel
     int *small_off = nullptr;
-    int small_blocks[ugks::SK_COUNT] = {};
+    int small_blocks[ugks::SK_COUNT] = {}, small_threads[ugks::SK_COUNT] = {};
     size_t small_smem[ugks::SK_COUNT] = {};
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
@@ -1434,8 +1435,12 @@ void batch_build(ugks_batch *b)
     std::vector<int> off((size_t)ugks::SK_COUNT * (n + 1), 0);
     for (int k = 0; k < ugks::SK_COUNT; ++k) {
         int *o = &off[(size_t)k * (n + 1)];
+        long long items = 0;
+        for (int i = 0; i < n; ++i) items += ugks::small_kernel_items<T>(h[i], k);
+        b->small_threads[k] = ugks::small_kernel_threads(k, items);
         for (int i = 0; i < n; ++i) {
-            const long long nb = (long long)o[i] + ugks::small_kernel_blocks<T>(h[i], k);
+            const long long nb = (long long)o[i] + ugks::small_kernel_blocks(k, ugks::small_kernel_items<T>(h[i], k),
+                                                                             b->small_threads[k]);
             if (nb > INT32_MAX) fail(UGKS_EINVAL, "batch too large for one launch of kernel %d", k);
             o[i + 1] = (int)nb;
             b->small_smem[k] = std::max(b->small_smem[k], ugks::small_kernel_smem<T>(h[i], k));
@@ -1481,7 +1486,7 @@ void batch_capture(ugks_batch *b)
     const auto *dcs = (const ugks::DevCase<T> *)b->dcases;
     auto small = [&](int k) {
         cuda_ok(ugks::launch_small_batch<T>(b->D, k, dcs, b->small_off + (size_t)k * (n + 1), n, b->small_blocks[k],
-                                            b->small_smem[k], st),
+                                            b->small_threads[k], b->small_smem[k], st),
                 "batched step kernel");
     };
     cuda_ok(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal), "begin capture");

@@ -39,69 +39,90 @@ __device__ __forceinline__ Prim prim_of(const double *W, int D)
 {
     Prim p;
     p.rho = W[0];
+    const double ir = 1.0 / W[0];
     double ke = 0.0;
     for (int d = 0; d < MAXD; ++d) p.U[d] = 0.0;
     for (int d = 0; d < D; ++d) {
-        p.U[d] = W[1 + d] / W[0];
+        p.U[d] = W[1 + d] * ir;
         ke += p.U[d] * p.U[d];
     }
-    double E = W[D + 1] / W[0];
-    p.T = (2.0 / 3.0) * (E - 0.5 * ke);
-    p.lam = 1.0 / (2.0 * p.T);
+    p.T = (2.0 / 3.0) * (W[D + 1] * ir - 0.5 * ke);
+    p.lam = 0.5 / p.T;
     return p;
+}
+
+// the same from a primitive row (rho, U, T)
+template <int D> __device__ __forceinline__ void set_prim(const double *P, Prim &p)
+{
+    p.rho = P[0];
+    for (int d = 0; d < MAXD; ++d) p.U[d] = d < D ? P[1 + d] : 0.0;
+    p.T = P[D + 1];
+    p.lam = 0.5 / p.T;
 }
 
 constexpr double LOG2E = 1.4426950408889634073599246810018921;
 
 __device__ __forceinline__ double pref_of(double rho, double lam, int D)
 {
-    double a = lam / 3.141592653589793238462643383279502884;
+    const double a = lam * 0.31830988618379067153776752674502872;    // 1 / pi
     return D == 2 ? rho * a : rho * a * sqrt(a);
 }
 
-// collision time tau = mu_ref T^omega / (rho T)  (VHS viscosity, p = rho T)
+// dt / tau of a state, tau = mu_ref T^omega / (rho T) (VHS viscosity, p = rho T)
 template <typename T>
-__device__ __forceinline__ double tau_of(const DevCase<T> &dc, double rho, double Tmp)
+__device__ __forceinline__ double dt_over_tau(const DevCase<T> &dc, double rho, double Tmp)
 {
-    return dc.mu_ref * pow(Tmp, dc.omega) / (rho * Tmp);
+    return dc.dt_mu * rho * pow(Tmp, 1.0 - dc.omega);
+}
+
+// a record of Maxwellian, Shakhov and collision coefficients (CR_*) of the state
+// p with heat flux q; the divisions and the power are the length of the
+// kernels that form them (an FP64 operation has a latency of about 70 cycles)
+template <typename T, int D>
+__device__ __forceinline__ void cell_record(const DevCase<T> &dc, const Prim &p, const double *q, T *r)
+{
+    const double cc = 0.5 * dt_over_tau(dc, p.rho, p.T);
+    const double kappa = 0.8 * (1.0 - dc.Pr) * p.lam * p.lam / p.rho;
+    for (int d = 0; d < 3; ++d) r[CR_U + d] = (T)p.U[d];
+    r[CR_LAM] = (T)p.lam;
+    r[CR_PREF] = (T)pref_of(p.rho, p.lam, D);
+    for (int d = 0; d < 3; ++d) r[CR_KQ + d] = d < D ? (T)(kappa * q[d]) : T(0);
+    r[CR_C] = (T)cc;
+    r[CR_INV] = (T)(1.0 / (1.0 + cc));
+    r[CR_NB] = (T)(dc.nxi * p.T);
+    r[CR_NL2] = (T)(-p.lam * LOG2E);
 }
 
 // Time integrals of c1..c5 over [0, dt] (Sec. 2.4), written with x = dt/tau,
 // E = 1 - e^{-x}:  q1 = dt E/x, q2 = dt^2 (x e^{-x} - E)/x^2, q3 = dt (x - E)/x,
 // q4 = dt^2 (2E - x(1 + e^{-x}))/x^2, q5 = dt^2 (x^2/2 - x + E)/x^2.
-// Below x = 1/2 each bracket is summed from its Taylor series.
-__device__ void time_integrals(double dt, double tau, double q[5])
+// Below x = 1/2 the brackets cancel; with phi_n = sum_i (-x)^i / (i + n)! they
+// are phi_1, phi_2 - phi_1, x phi_2, -x (phi_2 - 2 phi_3) and x phi_3, where
+// phi_3 is summed to rounding and phi_2 = 1/2 - x phi_3, phi_1 = 1 - x phi_2.
+// (Summing the five series term by term took about 500 FP64 operations; an SM
+// retires 1.6 of them per cycle and lane-wise that was half of k_face_fin1.)
+__device__ __forceinline__ void time_integrals(double dt, double x, double q[5])
 {
-    const double x = dt / tau;
     if (x < 0.5) {
-        double s1 = 0, s2 = 0, s3 = 0, s4 = 0, s5 = 0;
-        double xp = 1.0;       // x^{j-2} for j >= 2
-        double inv_fact = 1.0; // 1/j!
-        double xm1 = 1.0;      // x^{j-1}
-        for (int j = 1; j <= 22; ++j) {
-            inv_fact /= (double)j;
-            const double sg = (j & 1) ? 1.0 : -1.0;   // (-1)^{j+1}
-            s1 += sg * xm1 * inv_fact;                  // E/x
-            if (j >= 2) {
-                const double xm2 = xp;                  // x^{j-2}
-                s2 += sg * (1.0 - (double)j) * xm2 * inv_fact;   // (E - x e)/x^2
-                s3 += -sg * xm1 * inv_fact;                      // (x - E)/x
-                if (j >= 3) {
-                    s4 += sg * (2.0 - (double)j) * xm2 * inv_fact;   // (2E - x(1+e))/x^2
-                    s5 += sg * xm2 * inv_fact;                        // (x^2/2 - x + E)/x^2
-                }
-                xp *= x;
-            }
-            xm1 *= x;
+        double f = 1.0;                    // (i + 3)! upwards, folded at compile time
+        double c[14];
+#pragma unroll
+        for (int i = 0; i < 14; ++i) {
+            f *= i == 0 ? 6.0 : (double)(i + 3);
+            c[i] = (i & 1 ? -1.0 : 1.0) / f;
         }
-        q[0] = dt * s1;
-        q[1] = -dt * dt * s2;
-        q[2] = dt * s3;
-        q[3] = dt * dt * s4;
-        q[4] = dt * dt * s5;
+        double p3 = c[13];
+#pragma unroll
+        for (int i = 12; i >= 0; --i) p3 = fma(p3, x, c[i]);
+        const double p2 = fma(-x, p3, 0.5), p1 = fma(-x, p2, 1.0);
+        q[0] = dt * p1;
+        q[1] = dt * dt * (p2 - p1);
+        q[2] = dt * x * p2;
+        q[3] = -dt * dt * x * fma(-2.0, p3, p2);
+        q[4] = dt * dt * x * p3;
     } else {
         const double e = exp(-x);
-        const double E = -expm1(-x);
+        const double E = 1.0 - e;
         const double ix = 1.0 / x, ix2 = ix * ix;
         q[0] = dt * E * ix;
         q[1] = dt * dt * (x * e - E) * ix2;
@@ -109,15 +130,6 @@ __device__ void time_integrals(double dt, double tau, double q[5])
         q[3] = dt * dt * (2.0 * E - x * (1.0 + e)) * ix2;
         q[4] = dt * dt * (0.5 * x * x - x + E) * ix2;
     }
-}
-
-// Venkatakrishnan factor on FP64 data (macro reconstruction)
-__device__ __forceinline__ double venkat_d(double d1, double d2, double e2)
-{
-    double a2 = d1 * d1 + e2;
-    double num = a2 + 2.0 * d1 * d2;
-    double den = a2 + d2 * (2.0 * d2 + d1);
-    return den > 0.0 ? num / den : 1.0;
 }
 
 // ------------------------------------------------------------ batched launches
@@ -162,7 +174,7 @@ __global__ void k_init_f(DevCase<T> dc)
     for (int d = 0; d < 3; ++d) rec[GR_U + d] = (T)p.U[d];
     rec[GR_LAM] = (T)p.lam;
     rec[GR_PREF] = (T)pref_of(p.rho, p.lam, D);
-    rec[GR_NB] = (T)(dc.nxi / (2.0 * p.lam));
+    rec[GR_NB] = (T)(dc.nxi * p.T);
     rec[GR_NL2] = (T)(-p.lam * LOG2E);
     const size_t rs = (size_t)NC * dc.nvp;
     for (int k = lane; k < dc.nvp; k += 32) {
@@ -215,18 +227,7 @@ __device__ __forceinline__ void prep_body(const DevCase<T> &dc, const int bx)
         Pc[0] = p.rho;
         for (int d = 0; d < D; ++d) Pc[1 + d] = p.U[d];
         Pc[D + 1] = p.T;
-        double tau = tau_of(dc, p.rho, p.T);
-        double kappa = 4.0 * (1.0 - dc.Pr) * p.lam * p.lam / (5.0 * p.rho);
-        T *r = dc.crec + (size_t)c * CREC;
-        for (int d = 0; d < 3; ++d) r[CR_U + d] = (T)p.U[d];
-        r[CR_LAM] = (T)p.lam;
-        r[CR_PREF] = (T)pref_of(p.rho, p.lam, D);
-        for (int d = 0; d < 3; ++d) r[CR_KQ + d] = d < D ? (T)(kappa * dc.q[(size_t)c * D + d]) : T(0);
-        const double cc = 0.5 * dc.dt / tau;
-        r[CR_C] = (T)cc;
-        r[CR_INV] = (T)(1.0 / (1.0 + cc));
-        r[CR_NB] = (T)(dc.nxi / (2.0 * p.lam));
-        r[CR_NL2] = (T)(-p.lam * LOG2E);
+        cell_record<T, D>(dc, p, dc.q + (size_t)c * D, dc.crec + (size_t)c * CREC);
         return;
     }
     const int g = t - dc.C;
@@ -249,7 +250,7 @@ __device__ __forceinline__ void prep_body(const DevCase<T> &dc, const int bx)
     for (int d = 0; d < 3; ++d) r[GR_U + d] = (T)p.U[d];
     r[GR_LAM] = (T)p.lam;
     r[GR_PREF] = (T)pref_of(p.rho, p.lam, D);
-    r[GR_NB] = (T)(dc.nxi / (2.0 * p.lam));
+    r[GR_NB] = (T)(dc.nxi * p.T);
     r[GR_NL2] = (T)(-p.lam * LOG2E);
 }
 
@@ -280,33 +281,66 @@ __device__ __forceinline__ void macro_grad_body(const DevCase<T> &dc, const int 
     const int q0 = dc.nb_ptr[c], q1 = dc.nb_ptr[c + 1];
     const int s0 = dc.cf_ptr[c], s1 = dc.cf_ptr[c + 1];
     const double e2 = dc.eps2_d[c];
-    double gp[D][M];
+    // every neighbour's row is read once for all components; the limiter's
+    // factor is taken at the largest and the most negative offset, as in
+    // cell_slope, with one division per component
+    double gp[D][M], vi[M];
+    Extrema<double> ex[M], d2x[M];
+#pragma unroll
     for (int m = 0; m < M; ++m) {
-        const double vi = Pc[m];
-        double g[D], vmax = vi, vmin = vi;
-        for (int d = 0; d < D; ++d) g[d] = 0.0;
-        for (int q = q0; q < q1; ++q) {
-            const int id = dc.nb_id[q];
-            const double vj = id >= 0 ? dc.prim[(size_t)id * M + m] : dc.primg[(size_t)(-id - 1) * M + m];
-            for (int d = 0; d < D; ++d) g[d] += dc.nb_a_d[(size_t)q * D + d] * (vj - vi);
-            vmax = fmax(vmax, vj);
-            vmin = fmin(vmin, vj);
-        }
-        if (dc.limiter) {
-            double phi = 1.0;
-            for (int s = s0; s < s1; ++s) {
-                double d2 = 0.0;
-                for (int d = 0; d < D; ++d) d2 += g[d] * dc.cf_r_d[(size_t)s * D + d];
-                double d1 = d2 > 0.0 ? vmax - vi : vmin - vi;
-                phi = fmin(phi, venkat_d(d1, d2, e2));
-            }
-            for (int d = 0; d < D; ++d) g[d] *= phi;
-        }
-        for (int d = 0; d < D; ++d) {
-            gp[d][m] = g[d];
-            dc.gradprim[((size_t)c * D + d) * M + m] = g[d];
+        vi[m] = Pc[m];
+        ex[m].set(vi[m]);
+        d2x[m].set(0.0);
+#pragma unroll
+        for (int d = 0; d < D; ++d) gp[d][m] = 0.0;
+    }
+    for (int q = q0; q < q1; ++q) {
+        const int id = dc.nb_id[q];
+        const double *row = id >= 0 ? dc.prim + (size_t)id * M : dc.primg + (size_t)(-id - 1) * M;
+        double a[D];
+#pragma unroll
+        for (int d = 0; d < D; ++d) a[d] = dc.nb_a_d[(size_t)q * D + d];
+#pragma unroll
+        for (int m = 0; m < M; ++m) {
+            const double vj = row[m], df = vj - vi[m];
+#pragma unroll
+            for (int d = 0; d < D; ++d) gp[d][m] += a[d] * df;
+            ex[m].add(vj);
         }
     }
+    if (dc.limiter) {
+        for (int s = s0; s < s1; ++s) {
+            double r[D];
+#pragma unroll
+            for (int d = 0; d < D; ++d) r[d] = dc.cf_r_d[(size_t)s * D + d];
+#pragma unroll
+            for (int m = 0; m < M; ++m) {
+                double d2 = 0.0;
+#pragma unroll
+                for (int d = 0; d < D; ++d) d2 += gp[d][m] * r[d];
+                d2x[m].add(d2);
+            }
+        }
+#pragma unroll
+        for (int m = 0; m < M; ++m) {
+            double num[2], den[2];
+#pragma unroll
+            for (int s = 0; s < 2; ++s) {
+                const double d1 = (s ? ex[m].bottom() : ex[m].top()) - vi[m];
+                const double d2 = s ? d2x[m].bottom() : d2x[m].top();
+                const double a2 = d1 * d1 + e2;
+                num[s] = a2 + 2.0 * d1 * d2;
+                den[s] = a2 + d2 * (2.0 * d2 + d1);
+            }
+            const double phi = min_ratio(num[0], den[0], num[1], den[1]);
+#pragma unroll
+            for (int d = 0; d < D; ++d) gp[d][m] *= phi;
+        }
+    }
+#pragma unroll
+    for (int d = 0; d < D; ++d)
+#pragma unroll
+        for (int m = 0; m < M; ++m) dc.gradprim[((size_t)c * D + d) * M + m] = gp[d][m];
     double uu = 0.0;
     for (int e = 0; e < D; ++e) uu += Pc[1 + e] * Pc[1 + e];
     for (int d = 0; d < D; ++d) {
@@ -336,39 +370,33 @@ __global__ void k_macro_grad_batch(const DevCase<T> *__restrict__ cases, const i
 }
 
 // ------------------------------------------------------------ face pass
-// face state reconstructed in primitive variables, P_c + gradP_c . r, returned
-// as conserved variables; the cell average is used if rho or T would not be
-// positive
+// face state P_c + gradP_c . r in primitive variables (rho, U, T); the cell
+// average is used if rho or T would not be positive
 template <int D>
-__device__ __forceinline__ void face_state(const double *P, const double *gradP, int c, const double *r,
-                                           double *Ws)
+__device__ __forceinline__ void face_state(const double *P, const double *gradP, int c, const double *r, Prim &p)
 {
     constexpr int M = D + 2;
-    double pf[M];
+    double pf[M], av[M];
+#pragma unroll
     for (int m = 0; m < M; ++m) {
-        double s = P[(size_t)c * M + m];
+        double s = av[m] = P[(size_t)c * M + m];
+#pragma unroll
         for (int d = 0; d < D; ++d) s += gradP[((size_t)c * D + d) * M + m] * r[d];
         pf[m] = s;
     }
-    if (!(pf[0] > 0.0) || !(pf[D + 1] > 0.0))
-        for (int m = 0; m < M; ++m) pf[m] = P[(size_t)c * M + m];
-    double ke = 0.0;
-    Ws[0] = pf[0];
-    for (int d = 0; d < D; ++d) {
-        Ws[1 + d] = pf[0] * pf[1 + d];
-        ke += pf[1 + d] * pf[1 + d];
-    }
-    Ws[D + 1] = pf[0] * (0.5 * ke + 1.5 * pf[D + 1]);
+    const bool ok = pf[0] > 0.0 && pf[D + 1] > 0.0;
+#pragma unroll
+    for (int m = 0; m < M; ++m) pf[m] = ok ? pf[m] : av[m];
+    set_prim<D>(pf, p);
 }
 
 template <typename T, int D>
-__device__ __forceinline__ void side_record(const double *Ws, double nxi, T *rec)
+__device__ __forceinline__ void side_record(const Prim &p, double nxi, T *rec)
 {
-    Prim p = prim_of(Ws, D);
     for (int d = 0; d < 3; ++d) rec[GR_U + d] = (T)p.U[d];
     rec[GR_LAM] = (T)p.lam;
     rec[GR_PREF] = (T)pref_of(p.rho, p.lam, D);
-    rec[GR_NB] = (T)(nxi / (2.0 * p.lam));
+    rec[GR_NB] = (T)(nxi * p.T);
     rec[GR_NL2] = (T)(-p.lam * LOG2E);
 }
 
@@ -407,14 +435,14 @@ __device__ __forceinline__ void face_pre_body(const DevCase<T> &dc, const int bx
     const int typ = dc.ftype[f];
     if (typ == FT_WALL) return;
     const int L = dc.fL[f];
-    double WL[M], WR[M], rL[D], rR[D];
+    double rL[D], rR[D];
+    Prim pL, pR;
     for (int d = 0; d < D; ++d) rL[d] = dc.frL_d[(size_t)f * D + d];
-    face_state<D>(dc.prim, dc.gradprim, L, rL, WL);
+    face_state<D>(dc.prim, dc.gradprim, L, rL, pL);
     double *dW0 = dc.fdW0 + (size_t)f * D * M;
     double *q0 = dc.fq0 + (size_t)f * D;
     if (typ == FT_FARFIELD) {
-        const int g = dc.faux[f];
-        for (int m = 0; m < M; ++m) WR[m] = dc.Wg[(size_t)g * M + m];
+        set_prim<D>(dc.primg + (size_t)dc.faux[f] * M, pR);
         for (int d = 0; d < D; ++d) {
             for (int m = 0; m < M; ++m) dW0[d * M + m] = 0.5 * dc.gradW[((size_t)L * D + d) * M + m];
             q0[d] = 0.5 * dc.q[(size_t)L * D + d];
@@ -422,16 +450,15 @@ __device__ __forceinline__ void face_pre_body(const DevCase<T> &dc, const int bx
     } else {
         const int R = dc.fR[f];
         for (int d = 0; d < D; ++d) rR[d] = dc.frR_d[(size_t)f * D + d];
-        face_state<D>(dc.prim, dc.gradprim, R, rR, WR);
+        face_state<D>(dc.prim, dc.gradprim, R, rR, pR);
         for (int d = 0; d < D; ++d) {
             for (int m = 0; m < M; ++m)
                 dW0[d * M + m] = 0.5 * (dc.gradW[((size_t)L * D + d) * M + m] + dc.gradW[((size_t)R * D + d) * M + m]);
             q0[d] = 0.5 * (dc.q[(size_t)L * D + d] + dc.q[(size_t)R * D + d]);
         }
     }
-    side_record<T, D>(WL, dc.nxi, dc.fside + (size_t)f * 2 * GREC);
-    side_record<T, D>(WR, dc.nxi, dc.fside + (size_t)f * 2 * GREC + GREC);
-    Prim pL = prim_of(WL, D), pR = prim_of(WR, D);
+    side_record<T, D>(pL, dc.nxi, dc.fside + (size_t)f * 2 * GREC);
+    side_record<T, D>(pR, dc.nxi, dc.fside + (size_t)f * 2 * GREC + GREC);
     for (int d = 0; d < D; ++d) dc.fUref[(size_t)f * D + d] = 0.5 * (pL.U[d] + pR.U[d]);
     if (dc.w0_analytic) {
         // W0 from the analytic half-range moments (continuous velocity space),
@@ -753,14 +780,8 @@ __device__ __forceinline__ void face_fin1_body(const DevCase<T> &dc, const int b
     for (int d = 0; d < 3; ++d) r[FR_U + d] = (T)p.U[d];
     r[FR_LAM] = (T)p.lam;
     r[FR_PREF] = (T)pref_of(p.rho, p.lam, D);
-    const double kappa = 4.0 * (1.0 - dc.Pr) * p.lam * p.lam / (5.0 * p.rho);
-    for (int d = 0; d < 3; ++d) r[FR_KQ + d] = d < D ? (T)(kappa * dc.fq0[(size_t)f * D + d]) : T(0);
-    double *qs = dc.fqs + (size_t)f * 5;         // kept in FP64 for k_face_fin2
-    time_integrals(dc.dt, tau_of(dc, p.rho, p.T), qs);
-    for (int i = 0; i < 5; ++i) r[FR_QS + i] = (T)qs[i];
-    r[FR_NB] = (T)(dc.nxi / (2.0 * p.lam));
-    r[FR_XB] = (T)(dc.nxi * (dc.nxi + 2.0) / (4.0 * p.lam * p.lam));
     r[FR_NL2] = (T)(-p.lam * LOG2E);
+    time_integrals(dc.dt, dt_over_tau(dc, p.rho, p.T), dc.fqs + (size_t)f * 5);   // FP64, for k_face_fin2
 }
 
 template <typename T, int D, int NC>
@@ -1041,88 +1062,94 @@ __global__ void k_face_sum2_sep_batch(const DevCase<T> *__restrict__ cases, cons
     face_sum2_sep_body<T, D, NC>(dc, bx);
 }
 
-// M_c and T_c,d of k_face_sum2 from the 1-D moments m[d][0..5] (tensor grids)
+// the distinct moments R of k_face_sum2 from the 1-D moments m[d][0..5] of a
+// tensor grid: products over the axes
 template <int D>
-__device__ void sep_moments(const double m[D][6], double pref, double nb, double xb, double *S)
+__device__ __forceinline__ void sep_moments(const double (&m)[D][6], double pref, double *R)
 {
-    constexpr int NS = Sym<D>::N;
-    constexpr int M = D + 2;
-    auto Q = [&](const int *a) {
-        double r = pref;
-        for (int d = 0; d < D; ++d) r *= m[d][a[d]];
-        return r;
+    using Mo = Mono<D>;
+    auto Q = [&](int a, int b, int c) {
+        const double r = pref * m[0][a] * m[1][b];
+        return D == 3 ? r * m[D - 1][c] : r;
     };
-    for (int t = -1; t < D; ++t) {          // t = -1: M_c; t = d: T_c,d (extra factor c_d)
-        int base[3] = {0, 0, 0};
-        if (t >= 0) base[t] = 1;
-        int idx = 0;
-        for (int i = 0; i < M; ++i)
-            for (int j = i; j < M; ++j) {
-                double val;
-                int a[3] = {base[0], base[1], base[2]};
-                const bool iE = i == M - 1, jE = j == M - 1;
-                if (!iE && !jE) {
-                    if (i > 0) a[i - 1]++;
-                    if (j > 0) a[j - 1]++;
-                    val = Q(a);
-                } else if (!iE || !jE) {
-                    // psi_o (|c|^2 + xi^2)/2 with psi_o = 1 or c_(o-1)
-                    const int o = iE ? j : i;
-                    if (o > 0) a[o - 1]++;
-                    double s2 = 0.0;
-                    for (int e = 0; e < D; ++e) {
-                        int b[3] = {a[0], a[1], a[2]};
-                        b[e] += 2;
-                        s2 += Q(b);
-                    }
-                    val = 0.5 * (s2 + nb * Q(a));
-                } else {
-                    double s4 = 0.0, s2 = 0.0;
-                    for (int e = 0; e < D; ++e) {
-                        int b[3] = {a[0], a[1], a[2]};
-                        b[e] += 2;
-                        s2 += Q(b);
-                        for (int g = 0; g < D; ++g) {
-                            int c4[3] = {b[0], b[1], b[2]};
-                            c4[g] += 2;
-                            s4 += Q(c4);
-                        }
-                    }
-                    val = 0.25 * (s4 + 2.0 * nb * s2 + xb * Q(a));
-                }
-                S[NS * (t + 1) + idx] = val;
-                ++idx;
-            }
+    // |c|^2n times the monomial of exponents (a, b, c)
+    auto Q2 = [&](int a, int b, int c) {
+        const double s = Q(a + 2, b, c) + Q(a, b + 2, c);
+        return D == 3 ? s + Q(a, b, c + 2) : s;
+    };
+    auto Q4 = [&](int a, int b, int c) {
+        const double s = Q(a + 4, b, c) + Q(a, b + 4, c) + 2.0 * Q(a + 2, b + 2, c);
+        return D == 3 ? s + Q(a, b, c + 4) + 2.0 * (Q(a + 2, b, c + 2) + Q(a, b + 2, c + 2)) : s;
+    };
+    R[0] = Q(0, 0, 0);
+    R[Mo::OQ4] = Q4(0, 0, 0);
+#pragma unroll
+    for (int d = 0; d < D; ++d) {
+        const int x = d == 0, y = d == 1, z = d == 2;
+        R[Mo::O1 + d] = Q(x, y, z);
+        R[Mo::OQ4 + 1 + d] = Q4(x, y, z);
+#pragma unroll
+        for (int e = d; e < D; ++e) {
+            const int xe = x + (e == 0), ye = y + (e == 1), ze = z + (e == 2);
+            R[Mo::O2 + pair_index(D, d, e)] = Q(xe, ye, ze);
+            R[Mo::OQ2 + pair_index(D, d, e)] = Q2(xe, ye, ze);
+#pragma unroll
+            for (int g = e; g < D; ++g)
+                R[Mo::O3 + triple_index(D, d, e, g)] = Q(xe + (g == 0), ye + (g == 1), ze + (g == 2));
+        }
     }
 }
 
-// Cholesky solve of the SPD system A x = b (n <= 5), A overwritten
-__device__ void chol_solve(int n, double *A, double *b, int nrhs, int ldb)
+// A = L diag(d) L^T of a symmetric positive definite matrix (packed upper
+// triangle t(i, j), i <= j); inv[i] = 1 / d_i, L below the diagonal in place of
+// the entries.  Five divisions for the factor and none in the solves (the
+// Cholesky form took 5 square roots and 50 divisions for the four right-hand
+// sides, FP64 operations of about ten instructions each).
+template <int M> __device__ __forceinline__ constexpr int tri(int i, int j) { return i * M - i * (i - 1) / 2 + (j - i); }
+
+template <int M>
+__device__ __forceinline__ void ldl_factor(double *A, double (&inv)[M])
 {
-    for (int j = 0; j < n; ++j) {
-        double s = A[j * n + j];
-        for (int k = 0; k < j; ++k) s -= A[j * n + k] * A[j * n + k];
-        const double Ljj = sqrt(s);
-        A[j * n + j] = Ljj;
-        for (int i = j + 1; i < n; ++i) {
-            double t = A[i * n + j];
-            for (int k = 0; k < j; ++k) t -= A[i * n + k] * A[j * n + k];
-            A[i * n + j] = t / Ljj;
+#pragma unroll
+    for (int j = 0; j < M; ++j) {
+        double dj = A[tri<M>(j, j)];
+        double w[M];                             // L_jk d_k
+#pragma unroll
+        for (int k = 0; k < j; ++k) {
+            w[k] = A[tri<M>(k, j)];
+            const double l = w[k] * inv[k];
+            dj -= l * w[k];
+        }
+        inv[j] = 1.0 / dj;
+        // A(j, i) for i > j: subtract sum_k L_jk d_k L_ik, kept as L_ij d_j
+#pragma unroll
+        for (int i = j + 1; i < M; ++i) {
+            double t = A[tri<M>(j, i)];
+#pragma unroll
+            for (int k = 0; k < j; ++k) t -= w[k] * inv[k] * A[tri<M>(k, i)];
+            A[tri<M>(j, i)] = t;
         }
     }
-    for (int r = 0; r < nrhs; ++r) {
-        double *x = b + r * ldb;
-        for (int i = 0; i < n; ++i) {
-            double t = x[i];
-            for (int k = 0; k < i; ++k) t -= A[i * n + k] * x[k];
-            x[i] = t / A[i * n + i];
-        }
-        for (int i = n - 1; i >= 0; --i) {
-            double t = x[i];
-            for (int k = i + 1; k < n; ++k) t -= A[k * n + i] * x[k];
-            x[i] = t / A[i * n + i];
-        }
-    }
+    // entries (j, i) hold L_ij d_j: scale to L_ij
+#pragma unroll
+    for (int j = 0; j < M; ++j)
+#pragma unroll
+        for (int i = j + 1; i < M; ++i) A[tri<M>(j, i)] *= inv[j];
+}
+
+template <int M>
+__device__ __forceinline__ void ldl_solve(const double *A, const double (&inv)[M], double *x)
+{
+#pragma unroll
+    for (int i = 1; i < M; ++i)
+#pragma unroll
+        for (int k = 0; k < i; ++k) x[i] -= A[tri<M>(k, i)] * x[k];
+#pragma unroll
+    for (int i = 0; i < M; ++i) x[i] *= inv[i];
+#pragma unroll
+    for (int i = M - 2; i >= 0; --i)
+#pragma unroll
+        for (int k = i + 1; k < M; ++k) x[i] -= A[tri<M>(i, k)] * x[k];
 }
 
 // slopes of g0 in the centred basis: M0 = L Mc L^T, sum_k w u_d psi psi^T g0 =
@@ -1135,85 +1162,69 @@ __device__ __forceinline__ void face_fin2_body(const DevCase<T> &dc, const int b
     const int f = bx * blockDim.x + threadIdx.x;
     constexpr int M = D + 2, NS = Sym<D>::N, S2 = NS * (D + 1);
     if (f >= dc.F || dc.ftype[f] == FT_WALL) return;
-    double Ssep[S2];
-    const double *S = dc.fsum2 + (size_t)f * S2;
+    const double *pp = dc.fprim0 + (size_t)f * M;
+    const double rho0 = pp[0], lam0 = pp[D + 1], i2l = 0.5 / lam0;
+    const double nb = dc.nxi * i2l, xb = dc.nxi * (dc.nxi + 2.0) * i2l * i2l, pref = pref_of(rho0, lam0, D);
+    double R[Mono<D>::N], S[S2];
+    const double *sum2 = dc.fsum2 + (size_t)f * S2;
     if (dc.sep) {
         double m1[D][6];
+#pragma unroll
         for (int d = 0; d < D; ++d)
-            for (int pw = 0; pw < 6; ++pw) m1[d][pw] = S[d * 6 + pw];
-        const double *pq = dc.fprim0 + (size_t)f * M;
-        const double lam0 = pq[D + 1];
-        sep_moments<D>(m1, pref_of(pq[0], lam0, D), dc.nxi / (2.0 * lam0),
-                       dc.nxi * (dc.nxi + 2.0) / (4.0 * lam0 * lam0), Ssep);
-        S = Ssep;
+#pragma unroll
+            for (int pw = 0; pw < 6; ++pw) m1[d][pw] = sum2[d * 6 + pw];
+        sep_moments<D>(m1, pref, R);
     } else {
-        const double lam0 = dc.fprim0[(size_t)f * M + D + 1];
-        mono_moments<D>(S, dc.nxi / (2.0 * lam0), dc.nxi * (dc.nxi + 2.0) / (4.0 * lam0 * lam0), Ssep);
-        S = Ssep;
+#pragma unroll
+        for (int i = 0; i < Mono<D>::N; ++i) R[i] = sum2[i];
     }
-    double Mc[M * M], Tc[D][M * M];
-    {
-        int t = 0;
-        for (int i = 0; i < M; ++i)
-            for (int j = i; j < M; ++j) {
-                Mc[i * M + j] = Mc[j * M + i] = S[t];
-                for (int d = 0; d < D; ++d) Tc[d][i * M + j] = Tc[d][j * M + i] = S[NS * (1 + d) + t];
-                ++t;
-            }
-    }
-    const double *pp = dc.fprim0 + (size_t)f * M;
+    mono_moments<D>(R, nb, xb, S);
     double U0[D], uu = 0.0;
+#pragma unroll
     for (int d = 0; d < D; ++d) {
         U0[d] = pp[1 + d];
         uu += U0[d] * U0[d];
     }
-    // right-hand sides L^{-1} dW0_d
-    double B[(D + 1) * M];
+    // right-hand sides L^{-1} dW0_d, then B[d] = beta_d, B[D] = beta_A
+    double B[(D + 1) * M], inv[M], xa[M];
     const double *dW = dc.fdW0 + (size_t)f * D * M;
+    ldl_factor<M>(S, inv);                  // the first NS entries: Mc
+#pragma unroll
     for (int d = 0; d < D; ++d) {
         const double *g = dW + d * M;
         double *x = B + d * M;
         x[0] = g[0];
         double um = 0.0;
+#pragma unroll
         for (int e = 0; e < D; ++e) {
             x[1 + e] = g[1 + e] - U0[e] * g[0];
             um += U0[e] * g[1 + e];
         }
         x[D + 1] = g[D + 1] - um + 0.5 * uu * g[0];
+        ldl_solve<M>(S, inv, x);
     }
-    double A[M * M];
-    for (int i = 0; i < M * M; ++i) A[i] = Mc[i];
-    chol_solve(M, A, B, D, M);              // B[d] = beta_d ; A holds the factor
-    double *xa = B + D * M;
+#pragma unroll
     for (int i = 0; i < M; ++i) {
         double s = 0.0;
+#pragma unroll
         for (int d = 0; d < D; ++d)
-            for (int j = 0; j < M; ++j) s += Tc[d][i * M + j] * B[d * M + j];
+#pragma unroll
+            for (int j = 0; j < M; ++j) s += S[NS * (1 + d) + (i <= j ? tri<M>(i, j) : tri<M>(j, i))] * B[d * M + j];
         xa[i] = -s;
     }
-    // solve with the stored factor
+    ldl_solve<M>(S, inv, xa);
+#pragma unroll
     for (int i = 0; i < M; ++i) {
-        double t = xa[i];
-        for (int k = 0; k < i; ++k) t -= A[i * M + k] * xa[k];
-        xa[i] = t / A[i * M + i];
-    }
-    for (int i = M - 1; i >= 0; --i) {
-        double t = xa[i];
-        for (int k = i + 1; k < M; ++k) t -= A[k * M + i] * xa[k];
-        xa[i] = t / A[i * M + i];
-    }
-    for (int i = 0; i < M; ++i)
+#pragma unroll
         for (int d = 0; d < D; ++d) xa[i] -= U0[d] * B[d * M + i];
-    T *r = dc.frec + (size_t)f * FREC;
-    for (int i = 0; i < (D + 1) * M; ++i) r[FR_BETA + i] = (T)B[i];
+        B[D * M + i] = xa[i];
+    }
 
     // Expand the equilibrium part of the interface distribution,
     // q3 (g0 + g0+) + q4 u.grad g0 + q5 dg0/dt, into H0(c) P_m(c), c = u - U0:
     //   h: sh = 1 + (kq.c)(2 lam |c|^2 - D - 2), slope terms of int (beta.psi_c) g0 dxi
     //   b: sh = nb [1 + (kq.c)(2 lam |c|^2 - D)], slope terms of int xi^2 (beta.psi_c) g0 dxi
     // with u_d = c_d + U0_d.
-    const double rho0 = pp[0], lam0 = pp[D + 1];
-    const double nb = dc.nxi / (2.0 * lam0), xb = dc.nxi * (dc.nxi + 2.0) / (4.0 * lam0 * lam0);
     const double kappa = 4.0 * (1.0 - dc.Pr) * lam0 * lam0 / (5.0 * rho0);
     double kq[D];
     for (int d = 0; d < D; ++d) kq[d] = kappa * dc.fq0[(size_t)f * D + d];
@@ -1224,25 +1235,30 @@ __device__ __forceinline__ void face_fin2_body(const DevCase<T> &dc, const int b
     x[X::EX] = (T)(std::is_same<T, float>::value ? -lam0 * LOG2E : -lam0);
     x[X::Q1] = (T)qs[0];
     x[X::Q2] = (T)qs[1];
-    x[X::PREF] = (T)pref_of(rho0, lam0, D);
+    x[X::PREF] = (T)pref;
     constexpr int NB = Poly<D>::NB, NP = Poly<D>::N;
+#pragma unroll
     for (int m = 0; m < NC; ++m) {
         const double sm = m == 0 ? 1.0 : nb;            // scale of the b moments
         const double xm = m == 0 ? nb : xb;             // xi^2 (resp. xi^4) factor of beta_E / 2
         const double sh0 = m == 0 ? 1.0 : nb;
         const double shl = m == 0 ? -(double)(D + 2) : -(double)D;
         double a0 = qs[2] * sh0, a[D], Bq[D][D], gam[D];
+#pragma unroll
         for (int e = 0; e < D; ++e) {
             a[e] = qs[2] * sh0 * shl * kq[e];
             gam[e] = qs[2] * sh0 * 2.0 * lam0 * kq[e];
+#pragma unroll
             for (int g = 0; g < D; ++g) Bq[e][g] = 0.0;
         }
         double diag = 0.0;
+#pragma unroll
         for (int d = 0; d < D; ++d) {
             const double *bd = B + d * M;                // beta^(d) in the psi_c basis
             const double alpha = sm * bd[0] + 0.5 * bd[D + 1] * xm;
             a0 += qs[3] * U0[d] * alpha;
             a[d] += qs[3] * alpha;
+#pragma unroll
             for (int e = 0; e < D; ++e) {
                 a[e] += qs[3] * U0[d] * sm * bd[1 + e];
                 Bq[d][e] += qs[3] * sm * bd[1 + e];
@@ -1252,15 +1268,20 @@ __device__ __forceinline__ void face_fin2_body(const DevCase<T> &dc, const int b
         }
         const double alphaA = sm * xa[0] + 0.5 * xa[D + 1] * xm;
         a0 += qs[4] * alphaA;
+#pragma unroll
         for (int e = 0; e < D; ++e) a[e] += qs[4] * sm * xa[1 + e];
         diag += qs[4] * 0.5 * sm * xa[D + 1];
         T *pm = x + X::POLY + m * NP;
         pm[0] = (T)a0;
+#pragma unroll
         for (int e = 0; e < D; ++e) pm[1 + e] = (T)a[e];
         int t = 1 + D;
+#pragma unroll
         for (int e = 0; e < D; ++e)
+#pragma unroll
             for (int g = e; g < D; ++g)
                 pm[t++] = (T)(e == g ? Bq[e][e] + diag : Bq[e][g] + Bq[g][e]);
+#pragma unroll
         for (int e = 0; e < D; ++e) pm[1 + D + NB + e] = (T)gam[e];
     }
 }
@@ -1388,24 +1409,31 @@ __device__ __forceinline__ void wall_sum_body(const DevCase<T> &dc, const int bx
             }
         }
     }
+    // the warps' sums by recursive halving (16 FP64 additions per warp instead of
+    // 5 NR), then one thread per value adds the warps
+    double t[16];
 #pragma unroll
-    for (int i = 0; i < NR; ++i) {
-        const double t = warp_sum(v[i].value());
-        if (lane == 0) red[i][warp] = t;
+    for (int i = 0; i < 16; ++i) t[i] = i < NR ? v[i < NR ? i : 0].value() : 0.0;
+    const double ts = warp_transpose_sum<double, 16>(t);
+    if ((lane & 1) == 0 && (lane >> 1) < NR) red[lane >> 1][warp] = ts;
+    __syncthreads();
+    if (threadIdx.x < NR) {
+        double a = 0.0;
+        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) a += red[threadIdx.x][w];
+        red[threadIdx.x][0] = a;
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        double a[NR];
-        for (int i = 0; i < NR; ++i) {
-            a[i] = 0.0;
-            for (int w = 0; w < (int)(blockDim.x >> 5); ++w) a[i] += red[i][w];
+    if (threadIdx.x <= M) {
+        const double rw = -red[0][0] / red[1][0];
+        const int m = threadIdx.x - 1;
+        if (m >= 0) {
+            dc.wall_F[(size_t)s * M + m] = red[2 + m][0] + rw * red[2 + M + m][0];
+        } else {
+            dc.rho_w[s] = rw;
+            T *w = dc.wrec + (size_t)s * GREC;
+            for (int i = 0; i < GREC; ++i) w[i] = wr[i];
+            w[GR_PREF] = (T)pref_of(rw, lw, D);
         }
-        const double rw = -a[0] / a[1];
-        dc.rho_w[s] = rw;
-        T *w = dc.wrec + (size_t)s * GREC;
-        for (int i = 0; i < GREC; ++i) w[i] = wr[i];
-        w[GR_PREF] = (T)pref_of(rw, lw, D);
-        for (int m = 0; m < M; ++m) dc.wall_F[(size_t)s * M + m] = a[2 + m] + rw * a[2 + M + m];
     }
 }
 
@@ -1809,7 +1837,6 @@ template <typename T, int D, int NC>
 __device__ __forceinline__ void update_W_body(const DevCase<T> &dc, const int bx)
 {
     constexpr int M = D + 2;
-    __shared__ double red[2 * M][8];
     const int c = bx * blockDim.x + threadIdx.x;
     double dsq[M], wsq[M];
     for (int m = 0; m < M; ++m) dsq[m] = wsq[m] = 0.0;
@@ -1827,33 +1854,16 @@ __device__ __forceinline__ void update_W_body(const DevCase<T> &dc, const int bx
         }
         Prim p = prim_of(Wc, D);
         if (!(p.rho > 0.0) || !(p.T > 0.0) || !isfinite(p.rho) || !isfinite(p.T)) atomicOr(dc.flags, 1);
-        const double tau = tau_of(dc, p.rho, p.T);
-        const double kappa = 4.0 * (1.0 - dc.Pr) * p.lam * p.lam / (5.0 * p.rho);
-        T *r = dc.krec + (size_t)c * CREC;
-        for (int d = 0; d < 3; ++d) r[CR_U + d] = (T)p.U[d];
-        r[CR_LAM] = (T)p.lam;
-        r[CR_PREF] = (T)pref_of(p.rho, p.lam, D);
-        for (int d = 0; d < 3; ++d) r[CR_KQ + d] = d < D ? (T)(kappa * dc.q[(size_t)c * D + d]) : T(0);
-        const double cc = 0.5 * dc.dt / tau;
-        r[CR_C] = (T)cc;
-        r[CR_INV] = (T)(1.0 / (1.0 + cc));
-        r[CR_NB] = (T)(dc.nxi / (2.0 * p.lam));
-        r[CR_NL2] = (T)(-p.lam * LOG2E);
+        cell_record<T, D>(dc, p, dc.q + (size_t)c * D, dc.krec + (size_t)c * CREC);
     }
-    // deterministic block partials of the residual
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    // residual partials of the warp's 32 cells, whatever the block size
+    const int w = c >> 5;
     for (int m = 0; m < M; ++m) {
-        double a = warp_sum(dsq[m]), b = warp_sum(wsq[m]);
-        if (lane == 0) {
-            red[m][warp] = a;
-            red[M + m][warp] = b;
+        const double a = warp_sum(dsq[m]), b = warp_sum(wsq[m]);
+        if ((threadIdx.x & 31) == 0 && c < dc.C) {
+            dc.res_part[(size_t)w * 2 * M + m] = a;
+            dc.res_part[(size_t)w * 2 * M + M + m] = b;
         }
-    }
-    __syncthreads();
-    if (threadIdx.x < 2 * M) {
-        double s = 0.0;
-        for (int w = 0; w < 8; ++w) s += red[threadIdx.x][w];
-        dc.res_part[(size_t)bx * 2 * M + threadIdx.x] = s;
     }
 }
 
@@ -1871,20 +1881,23 @@ __global__ void __launch_bounds__(256) k_update_W_batch(const DevCase<T> *__rest
     update_W_body<T, D, NC>(dc, bx);
 }
 
+// one block of RES_THREADS threads: lane sums of the partials, then the lanes in order
+constexpr int RES_THREADS = 512;
 template <int M>
-__global__ void k_residual(const double *res_part, int nblocks, double *res)
+__global__ void __launch_bounds__(RES_THREADS) k_residual(const double *res_part, int nparts, double *res)
 {
-    __shared__ double acc[2 * M][32];
+    __shared__ double acc[2 * M][RES_THREADS / 32];
     const int t = threadIdx.x;
     for (int i = 0; i < 2 * M; ++i) {
         double s = 0.0;
-        for (int b = t; b < nblocks; b += 32) s += res_part[(size_t)b * 2 * M + i];
-        acc[i][t] = s;
+        for (int b = t; b < nparts; b += RES_THREADS) s += res_part[(size_t)b * 2 * M + i];
+        s = warp_sum(s);
+        if ((t & 31) == 0) acc[i][t >> 5] = s;
     }
-    __syncwarp();
+    __syncthreads();
     if (t < M) {
         double a = 0.0, b = 0.0;
-        for (int w = 0; w < 32; ++w) {
+        for (int w = 0; w < RES_THREADS / 32; ++w) {
             a += acc[t][w];
             b += acc[M + t][w];
         }
@@ -2285,31 +2298,65 @@ cudaError_t launch_gather(const DevCase<T> &dc, cudaStream_t st)
     return cudaSuccess;
 }
 
-// Blocks, threads and dynamic shared memory of the per-case kernels of a step
-// (SmallKernel order); 0 blocks: the case does not run that kernel.
-template <typename T, int D>
-static int sk_blocks(const DevCase<T> &dc, int k)
+// Work items, threads per block, blocks and dynamic shared memory of the per-case
+// kernels of a step (SmallKernel order); 0 items: the case does not run that
+// kernel.  The kernels with a thread per cell or face are chains of FP64
+// operations, which an SM retires at one warp instruction in 20 cycles: on small
+// meshes one-warp blocks spread them over all SMs (20 x 20 cells, 840 faces:
+// k_update_W 24 -> 12.5 us, k_macro_grad 27 -> 12.6, k_face_fin1 28 -> 8.7,
+// k_face_fin2 29 -> 16, with the operations saved in them).
+constexpr int kSpread = 152 * 128;           // up to here one-warp blocks do not fill the chip
+
+template <typename T>
+static int sk_items(const DevCase<T> &dc, int k)
 {
     const int C = dc.C, F = dc.F;
-    const bool faces = F > 0, sums1 = faces && !dc.w0_analytic;
+    const bool sums1 = !dc.w0_analytic;
     switch (k) {
-    case SK_PREP: return cdiv(C + dc.G, 128);
-    case SK_MACRO_GRAD: return cdiv(C, 128);
-    case SK_FACE_PRE: return faces ? cdiv(F, 128) : 0;
-    case SK_FACE_SUM1_SEP: return sums1 && dc.sep1 ? cdiv(F, SUM1_SEP_WARPS) : 0;
-    case SK_FACE_SUM1: return sums1 && !dc.sep1 ? cdiv(F, 8) : 0;
-    case SK_FACE_FIN1: return faces ? cdiv(F, 128) : 0;
-    case SK_FACE_SUM2_SEP: return faces && dc.sep ? cdiv(F, 8) : 0;
-    case SK_FACE_SUM2: return faces && !dc.sep ? cdiv(F, 8) : 0;
-    case SK_FACE_FIN2: return faces ? cdiv(F, 64) : 0;
+    case SK_PREP: return C + dc.G;
+    case SK_FACE_SUM1_SEP: return sums1 && dc.sep1 ? F : 0;
+    case SK_FACE_SUM1: return sums1 && !dc.sep1 ? F : 0;
+    case SK_FACE_SUM2_SEP: return dc.sep ? F : 0;
+    case SK_FACE_SUM2: return !dc.sep ? F : 0;
+    case SK_FACE_PRE:
+    case SK_FACE_FIN1:
+    case SK_FACE_FIN2: return F;
     case SK_WALL_SUM: return dc.NW;
-    case SK_UPDATE_W: return cdiv(C, 256);
-    case SK_COLLIDE: return cdiv(C, 8);
+    case SK_MACRO_GRAD:
+    case SK_UPDATE_W:
+    case SK_COLLIDE: return C;
     default: return 0;
     }
 }
 
-constexpr int kSkThreads[SK_COUNT] = {128, 128, 128, 32 * SUM1_SEP_WARPS, 256, 128, 256, 256, 64, 256, 256, 256};
+static int sk_threads(int k, long long items)
+{
+    switch (k) {
+    case SK_FACE_SUM1_SEP: return 32 * SUM1_SEP_WARPS;
+    case SK_FACE_SUM1:
+    case SK_FACE_SUM2_SEP:
+    case SK_FACE_SUM2:
+    case SK_WALL_SUM:
+    case SK_COLLIDE: return 256;
+    case SK_FACE_FIN2: return items <= kSpread ? 32 : 64;
+    default: return items <= kSpread ? 32 : 128;
+    }
+}
+
+// items per block: a warp each in the sums and the collision pass, a block each
+// in the wall pass, a thread each in the others
+static int sk_blocks(int k, int items, int threads)
+{
+    switch (k) {
+    case SK_WALL_SUM: return items;
+    case SK_FACE_SUM1_SEP:
+    case SK_FACE_SUM1:
+    case SK_FACE_SUM2_SEP:
+    case SK_FACE_SUM2:
+    case SK_COLLIDE: return cdiv(items, threads / 32);
+    default: return cdiv(items, threads);
+    }
+}
 
 template <typename T, int D>
 static size_t sk_smem(const DevCase<T> &dc, int k)
@@ -2321,11 +2368,10 @@ static size_t sk_smem(const DevCase<T> &dc, int k)
 // one per-case kernel, for one case (cases == nullptr) or for the cases of a
 // batch (block offsets off[0..n])
 template <typename T, int D, int NC>
-static cudaError_t sk_launch(int k, int blocks, size_t smem, cudaStream_t st, const DevCase<T> *dc,
+static cudaError_t sk_launch(int k, int blocks, int nt, size_t smem, cudaStream_t st, const DevCase<T> *dc,
                              const DevCase<T> *cases, const int *off, int n)
 {
     if (blocks <= 0) return cudaSuccess;
-    const int nt = kSkThreads[k];
 #define UGKS_SK(ID, K)                                                                                  \
     case ID:                                                                                            \
         if (cases) K##_batch<T, D, NC><<<blocks, nt, smem, st>>>(cases, off, n);                        \
@@ -2360,7 +2406,8 @@ static cudaError_t sk_launch(int k, int blocks, size_t smem, cudaStream_t st, co
 template <typename T, int D, int NC>
 static void sk_case(const DevCase<T> &dc, int k, cudaStream_t st)
 {
-    sk_launch<T, D, NC>(k, sk_blocks<T, D>(dc, k), sk_smem<T, D>(dc, k), st, &dc, nullptr, nullptr, 0);
+    const int items = sk_items(dc, k), nt = sk_threads(k, items);
+    sk_launch<T, D, NC>(k, sk_blocks(k, items, nt), nt, sk_smem<T, D>(dc, k), st, &dc, nullptr, nullptr, 0);
 }
 
 template <typename T, int D, int NC>
@@ -2411,10 +2458,14 @@ cudaError_t launch_pre_gather(const DevCase<T> &dc, cudaStream_t st)
 }
 
 template <typename T>
-int small_kernel_blocks(const DevCase<T> &dc, int k)
+int small_kernel_items(const DevCase<T> &dc, int k)
 {
-    return dc.D == 2 ? sk_blocks<T, 2>(dc, k) : sk_blocks<T, 3>(dc, k);
+    return sk_items(dc, k);
 }
+
+int small_kernel_threads(int k, long long items) { return sk_threads(k, items); }
+
+int small_kernel_blocks(int k, int items, int threads) { return sk_blocks(k, items, threads); }
 
 template <typename T>
 size_t small_kernel_smem(const DevCase<T> &dc, int k)
@@ -2423,11 +2474,11 @@ size_t small_kernel_smem(const DevCase<T> &dc, int k)
 }
 
 template <typename T>
-cudaError_t launch_small_batch(int D, int k, const DevCase<T> *cases, const int *off, int n, int blocks, size_t smem,
-                               cudaStream_t st)
+cudaError_t launch_small_batch(int D, int k, const DevCase<T> *cases, const int *off, int n, int blocks, int threads,
+                               size_t smem, cudaStream_t st)
 {
-    if (D == 2) return sk_launch<T, 2, 2>(k, blocks, smem, st, nullptr, cases, off, n);
-    return sk_launch<T, 3, 1>(k, blocks, smem, st, nullptr, cases, off, n);
+    if (D == 2) return sk_launch<T, 2, 2>(k, blocks, threads, smem, st, nullptr, cases, off, n);
+    return sk_launch<T, 3, 1>(k, blocks, threads, smem, st, nullptr, cases, off, n);
 }
 
 template <typename T>
@@ -2497,10 +2548,10 @@ template cudaError_t launch_halo<double>(const DevCase<double> &, const int *, i
 template cudaError_t launch_halo<float>(const DevCase<float> &, const int *, int, size_t, void *, int,
                                         cudaStream_t);
 
-cudaError_t launch_residual(const double *res_part, int nblocks, int D, double *res, cudaStream_t st)
+cudaError_t launch_residual(const double *res_part, int nparts, int D, double *res, cudaStream_t st)
 {
-    if (D == 2) k_residual<4><<<1, 32, 0, st>>>(res_part, nblocks, res);
-    else k_residual<5><<<1, 32, 0, st>>>(res_part, nblocks, res);
+    if (D == 2) k_residual<4><<<1, RES_THREADS, 0, st>>>(res_part, nparts, res);
+    else k_residual<5><<<1, RES_THREADS, 0, st>>>(res_part, nparts, res);
     return cudaGetLastError();
 }
 
@@ -2541,13 +2592,13 @@ cudaError_t launch_density_range(const double *W, int C, int M, const unsigned c
 
 template cudaError_t launch_pre_gather<double>(const DevCase<double> &, cudaStream_t);
 template cudaError_t launch_pre_gather<float>(const DevCase<float> &, cudaStream_t);
-template int small_kernel_blocks<double>(const DevCase<double> &, int);
-template int small_kernel_blocks<float>(const DevCase<float> &, int);
+template int small_kernel_items<double>(const DevCase<double> &, int);
+template int small_kernel_items<float>(const DevCase<float> &, int);
 template size_t small_kernel_smem<double>(const DevCase<double> &, int);
 template size_t small_kernel_smem<float>(const DevCase<float> &, int);
-template cudaError_t launch_small_batch<double>(int, int, const DevCase<double> *, const int *, int, int, size_t,
-                                                cudaStream_t);
-template cudaError_t launch_small_batch<float>(int, int, const DevCase<float> *, const int *, int, int, size_t,
+template cudaError_t launch_small_batch<double>(int, int, const DevCase<double> *, const int *, int, int, int,
+                                                size_t, cudaStream_t);
+template cudaError_t launch_small_batch<float>(int, int, const DevCase<float> *, const int *, int, int, int, size_t,
                                                cudaStream_t);
 #define UGKS_GATHER(T)                                                                                        \
     template cudaError_t launch_flux<T>(int, int, int, int, int, int, cudaStream_t, const DevCase<T> *,       \

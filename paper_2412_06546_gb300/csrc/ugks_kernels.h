@@ -33,14 +33,17 @@ enum SmallKernel {
     SK_PREP, SK_MACRO_GRAD, SK_FACE_PRE, SK_FACE_SUM1_SEP, SK_FACE_SUM1, SK_FACE_FIN1,
     SK_FACE_SUM2_SEP, SK_FACE_SUM2, SK_FACE_FIN2, SK_WALL_SUM, SK_UPDATE_W, SK_COLLIDE, SK_COUNT
 };
-// blocks (0: not run) and dynamic shared memory of kernel k for a case (a host copy of its DevCase)
-template <typename T> int small_kernel_blocks(const DevCase<T> &dc, int k);
+// work items (0: not run) and dynamic shared memory of kernel k for a case (a host
+// copy of its DevCase), threads per block for a number of items, and blocks
+template <typename T> int small_kernel_items(const DevCase<T> &dc, int k);
+int small_kernel_threads(int k, long long items);
+int small_kernel_blocks(int k, int items, int threads);
 template <typename T> size_t small_kernel_smem(const DevCase<T> &dc, int k);
 // kernel k over n cases in one launch: cases[] a device array of their DevCase,
 // off[0..n] the device prefix sums of their block counts, blocks = off[n]
 template <typename T>
-cudaError_t launch_small_batch(int D, int k, const DevCase<T> *cases, const int *off, int n, int blocks, size_t smem,
-                               cudaStream_t st);
+cudaError_t launch_small_batch(int D, int k, const DevCase<T> *cases, const int *off, int n, int blocks, int threads,
+                               size_t smem, cudaStream_t st);
 template <typename T> cudaError_t launch_heatflux(const DevCase<T> &dc, cudaStream_t st);
 // state I/O between the internal layout and a host-layout staging buffer of
 // element type S (double or float)
@@ -48,7 +51,7 @@ template <typename T, typename S>
 cudaError_t launch_f_export(const DevCase<T> &dc, const long long *perm, int c0, int nc, S *out, cudaStream_t st);
 template <typename T, typename S>
 cudaError_t launch_f_import(const DevCase<T> &dc, const long long *perm, int c0, int nc, const S *in, cudaStream_t st);
-cudaError_t launch_residual(const double *res_part, int nblocks, int D, double *res, cudaStream_t st);
+cudaError_t launch_residual(const double *res_part, int nparts, int D, double *res, cudaStream_t st);
 // halo rows of the listed internal cells to (unpack = 0) or from (1) a device buffer of n rows of `row` bytes
 template <typename T>
 cudaError_t launch_halo(const DevCase<T> &dc, const int *cells, int n, size_t row, void *buf, int unpack,
