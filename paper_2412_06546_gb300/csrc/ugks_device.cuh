@@ -524,6 +524,11 @@ __device__ __forceinline__ P pnormal(const P (&u)[D], const T *n, T one)
 // exp(-lam c2) from the record's coefficient (-lam; -lam log2 e in FP32)
 __device__ __forceinline__ float gauss_ex(float ex, float c2) { return ex2_approx(__fmul_rn(ex, c2)); }
 __device__ __forceinline__ double gauss_ex(double ex, double c2) { return exp(ex * c2); }
+__device__ __forceinline__ float2 gauss_ex(float ex, float2 c2)
+{
+    const float2 t = pmul(c2, make_float2(ex, ex));
+    return make_float2(ex2_approx(t.x), ex2_approx(t.y));
+}
 
 // Sign tests and running extrema.  A double compare costs as much as an FP64
 // multiply (an SM retires 1.6 of either per cycle), so FP64 values are compared
@@ -537,6 +542,10 @@ __device__ __forceinline__ bool lt0(double x)
     const long long b = __double_as_longlong(x);
     return b < 0 && b != (long long)0x8000000000000000ull;
 }
+
+// min(x, 0)
+__device__ __forceinline__ float min0(float x) { return fminf(x, 0.f); }
+__device__ __forceinline__ double min0(double x) { return lt0(x) ? x : 0.0; }
 
 template <typename T> struct Extrema;
 template <> struct Extrema<float> {
@@ -636,6 +645,143 @@ __device__ __forceinline__ void entry_range(const DevCase<T> &dc, int c, int &e0
     }
 }
 
+// The entries of cell c and the rows of f they read (TV velocities of the lane,
+// fl = f_cur + its first one), from global memory.
+template <typename T, int D, int NC, int TV> struct GlobalCell {
+    using P = typename Pk<T, TV>::P;
+    static constexpr int NP = Pk<T, TV>::NP;
+    const DevCase<T> &dc;
+    const T *fl;
+    int c, e0;
+    __device__ __forceinline__ int4 ids(int e) const { return __ldg(dc.gi + e0 + e); }
+    __device__ __forceinline__ void values(int e, int at, T (&v)[4]) const
+    {
+        load_rec<4>(dc.gf + (size_t)(e0 + e) * GEnt<D>::LEN + at, v);
+    }
+    __device__ __forceinline__ void row_of(int cell, P (&x)[NC][NP]) const
+    {
+#pragma unroll
+        for (int m = 0; m < NC; ++m) ldp<T, TV>(fl + ((size_t)cell * NC + m) * dc.nvp, x[m]);
+    }
+    __device__ __forceinline__ void own(P (&x)[NC][NP]) const { row_of(c, x); }
+    __device__ __forceinline__ void row(int, const int4 &gi, P (&x)[NC][NP]) const { row_of(gi.x, x); }
+    __device__ __forceinline__ void record(int, int face, T (&x)[XRec<D>::LEN]) const
+    {
+        load_rec<XRec<D>::LEN>(dc.xrec + (size_t)face * XRec<D>::LEN, x);
+    }
+};
+
+// asynchronous copies of N bytes (4, 8 or 16) from global into shared memory
+template <int N> __device__ __forceinline__ void cp_async(void *smem, const void *global)
+{
+    const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(s), "l"(global), "n"(N) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N> __device__ __forceinline__ void cp_async_wait()
+{
+    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
+// B bytes of a lane (4 to 32) in chunks of at most 16
+template <int B> __device__ __forceinline__ void cp_async_lane(void *smem, const void *global)
+{
+    constexpr int CB = B < 16 ? B : 16;
+#pragma unroll
+    for (int q = 0; q < B / CB; ++q)
+        cp_async<CB>(static_cast<char *>(smem) + q * CB, static_cast<const char *>(global) + q * CB);
+}
+
+// TV values of a lane from shared memory into packs
+template <typename T, int TV>
+__device__ __forceinline__ void lds_pack(const unsigned char *p, typename Pk<T, TV>::P (&x)[Pk<T, TV>::NP])
+{
+    constexpr int CH = vec_chunk<T, TV>();
+    using V = typename VecOf<T, CH>::type;
+    T v[TV];
+#pragma unroll
+    for (int q = 0; q < TV / CH; ++q) {
+        const V w = reinterpret_cast<const V *>(p)[q];
+        const T *t = reinterpret_cast<const T *>(&w);
+#pragma unroll
+        for (int j = 0; j < CH; ++j) v[q * CH + j] = t[j];
+    }
+#pragma unroll
+    for (int j = 0; j < TV; ++j) pel<Pk<T, TV>::W>(x, j) = v[j];
+}
+
+// The same of a cell with NF entries, staged in the warp's shared memory by
+// asynchronous copies: its entries, the flux records of its faces and, per lane,
+// its TV velocities of the cell's and the neighbours' rows (a lane reads back
+// what it copied itself).
+template <typename T, int D, int NC, int TV, int NF> struct StagedCell {
+    using K = Pk<T, TV>;
+    using P = typename K::P;
+    using E = GEnt<D>;
+    using X = XRec<D>;
+    static constexpr int NP = K::NP;
+    static constexpr int ROW = 32 * TV * (int)sizeof(T);
+    static constexpr int GI = (NF + 1) * NC * ROW, GF = GI + NF * 16, XR = GF + NF * E::LEN * (int)sizeof(T);
+    static constexpr int BYTES = XR + NF * X::LEN * (int)sizeof(T);        // a multiple of 16
+    static_assert(BYTES % 16 == 0, "stages are 16-byte aligned");
+    unsigned char *s;
+    int lane;
+    // request cell c, whose entry ids lane e < NF holds in id
+    __device__ __forceinline__ void request(const DevCase<T> &dc, const T *fl, int c, const int4 &id) const
+    {
+        constexpr int B = TV * (int)sizeof(T);
+#pragma unroll
+        for (int e = 0; e <= NF; ++e) {
+            const int r = e < NF ? __shfl_sync(0xffffffffu, id.x, e < NF ? e : 0) : c;
+#pragma unroll
+            for (int m = 0; m < NC; ++m)
+                cp_async_lane<B>(s + (e * NC + m) * ROW + lane * B, fl + ((size_t)r * NC + m) * dc.nvp);
+        }
+        if (lane < NF) *reinterpret_cast<int4 *>(s + GI + lane * 16) = id;
+        constexpr int NG = NF * E::LEN * (int)sizeof(T) / 16;
+        const char *gf = reinterpret_cast<const char *>(dc.gf + (size_t)c * NF * E::LEN);
+#pragma unroll
+        for (int q = 0; q < (NG + 31) / 32; ++q)
+            if (q * 32 + lane < NG) cp_async<16>(s + GF + (q * 32 + lane) * 16, gf + (q * 32 + lane) * 16);
+        constexpr int XV = X::LEN * (int)sizeof(T) / 16, NX = NF * XV;
+#pragma unroll
+        for (int q = 0; q < (NX + 31) / 32; ++q) {
+            const int i = q * 32 + lane, e = i / XV;
+            const int face = __shfl_sync(0xffffffffu, id.y, e < NF ? e : 0);
+            if (i < NX)
+                cp_async<16>(s + XR + i * 16,
+                             reinterpret_cast<const char *>(dc.xrec + (size_t)face * X::LEN) + (i - e * XV) * 16);
+        }
+        cp_async_commit();
+    }
+    template <int N> __device__ __forceinline__ void read(int at, T (&v)[N]) const
+    {
+#pragma unroll
+        for (int q = 0; q < N * (int)sizeof(T) / 16; ++q) {
+            const int4 w = *reinterpret_cast<const int4 *>(s + at + q * 16);
+            const T *t = reinterpret_cast<const T *>(&w);
+#pragma unroll
+            for (int j = 0; j < 16 / (int)sizeof(T); ++j) v[q * (16 / (int)sizeof(T)) + j] = t[j];
+        }
+    }
+    __device__ __forceinline__ int4 ids(int e) const { return *reinterpret_cast<const int4 *>(s + GI + e * 16); }
+    __device__ __forceinline__ void values(int e, int at, T (&v)[4]) const
+    {
+        read<4>(GF + (e * E::LEN + at) * (int)sizeof(T), v);
+    }
+    __device__ __forceinline__ void row_of(int e, P (&x)[NC][NP]) const
+    {
+#pragma unroll
+        for (int m = 0; m < NC; ++m) lds_pack<T, TV>(s + (e * NC + m) * ROW + lane * TV * (int)sizeof(T), x[m]);
+    }
+    __device__ __forceinline__ void own(P (&x)[NC][NP]) const { row_of(NF, x); }
+    __device__ __forceinline__ void row(int e, const int4 &, P (&x)[NC][NP]) const { row_of(e, x); }
+    __device__ __forceinline__ void record(int e, int, T (&x)[X::LEN]) const
+    {
+        read<X::LEN>(XR + e * X::LEN * (int)sizeof(T), x);
+    }
+};
+
 // Micro reconstruction of cell c (Sec. 3.1 Step 2) for the TV consecutive
 // velocities of this lane: least-squares slope grad = sum_j a_cj (f_j - f_c),
 // Venkatakrishnan factor phi = min over the faces of c of (D1^2 + eps^2 +
@@ -643,13 +789,14 @@ __device__ __forceinline__ void entry_range(const DevCase<T> &dc, int c, int &e0
 // so that the reconstruction is non-negative at every face centre and at the
 // foot of the characteristic after one step: with dmin = min(0, min_f D2_f),
 // v = f_c + phi (dmin + min(0, -dt u.grad)); theta = f_c / (f_c - v) if v < 0.
-// fl points at f_cur + the lane's first velocity; fi returns f_c, g the scaled
-// slope, ug = u . g.  NF > 0: ne == NF entries, their rows all requested before
-// the first is used; NF = 0: any number.  A wall or padding entry reads the
-// cell itself (no difference, no extremum).
-template <typename T, int D, int NC, int TV, int NF>
-__device__ __forceinline__ void cell_slope(const DevCase<T> &dc, const T *__restrict__ fl, const int c, const int e0,
-                                           const int ne, const typename Pk<T, TV>::P (&u)[Pk<T, TV>::NP][D],
+// fi returns f_c, g the scaled slope, ug = u . g.  src gives the cell's entries
+// and rows (GlobalCell or the staged ones of the flux pass).  NF > 0: ne == NF
+// entries, their rows all requested before the first is used; NF = 0: any
+// number.  A wall or padding entry reads the cell itself (no difference, no
+// extremum).
+template <typename T, int D, int NC, int TV, int NF, typename Src>
+__device__ __forceinline__ void cell_slope(const DevCase<T> &dc, const Src &src, const int c, const int ne,
+                                           const typename Pk<T, TV>::P (&u)[Pk<T, TV>::NP][D],
                                            typename Pk<T, TV>::P (&fi)[NC][Pk<T, TV>::NP],
                                            typename Pk<T, TV>::P (&g)[NC][Pk<T, TV>::NP][D],
                                            typename Pk<T, TV>::P (&ug)[NC][Pk<T, TV>::NP])
@@ -658,14 +805,11 @@ __device__ __forceinline__ void cell_slope(const DevCase<T> &dc, const T *__rest
     using K = Pk<T, TV>;
     using P = typename K::P;
     constexpr int W = K::W, NP = K::NP;
-    const int nvp = dc.nvp;
-    const size_t rs = (size_t)NC * nvp;
-    const T *fc = fl + (size_t)c * rs;
     P nfi[NC][NP];
     Extrema<T> ex[NC][TV];
+    src.own(fi);
 #pragma unroll
     for (int m = 0; m < NC; ++m) {
-        ldp<T, TV>(fc + (size_t)m * nvp, fi[m]);
 #pragma unroll
         for (int i = 0; i < NP; ++i) {
             nfi[m][i] = pmul(fi[m][i], pbc<P>(T(-1)));
@@ -676,10 +820,9 @@ __device__ __forceinline__ void cell_slope(const DevCase<T> &dc, const T *__rest
         for (int j = 0; j < TV; ++j) ex[m][j].set(pel<W>(fi[m], j));
     }
     // f of the cell across an entry
-    auto across = [&](const int4 gi, P (&fj)[NC][NP]) {
-        const T *fo = fl + (size_t)gi.x * rs;
-#pragma unroll
-        for (int m = 0; m < NC; ++m) ldp<T, TV>(fo + (size_t)m * nvp, fj[m]);
+    auto across = [&](const int e, P (&fj)[NC][NP]) {
+        const int4 gi = src.ids(e);
+        src.row(e, gi, fj);
         if ((gi.z & 255) == FT_FARFIELD) {
             T gr[GREC];
             load_rec<GREC>(dc.grec + (size_t)gi.w * GREC, gr);
@@ -701,7 +844,7 @@ __device__ __forceinline__ void cell_slope(const DevCase<T> &dc, const T *__rest
     };
     auto slope_term = [&](const int e, P (&fj)[NC][NP]) {
         T a[4];
-        load_rec<4>(dc.gf + (size_t)e * E::LEN + (E::A / 4) * 4, a);
+        src.values(e, (E::A / 4) * 4, a);
 #pragma unroll
         for (int m = 0; m < NC; ++m)
 #pragma unroll
@@ -723,16 +866,16 @@ __device__ __forceinline__ void cell_slope(const DevCase<T> &dc, const T *__rest
     if constexpr (NF > 0) {
         P fj[NF][NC][NP];
 #pragma unroll
-        for (int e = 0; e < NF; ++e) across(__ldg(dc.gi + e0 + e), fj[e]);
+        for (int e = 0; e < NF; ++e) across(e, fj[e]);
 #pragma unroll
-        for (int e = 0; e < NF; ++e) slope_term(e0 + e, fj[e]);
+        for (int e = 0; e < NF; ++e) slope_term(e, fj[e]);
 #pragma unroll
         for (int e = 0; e < NF; e += 2) extrema(fj[e], fj[e + 1 < NF ? e + 1 : e], e + 1 < NF, ex);
     } else {
         for (int e = 0; e < ne; ++e) {
             P fj[NC][NP];
-            across(__ldg(dc.gi + e0 + e), fj);
-            slope_term(e0 + e, fj);
+            across(e, fj);
+            slope_term(e, fj);
             extrema(fj, fj, false, ex);
         }
     }
@@ -749,7 +892,7 @@ __device__ __forceinline__ void cell_slope(const DevCase<T> &dc, const T *__rest
         for (int j = 0; j < TV; ++j) d2x[m][j].set(T(0));
     auto offset = [&](const int e, P (&d2)[NC][NP]) {
         T r[4];
-        load_rec<4>(dc.gf + (size_t)e * E::LEN + (E::RS / 4) * 4, r);
+        src.values(e, (E::RS / 4) * 4, r);
 #pragma unroll
         for (int m = 0; m < NC; ++m)
 #pragma unroll
@@ -764,14 +907,14 @@ __device__ __forceinline__ void cell_slope(const DevCase<T> &dc, const T *__rest
 #pragma unroll
         for (int e = 0; e < NF; e += 2) {
             P x[NC][NP], y[NC][NP];
-            offset(e0 + e, x);
-            if (e + 1 < NF) offset(e0 + e + 1, y);
+            offset(e, x);
+            if (e + 1 < NF) offset(e + 1, y);
             extrema(x, y, e + 1 < NF, d2x);
         }
     } else {
         for (int e = 0; e < ne; ++e) {
             P x[NC][NP];
-            offset(e0 + e, x);
+            offset(e, x);
             extrema(x, x, false, d2x);
         }
     }
@@ -810,10 +953,7 @@ __device__ __forceinline__ void cell_slope(const DevCase<T> &dc, const T *__rest
             for (int d = 1; d < D; ++d) s = pfma(u[i][d], g[m][i][d], s);
             const P foot = pmul(s, ndt);
 #pragma unroll
-            for (int w = 0; w < W; ++w) {
-                const T ft = pel<W>(const_cast<P *>(&foot), w);
-                pel<W>(&low, w) = lt0(ft) ? ft : T(0);
-            }
+            for (int w = 0; w < W; ++w) pel<W>(&low, w) = min0(pel<W>(const_cast<P *>(&foot), w));
             low = padd(dn, low);
             P v = pfma(phi, low, fi[m][i]);
 #pragma unroll

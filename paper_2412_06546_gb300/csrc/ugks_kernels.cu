@@ -1365,7 +1365,7 @@ __device__ __forceinline__ void wall_sum_body(const DevCase<T> &dc, const int bx
         for (int j = 0; j < TW; ++j)
 #pragma unroll
             for (int d = 0; d < D; ++d) pel<K::W>(&up[j / K::W][d], j % K::W) = u[d][j];
-        if (out) cell_slope<T, D, NC, TW, 0>(dc, dc.f_cur + k0, c, e0, ne, up, fi, g, ug);
+        if (out) cell_slope<T, D, NC, TW, 0>(dc, GlobalCell<T, D, NC, TW>{dc, dc.f_cur + k0, c, e0}, c, ne, up, fi, g, ug);
 #pragma unroll
         for (int j = 0; j < TW; ++j) {
             const T uj[3] = {u[0][j], u[1][j], u[2][j]};
@@ -1478,10 +1478,14 @@ __global__ void __launch_bounds__(256) k_wall_sum_batch(const DevCase<T> *__rest
 // the update is in place.
 
 // One warp per cell and tile of 32 TV velocities, TV consecutive ones per lane;
-// the warps of a CTA take the P cells of a patch in turn.  Bound: instruction
-// issue and the latency of the neighbours' rows (16 warps per SM; DRAM at 9 % of
-// its peak).  TV = 4 reads an entry or a record for twice the velocities of
-// TV = 2 (107k-cell tetrahedral mesh: 9.1 against 12.4 ms of both kernels).
+// the warps of a CTA take the P cells of a patch in turn.  TV = 4 reads an entry
+// or a record for twice the velocities of TV = 2 (107k-cell tetrahedral mesh:
+// 9.1 against 12.4 ms of both kernels).  The next cell's rows, entries and
+// records are copied to shared memory while a cell is worked on (StagedCell):
+// with loads at their use the 16 warps of an SM waited for memory in 3.8 of 8.9
+// cycles per instruction, now in 1.3 of 7.1, and both kernels went from 8.14 to
+// 7.35 ms on that mesh and from 0.266 to 0.215 on 2,145 hexahedra x 4,080.
+// Bound: instruction issue (54 % of the issue slots, FMA pipe 51 %, DRAM 14 %).
 template <typename T, int D, int NC, int TV, int NF>
 __device__ __forceinline__ void flux_body(const DevCase<T> &dc, const int bx, const int chunk)
 {
@@ -1494,8 +1498,12 @@ __device__ __forceinline__ void flux_body(const DevCase<T> &dc, const int bx, co
     // patches fastest: the CTAs in flight cover neighbouring patches of one
     // tile, so that the rows of f and of the flux buffer they share stay in L2
     const int tile = bx / dc.n_patches, p = bx - tile * dc.n_patches;
-    const int kc = tile * V + TV * lane, k = chunk * dc.chunk + kc;   // in the chunk, of all
-    if (kc >= dc.chunk || k >= dc.nvp) return;                        // the last tile may be short
+    // the lane's first velocity in the chunk and of all; the last tile may be
+    // short: its lanes beyond the end repeat the tile's start and store nothing
+    const int kl = tile * V + TV * lane;
+    const bool live = kl < dc.chunk && chunk * dc.chunk + kl < dc.nvp;
+    const int kc = live ? kl : tile * V, k = chunk * dc.chunk + kc;
+    const unsigned all = live ? (1u << TV) - 1 : 0u;
     const int cb = p * dc.P, ce = min(dc.C, cb + dc.P);
     const T *__restrict__ fl = dc.f_cur + k;
     P u[NP][D];
@@ -1507,18 +1515,16 @@ __device__ __forceinline__ void flux_body(const DevCase<T> &dc, const int bx, co
         for (int i = 0; i < NP; ++i) u[i][d] = t[i];
     }
     const T dt = dc.dtT, hdt2 = T(0.5) * dc.dtT * dc.dtT;
-    for (int c = cb + warp; c < ce; c += nwarps) {
-        int e0 = c * NF, ne = NF;
-        if (NF == 0) entry_range(dc, c, e0, ne);
+    auto cell = [&](const int c, const auto &src, const int ne) {
         P fi[NC][NP], g[NC][NP][D], ug[NC][NP];
-        cell_slope<T, D, NC, TV, NF>(dc, fl, c, e0, ne, u, fi, g, ug);
+        cell_slope<T, D, NC, TV, NF>(dc, src, c, ne, u, fi, g, ug);
         auto face = [&](const int e) {
-            const int4 gi = __ldg(dc.gi + e);
+            const int4 gi = src.ids(e);
             const int type = gi.z & 255;
             if (type == FT_NONE) return;
             T rsv[4], nv[4];
-            load_rec<4>(dc.gf + (size_t)e * E::LEN + (E::RS / 4) * 4, rsv);
-            load_rec<4>(dc.gf + (size_t)e * E::LEN + E::N, nv);
+            src.values(e, (E::RS / 4) * 4, rsv);
+            src.values(e, E::N, nv);
             const T *r = rsv + E::RS % 4;
             P un[NP];
 #pragma unroll
@@ -1529,6 +1535,7 @@ __device__ __forceinline__ void flux_body(const DevCase<T> &dc, const int bx, co
             unsigned on = 0;
 #pragma unroll
             for (int j = 0; j < TV; ++j) on |= (gt0(pel<W>(un, j)) == own ? 1u : 0u) << j;
+            on &= all;
             P F[NC][NP];
             // value of the cell at the face centre
             auto at_face = [&](int m, int i) {
@@ -1554,10 +1561,10 @@ __device__ __forceinline__ void flux_body(const DevCase<T> &dc, const int bx, co
                         pel<W>(F[m], j) = (on >> j & 1) ? unj * out : (m == 0 ? unj * dt : unj * dt * wr[GR_NB]) * H;
                     }
                 }
-                on = (1u << TV) - 1;
+                on = all;
             } else {
                 T x[X::LEN];
-                load_rec<X::LEN>(dc.xrec + (size_t)gi.y * X::LEN, x);
+                src.record(e, gi.y, x);
                 P fup[NC][NP], ugf[NC][NP];
 #pragma unroll
                 for (int m = 0; m < NC; ++m)
@@ -1582,20 +1589,18 @@ __device__ __forceinline__ void flux_body(const DevCase<T> &dc, const int bx, co
                             pel<W>(ugf[m], j) = T(0);
                         }
                     }
-                    on = (1u << TV) - 1;
+                    on = all;
                 }
                 const P q1 = pbc<P>(x[X::Q1]), q2 = pbc<P>(x[X::Q2]);
 #pragma unroll
                 for (int i = 0; i < NP; ++i) {
-                    P cv[D], c2, h;
+                    P cv[D], c2;
 #pragma unroll
                     for (int d = 0; d < D; ++d) {
                         cv[d] = padd(u[i][d], pbc<P>(x[X::U + d]));
                         c2 = d == 0 ? pmul(cv[0], cv[0]) : pfma(cv[d], cv[d], c2);
                     }
-#pragma unroll
-                    for (int w = 0; w < W; ++w) pel<W>(&h, w) = gauss_ex(x[X::EX], pel<W>(&c2, w));
-                    h = pmul(h, pbc<P>(x[X::PREF]));
+                    const P h = pmul(gauss_ex(x[X::EX], c2), pbc<P>(x[X::PREF]));
 #pragma unroll
                     for (int m = 0; m < NC; ++m) {
                         const P eq = poly_eval<T, D, P>(x + X::POLY + m * Poly<D>::N, cv, c2);
@@ -1622,18 +1627,56 @@ __device__ __forceinline__ void flux_body(const DevCase<T> &dc, const int bx, co
         };
         if constexpr (NF > 0) {
 #pragma unroll
-            for (int e = 0; e < NF; ++e) face(e0 + e);
+            for (int e = 0; e < NF; ++e) face(e);
         } else {
-            for (int e = 0; e < ne; ++e) face(e0 + e);
+            for (int e = 0; e < ne; ++e) face(e);
+        }
+    };
+    if constexpr (NF > 0) {
+        // two stages per warp: while a cell is worked on, the next one's rows,
+        // entries and records are on their way, and the entry ids of the one
+        // after it (which the requests need) are being loaded
+        extern __shared__ __align__(16) unsigned char stages[];
+        using S = StagedCell<T, D, NC, TV, NF>;
+        const S st[2] = {{stages + (size_t)(2 * warp) * S::BYTES, lane}, {stages + (size_t)(2 * warp + 1) * S::BYTES, lane}};
+        auto ids = [&](int c) {
+            return lane < NF && c < ce ? __ldg(dc.gi + (size_t)c * NF + lane) : make_int4(0, 0, 0, 0);
+        };
+        int c = cb + warp;
+        if (c >= ce) return;
+        st[0].request(dc, fl, c, ids(c));
+        int4 id = ids(c + nwarps);
+        for (int b = 0; c < ce; c += nwarps, b ^= 1) {
+            __syncwarp();                                 // the stage to be filled has been read
+            const S &cur = st[b];
+            if (c + nwarps < ce) st[b ^ 1].request(dc, fl, c + nwarps, id);
+            else cp_async_commit();                       // an empty group, for the wait below
+            id = ids(c + 2 * nwarps);
+            cp_async_wait<1>();
+            __syncwarp();
+            cell(c, cur, NF);
+        }
+    } else {
+        for (int c = cb + warp; c < ce; c += nwarps) {
+            int e0, ne;
+            entry_range(dc, c, e0, ne);
+            cell(c, GlobalCell<T, D, NC, TV>{dc, fl, c, e0}, ne);
         }
     }
 }
 
+// dynamic shared memory of a CTA of the flux pass
+template <typename T, int D, int NC, int TV, int NF> constexpr int flux_smem(int nth)
+{
+    if constexpr (NF == 0) return 0;
+    else return nth / 32 * 2 * StagedCell<T, D, NC, TV, NF>::BYTES;
+}
+
 // 512-thread CTAs are held to 64 registers so that two fit an SM; 256-thread
-// CTAs take what ptxas chooses (118 registers for tetrahedra at TV = 4, two CTAs
-// per SM): held to 80 registers, three CTAs spill and measure 8.00 against
-// 8.30 ms on the 107k-cell tetrahedral mesh but 9.02 against 8.77 ms on 24k
-// cells x 28^3 and 1.81 against 1.74 ms on the 30k-cell triangulation.
+// CTAs take what ptxas chooses (108 registers for tetrahedra at TV = 4, two CTAs
+// per SM): held to 80 registers, three CTAs spill and measure 7.55 against
+// 7.12 ms on the 107k-cell tetrahedral mesh (with stage 1), 8.41 against 7.74 on
+// 24k cells x 28^3 and 1.58 against 1.52 on the 30k-cell triangulation.
 template <typename T, int D, int NC, int TV, int NF, int NTH>
 __global__ void __launch_bounds__(NTH, NTH >= 512 ? 2 : 0) k_flux(DevCase<T> dc, int chunk)
 {
@@ -1675,6 +1718,21 @@ template <> struct MomentSum<float2> {
 // velocities per lane.  Bound: the latency of its row loads (nf rows of the flux
 // buffer and f, which is written in place); the reduction at a group's end costs
 // as much as 250 velocities (see set_chunks in ugks_host.cu).
+//
+// The rows come through a ring of NS slots in shared memory, filled NS - 1
+// iterations ahead by asynchronous copies (a lane reads back what it copied, so
+// no barrier): without it a warp had the loads of one iteration in flight and
+// waited for them in 11 of 15 cycles per instruction (7.35 -> 7.12 ms of both
+// kernels on the 107k-cell mesh, 1.56 -> 1.52 on the 30k-cell triangulation).
+template <typename T, int NC, int NF> constexpr int stage1_stages()
+{
+    return (NF + 1) * NC * 4 * (int)sizeof(T) * 32 * 8 * 3 <= 64 * 1024 ? 3 : 2;
+}
+template <typename T, int NC, int NF> constexpr int stage1_smem()
+{
+    return NF == 0 ? 0 : stage1_stages<T, NC, NF>() * (NF + 1) * NC * 4 * (int)sizeof(T) * 32 * 8;
+}
+
 template <typename T, int D, int NC, int NF>
 __device__ __forceinline__ void stage1_body(const DevCase<T> &dc, const int bx, const int chunk)
 {
@@ -1693,6 +1751,24 @@ __device__ __forceinline__ void stage1_body(const DevCase<T> &dc, const int bx, 
     if (NF == 0) entry_range(dc, c, e0, ne);
     T cs[NF > 0 ? NF : 1];
     const T *Fr[NF > 0 ? NF : 1];
+    T *frow = dc.f_cur + (size_t)c * NC * dc.nvp + kb;
+    constexpr int B = 4 * (int)sizeof(T), NS = stage1_stages<T, NC, NF>(), ROWS = (NF + 1) * NC;
+    extern __shared__ __align__(16) unsigned char stages[];
+    unsigned char *const mine = stages + ((size_t)(threadIdx.x >> 5) * NS * ROWS * 32 + lane) * B;
+    // rows of the velocities at kc into ring slot q: the faces' fluxes, then f
+    auto request = [&](const int kc, const int q) {
+        if (kc < kn) {
+            unsigned char *dst = mine + (size_t)q * ROWS * 32 * B;
+#pragma unroll
+            for (int e = 0; e < NF; ++e)
+#pragma unroll
+                for (int m = 0; m < NC; ++m)
+                    cp_async_lane<B>(dst + (e * NC + m) * 32 * B, Fr[e] + (size_t)m * dc.chunk + kc);
+#pragma unroll
+            for (int m = 0; m < NC; ++m) cp_async_lane<B>(dst + (NF * NC + m) * 32 * B, frow + (size_t)m * dc.nvp + kc);
+        }
+        cp_async_commit();
+    };
     if constexpr (NF > 0) {
         // a padding entry reads the first face's row with coefficient 0
         const int f0 = __ldg(dc.gi + e0).y;
@@ -1702,6 +1778,8 @@ __device__ __forceinline__ void stage1_body(const DevCase<T> &dc, const int bx, 
             cs[e] = __ldg(dc.gf + (size_t)(e0 + e) * E::LEN + E::CS);
             Fr[e] = dc.flux + (size_t)(gi.z == FT_NONE ? f0 : gi.y) * NC * dc.chunk;
         }
+#pragma unroll
+        for (int q = 0; q < NS - 1; ++q) request(kg + 4 * lane + 128 * q, q);
     }
     T cr[CREC];
     load_rec<CREC>(dc.crec + (size_t)c * CREC, cr);
@@ -1709,35 +1787,29 @@ __device__ __forceinline__ void stage1_body(const DevCase<T> &dc, const int bx, 
     MomentSum<P> acc[M];
 #pragma unroll
     for (int i = 0; i < M; ++i) acc[i].zero();
-    T *frow = dc.f_cur + (size_t)c * NC * dc.nvp + kb;
+    int slot = 0;
     for (int kc = kg + 4 * lane; kc < kn; kc += 128) {
         P fs[NC][NP], R[NC][NP];
 #pragma unroll
-        for (int m = 0; m < NC; ++m) {
-            using V4 = typename VecOf<T, vec_chunk<T, 4>()>::type;
-            constexpr int CH = vec_chunk<T, 4>();
-#pragma unroll
-            for (int q = 0; q < 4 / CH; ++q) {                        // f is written below: ordinary loads
-                const V4 v = reinterpret_cast<const V4 *>(frow + (size_t)m * dc.nvp + kc)[q];
-                const T *ev = reinterpret_cast<const T *>(&v);
-#pragma unroll
-                for (int j = 0; j < CH; ++j) pel<W>(fs[m], q * CH + j) = ev[j];
-            }
+        for (int m = 0; m < NC; ++m)
 #pragma unroll
             for (int i = 0; i < NP; ++i) R[m][i] = pbc<P>(T(0));
-        }
         if constexpr (NF > 0) {
-            P Fv[NF][NC][NP];
+            request(kc + 128 * (NS - 1), slot == 0 ? NS - 1 : slot - 1);   // the slot read last
+            cp_async_wait<NS - 1>();
+            const unsigned char *src = mine + (size_t)slot * ROWS * 32 * B;
+            slot = slot == NS - 1 ? 0 : slot + 1;
 #pragma unroll
             for (int e = 0; e < NF; ++e)
 #pragma unroll
-                for (int m = 0; m < NC; ++m) ldp<T, 4>(Fr[e] + (size_t)m * dc.chunk + kc, Fv[e][m]);
+                for (int m = 0; m < NC; ++m) {
+                    P Fv[NP];
+                    lds_pack<T, 4>(src + (e * NC + m) * 32 * B, Fv);
 #pragma unroll
-            for (int e = 0; e < NF; ++e)
+                    for (int i = 0; i < NP; ++i) R[m][i] = pfma(pbc<P>(cs[e]), Fv[i], R[m][i]);
+                }
 #pragma unroll
-                for (int m = 0; m < NC; ++m)
-#pragma unroll
-                    for (int i = 0; i < NP; ++i) R[m][i] = pfma(pbc<P>(cs[e]), Fv[e][m][i], R[m][i]);
+            for (int m = 0; m < NC; ++m) lds_pack<T, 4>(src + (NF * NC + m) * 32 * B, fs[m]);
         } else {
             for (int e = 0; e < ne; ++e) {
                 const int4 gi = __ldg(dc.gi + e0 + e);
@@ -1750,6 +1822,10 @@ __device__ __forceinline__ void stage1_body(const DevCase<T> &dc, const int bx, 
                     for (int i = 0; i < NP; ++i) R[m][i] = pfma(ce, Fv[i], R[m][i]);
                 }
             }
+#pragma unroll
+            for (int m = 0; m < NC; ++m)                               // f is written below: ordinary loads
+#pragma unroll
+                for (int j = 0; j < 4; ++j) pel<W>(fs[m], j) = frow[(size_t)m * dc.nvp + kc + j];
         }
         P u[D][NP], wk[NP];
 #pragma unroll
@@ -1938,29 +2014,35 @@ __device__ __forceinline__ void collide_body(const DevCase<T> &dc, const int bx)
     for (int d = 0; d < NP; ++d) blk[d] = 0;
     double acc = 0.0;
     int nblk = 0;
-    // the f~ vectors of the next iteration are loaded before this one's
-    // arithmetic, so that a warp keeps a load in flight while it computes
+    // f~ comes through a ring of COLLIDE_SLOTS slots of shared memory per lane,
+    // filled by asynchronous copies COLLIDE_SLOTS - 1 iterations ahead
     T *frow = dc.f_cur + (size_t)c * rs;
-    V4 nxt[NC];
-    if (4 * lane < dc.nvp)
+    constexpr int B = 4 * (int)sizeof(T), COLLIDE_SLOTS = sizeof(T) == 4 ? 3 : 2;
+    __shared__ __align__(32) unsigned char ring[8 * COLLIDE_SLOTS * NC * 32 * B];
+    unsigned char *const mine = ring + ((threadIdx.x >> 5) * COLLIDE_SLOTS * NC * 32 + lane) * B;
+    auto request = [&](int k0, int q) {
+        if (k0 < dc.nvp)
 #pragma unroll
-        for (int m = 0; m < NC; ++m) nxt[m] = *reinterpret_cast<const V4 *>(frow + (size_t)m * dc.nvp + 4 * lane);
+            for (int m = 0; m < NC; ++m) cp_async_lane<B>(mine + (q * NC + m) * 32 * B, frow + (size_t)m * dc.nvp + k0);
+        cp_async_commit();
+    };
+#pragma unroll
+    for (int q = 0; q < COLLIDE_SLOTS - 1; ++q) request(128 * q + 4 * lane, q);
+    int slot = 0;
     for (int k00 = 0; k00 < dc.nvp; k00 += 128) {          // uniform over the warp
         const int k0 = k00 + 4 * lane;
+        request(k0 + 128 * (COLLIDE_SLOTS - 1), slot == 0 ? COLLIDE_SLOTS - 1 : slot - 1);
+        cp_async_wait<COLLIDE_SLOTS - 1>();
         if (k0 < dc.nvp) {
             T ft[NC][4], fn[NC][4];
 #pragma unroll
             for (int m = 0; m < NC; ++m) {
-                const V4 v = nxt[m];
+                const V4 v = *reinterpret_cast<const V4 *>(mine + (slot * NC + m) * 32 * B);
                 ft[m][0] = v.x;
                 ft[m][1] = v.y;
                 ft[m][2] = v.z;
                 ft[m][3] = v.w;
             }
-            if (k0 + 128 < dc.nvp)
-#pragma unroll
-                for (int m = 0; m < NC; ++m)
-                    nxt[m] = *reinterpret_cast<const V4 *>(frow + (size_t)m * dc.nvp + k0 + 128);
             // the lane's four velocities from the per-component arrays: each load
             // of the warp covers one contiguous span (the packed [k][4] records
             // of four consecutive velocities per lane would touch four times the
@@ -2001,6 +2083,7 @@ __device__ __forceinline__ void collide_body(const DevCase<T> &dc, const int bx)
                 *reinterpret_cast<V4 *>(frow + (size_t)m * dc.nvp + k0) = v;
             }
         }
+        slot = slot == COLLIDE_SLOTS - 1 ? 0 : slot + 1;
         if constexpr (F32) {
             if (++nblk == SUM_BLOCK / 4 || k00 + 128 >= dc.nvp) {
                 acc += block_to_fp64<NP>(blk);
@@ -2022,10 +2105,12 @@ __device__ __forceinline__ void collide_body(const DevCase<T> &dc, const int bx)
     }
 }
 
-// five 256-thread blocks per SM in the 2D FP32 form (48 registers); the 3D
-// FP32 form and the batched kernels would spill at that bound
+// four 256-thread blocks per SM in the 2D FP32 form (five would spill).  Ring of
+// 3 slots on the 30k x 60x50 and the 107k x 4,568 cases: 0.304 -> 0.236 ms (6.2
+// TB/s) and 0.766 -> 0.731 ms (5.4 TB/s; the latency of the arithmetic chain is
+// what is left in 3D); 4 and 6 slots 0.236 and 0.245, 0.738 and 0.728.
 template <typename T, int D, int NC>
-__global__ void __launch_bounds__(256, sizeof(T) == 4 && D == 2 ? 5 : 0) k_collide(DevCase<T> dc)
+__global__ void __launch_bounds__(256, sizeof(T) == 4 && D == 2 ? 4 : 0) k_collide(DevCase<T> dc)
 {
     collide_body<T, D, NC>(dc, blockIdx.x);
 }
@@ -2208,8 +2293,16 @@ template <typename T, int D, int NC, int TV, int NF, int NTH>
 static cudaError_t flux_launch(int blocks, int chunk, cudaStream_t st, const DevCase<T> *dc, const DevCase<T> *cases,
                                const int *off, int n)
 {
-    if (cases) k_flux_batch<T, D, NC, TV, NF, NTH><<<blocks, NTH, 0, st>>>(cases, off, n, chunk);
-    else k_flux<T, D, NC, TV, NF, NTH><<<blocks, NTH, 0, st>>>(*dc, chunk);
+    constexpr int smem = flux_smem<T, D, NC, TV, NF>(NTH);
+    if (smem > 48 * 1024) {
+        const cudaError_t e = cases ? cudaFuncSetAttribute(k_flux_batch<T, D, NC, TV, NF, NTH>,
+                                                           cudaFuncAttributeMaxDynamicSharedMemorySize, smem)
+                                    : cudaFuncSetAttribute(k_flux<T, D, NC, TV, NF, NTH>,
+                                                           cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e != cudaSuccess) return e;
+    }
+    if (cases) k_flux_batch<T, D, NC, TV, NF, NTH><<<blocks, NTH, smem, st>>>(cases, off, n, chunk);
+    else k_flux<T, D, NC, TV, NF, NTH><<<blocks, NTH, smem, st>>>(*dc, chunk);
     return cudaGetLastError();
 }
 
@@ -2253,8 +2346,16 @@ template <typename T, int D, int NC, int NF>
 static cudaError_t stage1_launch(int blocks, int chunk, cudaStream_t st, const DevCase<T> *dc, const DevCase<T> *cases,
                                  const int *off, int n)
 {
-    if (cases) k_stage1_batch<T, D, NC, NF><<<blocks, 256, 0, st>>>(cases, off, n, chunk);
-    else k_stage1<T, D, NC, NF><<<blocks, 256, 0, st>>>(*dc, chunk);
+    constexpr int smem = stage1_smem<T, NC, NF>();
+    if (smem > 48 * 1024) {
+        const cudaError_t e = cases ? cudaFuncSetAttribute(k_stage1_batch<T, D, NC, NF>,
+                                                           cudaFuncAttributeMaxDynamicSharedMemorySize, smem)
+                                    : cudaFuncSetAttribute(k_stage1<T, D, NC, NF>,
+                                                           cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e != cudaSuccess) return e;
+    }
+    if (cases) k_stage1_batch<T, D, NC, NF><<<blocks, 256, smem, st>>>(cases, off, n, chunk);
+    else k_stage1<T, D, NC, NF><<<blocks, 256, smem, st>>>(*dc, chunk);
     return cudaGetLastError();
 }
 
