@@ -103,11 +103,11 @@ typedef struct {
     double inf_rho, inf_U[3], inf_T; /* far-field state */
     int32_t precision;      /* UGKS_FP64 or UGKS_FP32 */
     const double *prim_init;/* [n_cells][dim+2] initial (rho, U, T), or NULL: far-field state */
-    int32_t patch_cells;    /* tiling of the flux pass: cells per CTA (0: autotuned by timing the pass on
+    int32_t patch_cells;    /* tiling of the flux pass: cells per patch (0: autotuned by timing the pass on
                                this case, cached per case shape) */
     int32_t vtile;          /* velocities per warp of the flux pass, 32, 64 or 128 (0: automatic) */
-    int32_t gather_threads; /* threads per CTA of the flux pass, 256 or 512 (512 only for UGKS_FP32 with
-                               vtile <= 64; 0: automatic, 256 unless the autotuner picks 512) */
+    int32_t gather_threads; /* threads per patch of the flux pass, 256 or 512 (512 only for UGKS_FP32 with
+                               vtile <= 64; 0: 256), in CTAs of 128 */
     int32_t gather_tile_group; /* velocity tiles per moment group of stage 1: the moments of a cell's flux
                                residual are summed over groups of this many tiles, the groups in FP64
                                (1 .. 1024, larger values are clamped to the number of tiles, and to what
@@ -140,7 +140,7 @@ typedef struct {
     int32_t n_patches, patch_cells, vtile;  /* tiling of the flux pass in use */
     int64_t kernel_launches_per_step;
     int64_t n_wall_faces;               /* faces of type UGKS_FACE_WALL */
-    int32_t gather_threads;             /* threads per CTA of the flux pass in use */
+    int32_t gather_threads;             /* threads per patch of the flux pass in use */
     int32_t gather_tile_group;          /* velocity tiles per moment group of stage 1 in use */
 } ugks_info_t;
 
@@ -239,7 +239,7 @@ ugks_status ugks_profile_end(ugks_case *c, double *ms, int32_t n, int32_t *steps
 /* Batched stepping of several cases (one GPU).  The cases must share the
  * dimension and precision.  Each batch step runs every kernel once for all cases
  * (block offsets per case), the flux and stage-1 kernels once per velocity chunk
- * and per (velocity tile, block size, faces per cell) present in the batch, so a
+ * and per (velocity tile, faces per cell) present in the batch, so a
  * step is about a dozen launches whatever the number of cases.  The whole
  * step is captured once as a CUDA graph on `stream` (cudaStream_t, NULL: a
  * stream of the batch's own) and replayed.  Results are bit-identical to

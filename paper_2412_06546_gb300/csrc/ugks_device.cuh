@@ -150,8 +150,8 @@ struct DevCase {
                                   // SUM1_SEP_MAX_NL nodes (separable half-range sums)
     const T *axis[3], *axw[3];
     // tiling of the flux and stage-1 passes
-    int P, n_patches, vtile;      // cells per CTA and velocities per warp of the flux pass
-    int nth;                      // threads per CTA of the flux pass (256, or 512 for FP32 at vtile <= 64)
+    int P, n_patches, vtile;      // cells per patch and velocities per warp of the flux pass
+    int nth;                      // threads per patch (256, or 512 for FP32 at vtile <= 64), in CTAs of 128
     int chunk, n_chunks;          // velocities per chunk (a multiple of gvel), chunks
     int gvel, n_groups;           // velocities of a cell per warp of stage 1 (a multiple of vtile), groups per cell
 };

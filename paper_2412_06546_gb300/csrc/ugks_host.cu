@@ -772,32 +772,30 @@ void set_chunks(ugks_case *c, int tile_group)
     c->n_chunks = (nvp + c->chunk - 1) / c->chunk;
 }
 
-// Autotuner of the flux pass: cells per CTA, velocities per warp and threads per
-// CTA are chosen by timing the flux and stage-1 passes themselves on this case
-// (before the state is initialised for the caller), and the choice is cached
-// per (dimension, precision, velocity count, mesh-size bucket) for later cases
-// of the same shape.
+// Autotuner of the flux pass: cells per patch and velocities per warp are chosen
+// by timing the flux and stage-1 passes themselves on this case (before the
+// state is initialised for the caller), and the choice is cached per (dimension,
+// precision, velocity count, mesh-size bucket) for later cases of the same shape.
 struct Tiling {
-    int P = 0, vtile = 0, nth = 256;
+    int P = 0, vtile = 0;
 };
 std::mutex g_tune_mutex;
 std::map<std::string, Tiling> g_tune_cache;
 
 template <typename T>
-void set_tiling(ugks_case *c, ugks::DevCase<T> &dc, int P, int vtile, int nth)
+void set_tiling(ugks_case *c, ugks::DevCase<T> &dc, int P, int vtile)
 {
     dc.P = c->P = P;
     dc.n_patches = c->n_patches = (int)((c->C + P - 1) / P);
     dc.vtile = c->vtile = vtile;
-    dc.nth = c->nth = nth;
 }
 
 template <typename T>
-void autotune(ugks_case *c, ugks::DevCase<T> &dc, bool tune_vtile, bool tune_threads)
+void autotune(ugks_case *c, ugks::DevCase<T> &dc, bool tune_vtile)
 {
     char key[160];
     snprintf(key, sizeof(key), "D%d_nf%d_p%d_vt%d_t%d_g%d_nv%lld_c%d", c->D, c->nf, c->prec,
-             tune_vtile ? 0 : c->vtile, tune_threads ? 0 : c->nth, c->gvel, (long long)c->Nv,
+             tune_vtile ? 0 : c->vtile, c->nth, c->gvel, (long long)c->Nv,
              (int)std::lround(std::log2((double)c->C)));
     Tiling best;
     {
@@ -806,40 +804,37 @@ void autotune(ugks_case *c, ugks::DevCase<T> &dc, bool tune_vtile, bool tune_thr
         if (it != g_tune_cache.end()) best = it->second;
     }
     if (best.P == 0) {
-        std::vector<int> vc = {c->vtile}, tc = {c->nth};
+        std::vector<int> vc = {c->vtile};
         if (tune_vtile) vc = c->prec == UGKS_FP64 ? std::vector<int>{32, 64} : std::vector<int>{64, 128};
-        if (tune_threads && c->prec == UGKS_FP32) tc = {256, 512};
         cuda_ok(ugks::launch_pre_gather(dc, c->stream), "autotune prep");
         cudaEvent_t e0, e1;
         cuda_ok(cudaEventCreate(&e0), "event");
         cuda_ok(cudaEventCreate(&e1), "event");
         float best_ms = 0.f;
-        for (int nth : tc)
-            for (int vt : vc) {
-                if ((c->chunk % vt && c->n_chunks > 1) || (nth == 512 && vt > 64)) continue;
-                for (int P : {8, 16, 32, 64}) {
-                    if (P < nth / 32) continue;          // a warp per cell
-                    if (P > 16 && P > c->C / 64) continue;
-                    set_tiling(c, dc, P, vt, nth);
-                    cuda_ok(ugks::launch_gather(dc, c->stream), "autotune gather");
-                    cuda_ok(cudaEventRecord(e0, c->stream), "event");
-                    for (int r = 0; r < 2; ++r) cuda_ok(ugks::launch_gather(dc, c->stream), "autotune gather");
-                    cuda_ok(cudaEventRecord(e1, c->stream), "event");
-                    cuda_ok(cudaEventSynchronize(e1), "event");
-                    float ms = 0.f;
-                    cuda_ok(cudaEventElapsedTime(&ms, e0, e1), "event");
-                    if (best.P == 0 || ms < best_ms) {
-                        best = {P, vt, nth};
-                        best_ms = ms;
-                    }
+        for (int vt : vc) {
+            if ((c->chunk % vt && c->n_chunks > 1) || (c->nth == 512 && vt > 64)) continue;
+            for (int P : {8, 16, 32, 64}) {
+                if (P > 8 && (P < c->nth / 32 || P > std::max<int64_t>(16, c->C / 64))) continue;
+                set_tiling(c, dc, P, vt);
+                cuda_ok(ugks::launch_gather(dc, c->stream), "autotune gather");
+                cuda_ok(cudaEventRecord(e0, c->stream), "event");
+                for (int r = 0; r < 2; ++r) cuda_ok(ugks::launch_gather(dc, c->stream), "autotune gather");
+                cuda_ok(cudaEventRecord(e1, c->stream), "event");
+                cuda_ok(cudaEventSynchronize(e1), "event");
+                float ms = 0.f;
+                cuda_ok(cudaEventElapsedTime(&ms, e0, e1), "event");
+                if (best.P == 0 || ms < best_ms) {
+                    best = {P, vt};
+                    best_ms = ms;
                 }
             }
+        }
         cudaEventDestroy(e0);
         cudaEventDestroy(e1);
         std::lock_guard<std::mutex> lock(g_tune_mutex);
         g_tune_cache[key] = best;
     }
-    set_tiling(c, dc, best.P, best.vtile, best.nth);
+    set_tiling(c, dc, best.P, best.vtile);
 }
 
 ugks_status guard(const std::function<void()> &fn)
@@ -1034,7 +1029,7 @@ ugks_status ugks_create(const ugks_mesh *mesh, const ugks_vgrid *vgrid, const ug
             cuda_ok(ugks::launch_init(dc, c->stream), "init");
             if (params->patch_cells == 0) {
                 // the trial passes overwrite f in place: initialise it again
-                autotune(c.get(), dc, params->vtile == 0, params->gather_threads == 0);
+                autotune(c.get(), dc, params->vtile == 0);
                 cuda_ok(ugks::launch_init(dc, c->stream), "init");
             }
             c->vt_group = params->gather_tile_group > 0
@@ -1394,10 +1389,10 @@ struct ugks_batch {
     bool own_stream = false;
     void *dcases = nullptr;         // device array of DevCase<T>
     // the flux and stage-1 passes, one launch each per chunk over the cases of a
-    // group (same velocity tile, threads per CTA and entry count): per chunk
+    // group (same velocity tile and entry count): per chunk
     // the block offsets of both kernels over all cases of the batch
     struct Group {
-        int vtile = 0, nth = 256, nf = 0, n_chunks = 0;
+        int vtile = 0, nf = 0, n_chunks = 0;
         int *off = nullptr;                  // [n_chunks][2][n + 1]
         std::vector<int> blocks;             // [n_chunks][2]
     };
@@ -1451,12 +1446,11 @@ void batch_build(ugks_batch *b)
     cuda_ok(cudaMemcpy(b->small_off, off.data(), off.size() * sizeof(int), cudaMemcpyHostToDevice), "batch upload");
     for (auto *first : b->cases) {
         auto in_group = [&](const ugks_case *c) {
-            return c->vtile == first->vtile && c->nth == first->nth && c->nf == first->nf;
+            return c->vtile == first->vtile && c->nf == first->nf;
         };
         if (first != *std::find_if(b->cases.begin(), b->cases.end(), in_group)) continue;   // its group is there
         ugks_batch::Group g;
         g.vtile = first->vtile;
-        g.nth = first->nth;
         g.nf = first->nf;
         for (auto *c : b->cases)
             if (in_group(c)) g.n_chunks = std::max(g.n_chunks, c->n_chunks);
@@ -1494,7 +1488,7 @@ void batch_capture(ugks_batch *b)
     for (const auto &g : b->groups)
         for (int r = 0; r < g.n_chunks; ++r) {
             const int *off = g.off + (size_t)r * 2 * (n + 1);
-            cuda_ok(ugks::launch_flux<T>(b->D, g.nf, g.vtile, g.nth, g.blocks[2 * r], r, st, nullptr, dcs, off, n),
+            cuda_ok(ugks::launch_flux<T>(b->D, g.nf, g.vtile, g.blocks[2 * r], r, st, nullptr, dcs, off, n),
                     "batched flux pass");
             cuda_ok(ugks::launch_stage1<T>(b->D, g.nf, g.blocks[2 * r + 1], r, st, nullptr, dcs, off + n + 1, n),
                     "batched stage 1");

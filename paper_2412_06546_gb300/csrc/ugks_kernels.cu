@@ -1478,7 +1478,8 @@ __global__ void __launch_bounds__(256) k_wall_sum_batch(const DevCase<T> *__rest
 // the update is in place.
 
 // One warp per cell and tile of 32 TV velocities, TV consecutive ones per lane;
-// the warps of a CTA take the P cells of a patch in turn.  TV = 4 reads an entry
+// the nth / 32 warps of a patch (in CTAs of four) take its P cells in turn.  TV =
+// 4 reads an entry
 // or a record for twice the velocities of TV = 2 (107k-cell tetrahedral mesh:
 // 9.1 against 12.4 ms of both kernels).  The next cell's rows, entries and
 // records are copied to shared memory while a cell is worked on (StagedCell):
@@ -1486,6 +1487,8 @@ __global__ void __launch_bounds__(256) k_wall_sum_batch(const DevCase<T> *__rest
 // cycles per instruction, now in 1.3 of 7.1, and both kernels went from 8.14 to
 // 7.35 ms on that mesh and from 0.266 to 0.215 on 2,145 hexahedra x 4,080.
 // Bound: instruction issue (54 % of the issue slots, FMA pipe 51 %, DRAM 14 %).
+constexpr int FLUX_THREADS = 128;
+
 template <typename T, int D, int NC, int TV, int NF>
 __device__ __forceinline__ void flux_body(const DevCase<T> &dc, const int bx, const int chunk)
 {
@@ -1494,10 +1497,13 @@ __device__ __forceinline__ void flux_body(const DevCase<T> &dc, const int bx, co
     using K = Pk<T, TV>;
     using P = typename K::P;
     constexpr int W = K::W, NP = K::NP, V = 32 * TV;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
     // patches fastest: the CTAs in flight cover neighbouring patches of one
     // tile, so that the rows of f and of the flux buffer they share stay in L2
-    const int tile = bx / dc.n_patches, p = bx - tile * dc.n_patches;
+    const int split = dc.nth / FLUX_THREADS, ncta = dc.n_patches * split;
+    const int tile = bx / ncta, p = (bx - tile * ncta) / split;
+    const int lane = threadIdx.x & 31, nwarps = dc.nth >> 5;
+    const int mine = threadIdx.x >> 5;                                // in the CTA
+    const int warp = mine + (bx - tile * ncta - p * split) * (FLUX_THREADS / 32);   // on the patch
     // the lane's first velocity in the chunk and of all; the last tile may be
     // short: its lanes beyond the end repeat the tile's start and store nothing
     const int kl = tile * V + TV * lane;
@@ -1638,7 +1644,7 @@ __device__ __forceinline__ void flux_body(const DevCase<T> &dc, const int bx, co
         // after it (which the requests need) are being loaded
         extern __shared__ __align__(16) unsigned char stages[];
         using S = StagedCell<T, D, NC, TV, NF>;
-        const S st[2] = {{stages + (size_t)(2 * warp) * S::BYTES, lane}, {stages + (size_t)(2 * warp + 1) * S::BYTES, lane}};
+        const S st[2] = {{stages + (size_t)(2 * mine) * S::BYTES, lane}, {stages + (size_t)(2 * mine + 1) * S::BYTES, lane}};
         auto ids = [&](int c) {
             return lane < NF && c < ce ? __ldg(dc.gi + (size_t)c * NF + lane) : make_int4(0, 0, 0, 0);
         };
@@ -1666,25 +1672,28 @@ __device__ __forceinline__ void flux_body(const DevCase<T> &dc, const int bx, co
 }
 
 // dynamic shared memory of a CTA of the flux pass
-template <typename T, int D, int NC, int TV, int NF> constexpr int flux_smem(int nth)
+template <typename T, int D, int NC, int TV, int NF> constexpr int flux_smem()
 {
     if constexpr (NF == 0) return 0;
-    else return nth / 32 * 2 * StagedCell<T, D, NC, TV, NF>::BYTES;
+    else return FLUX_THREADS / 32 * 2 * StagedCell<T, D, NC, TV, NF>::BYTES;
 }
 
-// 512-thread CTAs are held to 64 registers so that two fit an SM; 256-thread
-// CTAs take what ptxas chooses (108 registers for tetrahedra at TV = 4, two CTAs
-// per SM): held to 80 registers, three CTAs spill and measure 7.55 against
-// 7.12 ms on the 107k-cell tetrahedral mesh (with stage 1), 8.41 against 7.74 on
-// 24k cells x 28^3 and 1.58 against 1.52 on the 30k-cell triangulation.
-template <typename T, int D, int NC, int TV, int NF, int NTH>
-__global__ void __launch_bounds__(NTH, NTH >= 512 ? 2 : 0) k_flux(DevCase<T> dc, int chunk)
+// CTAs of four warps: 20 warps fit an SM at 96 registers (tetrahedra and
+// hexahedra, FP32 at TV = 4) and 16 at the 120 of the 2D kernels, against 16 in
+// CTAs of eight, and the last wave ends sooner.  Both kernels, 107k-cell
+// tetrahedral mesh 7.12 -> 6.59 ms (6.88 at four CTAs per SM), 24k cells x 28^3 7.73 -> 7.32,
+// 30k-cell triangulation 1.52 -> 1.47 (1.56 at five CTAs per SM, which spill in
+// 2D); CTAs of six warps 7.11, 7.84 and 1.57, of two 6.62, 7.34 and 1.55.
+template <typename T, int D, int TV> constexpr int flux_min_ctas() { return sizeof(T) == 4 && TV == 4 ? (D == 3 ? 5 : 4) : 0; }
+
+template <typename T, int D, int NC, int TV, int NF>
+__global__ void __launch_bounds__(FLUX_THREADS, flux_min_ctas<T, D, TV>()) k_flux(DevCase<T> dc, int chunk)
 {
     flux_body<T, D, NC, TV, NF>(dc, blockIdx.x, chunk);
 }
 
-template <typename T, int D, int NC, int TV, int NF, int NTH>
-__global__ void __launch_bounds__(NTH, NTH >= 512 ? 2 : 0)
+template <typename T, int D, int NC, int TV, int NF>
+__global__ void __launch_bounds__(FLUX_THREADS, flux_min_ctas<T, D, TV>())
     k_flux_batch(const DevCase<T> *__restrict__ cases, const int *__restrict__ off, int n, int chunk)
 {
     int bx;
@@ -2287,39 +2296,31 @@ __global__ void __launch_bounds__(256) k_halo_unpack(DevCase<T> dc, const int *c
 static inline int cdiv(long long a, int b) { return (int)((a + b - 1) / b); }
 
 // The two kernels of a chunk, for one case (cases == nullptr) or for those of a
-// batch (block offsets off[0..n]).  All cases of a launch share the tiling's
-// velocities per lane tv and threads nth, and the entry count nf.
-template <typename T, int D, int NC, int TV, int NF, int NTH>
+// batch (block offsets off[0..n]).  All cases of a launch share the velocities
+// per lane tv and the entry count nf.
+template <typename T, int D, int NC, int TV, int NF>
 static cudaError_t flux_launch(int blocks, int chunk, cudaStream_t st, const DevCase<T> *dc, const DevCase<T> *cases,
                                const int *off, int n)
 {
-    constexpr int smem = flux_smem<T, D, NC, TV, NF>(NTH);
+    constexpr int smem = flux_smem<T, D, NC, TV, NF>();
     if (smem > 48 * 1024) {
-        const cudaError_t e = cases ? cudaFuncSetAttribute(k_flux_batch<T, D, NC, TV, NF, NTH>,
-                                                           cudaFuncAttributeMaxDynamicSharedMemorySize, smem)
-                                    : cudaFuncSetAttribute(k_flux<T, D, NC, TV, NF, NTH>,
-                                                           cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        const cudaError_t e =
+            cases ? cudaFuncSetAttribute(k_flux_batch<T, D, NC, TV, NF>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)
+                  : cudaFuncSetAttribute(k_flux<T, D, NC, TV, NF>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (e != cudaSuccess) return e;
     }
-    if (cases) k_flux_batch<T, D, NC, TV, NF, NTH><<<blocks, NTH, smem, st>>>(cases, off, n, chunk);
-    else k_flux<T, D, NC, TV, NF, NTH><<<blocks, NTH, smem, st>>>(*dc, chunk);
+    if (cases) k_flux_batch<T, D, NC, TV, NF><<<blocks, FLUX_THREADS, smem, st>>>(cases, off, n, chunk);
+    else k_flux<T, D, NC, TV, NF><<<blocks, FLUX_THREADS, smem, st>>>(*dc, chunk);
     return cudaGetLastError();
 }
 
 template <typename T, int D, int NC, int NF>
-static cudaError_t flux_tiled(int tv, int nth, int blocks, int chunk, cudaStream_t st, const DevCase<T> *dc,
+static cudaError_t flux_tiled(int tv, int blocks, int chunk, cudaStream_t st, const DevCase<T> *dc,
                               const DevCase<T> *cases, const int *off, int n)
 {
-    if (nth == 512) {
-        if constexpr (std::is_same<T, float>::value) {
-            if (tv == 1) return flux_launch<T, D, NC, 1, NF, 512>(blocks, chunk, st, dc, cases, off, n);
-            if (tv == 2) return flux_launch<T, D, NC, 2, NF, 512>(blocks, chunk, st, dc, cases, off, n);
-        }
-        return cudaErrorInvalidValue;
-    }
-    if (tv == 1) return flux_launch<T, D, NC, 1, NF, 256>(blocks, chunk, st, dc, cases, off, n);
-    if (tv == 2) return flux_launch<T, D, NC, 2, NF, 256>(blocks, chunk, st, dc, cases, off, n);
-    if (tv == 4) return flux_launch<T, D, NC, 4, NF, 256>(blocks, chunk, st, dc, cases, off, n);
+    if (tv == 1) return flux_launch<T, D, NC, 1, NF>(blocks, chunk, st, dc, cases, off, n);
+    if (tv == 2) return flux_launch<T, D, NC, 2, NF>(blocks, chunk, st, dc, cases, off, n);
+    if (tv == 4) return flux_launch<T, D, NC, 4, NF>(blocks, chunk, st, dc, cases, off, n);
     return cudaErrorInvalidValue;
 }
 
@@ -2327,19 +2328,19 @@ static cudaError_t flux_tiled(int tv, int nth, int blocks, int chunk, cudaStream
 // tetrahedra, hexahedra; a mesh with another largest count takes the next one
 // above, one beyond MAX_NF the kernels that loop over the cells' own counts
 template <typename T>
-cudaError_t launch_flux(int D, int nf, int vtile, int nth, int blocks, int chunk, cudaStream_t st,
-                        const DevCase<T> *dc, const DevCase<T> *cases, const int *off, int n)
+cudaError_t launch_flux(int D, int nf, int vtile, int blocks, int chunk, cudaStream_t st, const DevCase<T> *dc,
+                        const DevCase<T> *cases, const int *off, int n)
 {
     const int tv = vtile / 32;
     if (blocks <= 0) return cudaSuccess;
     if (D == 2) {
-        if (nf == 3) return flux_tiled<T, 2, 2, 3>(tv, nth, blocks, chunk, st, dc, cases, off, n);
-        if (nf == 4) return flux_tiled<T, 2, 2, 4>(tv, nth, blocks, chunk, st, dc, cases, off, n);
-        return flux_tiled<T, 2, 2, 0>(tv, nth, blocks, chunk, st, dc, cases, off, n);
+        if (nf == 3) return flux_tiled<T, 2, 2, 3>(tv, blocks, chunk, st, dc, cases, off, n);
+        if (nf == 4) return flux_tiled<T, 2, 2, 4>(tv, blocks, chunk, st, dc, cases, off, n);
+        return flux_tiled<T, 2, 2, 0>(tv, blocks, chunk, st, dc, cases, off, n);
     }
-    if (nf == 4) return flux_tiled<T, 3, 1, 4>(tv, nth, blocks, chunk, st, dc, cases, off, n);
-    if (nf == 6) return flux_tiled<T, 3, 1, 6>(tv, nth, blocks, chunk, st, dc, cases, off, n);
-    return flux_tiled<T, 3, 1, 0>(tv, nth, blocks, chunk, st, dc, cases, off, n);
+    if (nf == 4) return flux_tiled<T, 3, 1, 4>(tv, blocks, chunk, st, dc, cases, off, n);
+    if (nf == 6) return flux_tiled<T, 3, 1, 6>(tv, blocks, chunk, st, dc, cases, off, n);
+    return flux_tiled<T, 3, 1, 0>(tv, blocks, chunk, st, dc, cases, off, n);
 }
 
 template <typename T, int D, int NC, int NF>
@@ -2377,7 +2378,7 @@ cudaError_t launch_stage1(int D, int nf, int blocks, int chunk, cudaStream_t st,
 template <typename T> int flux_blocks(const DevCase<T> &dc, int chunk)
 {
     const int left = dc.nvp - chunk * dc.chunk;
-    return left > 0 ? dc.n_patches * cdiv(std::min(left, dc.chunk), dc.vtile) : 0;
+    return left > 0 ? dc.n_patches * (dc.nth / FLUX_THREADS) * cdiv(std::min(left, dc.chunk), dc.vtile) : 0;
 }
 
 template <typename T> int stage1_blocks(const DevCase<T> &dc, int chunk)
@@ -2391,7 +2392,7 @@ template <typename T>
 cudaError_t launch_gather(const DevCase<T> &dc, cudaStream_t st)
 {
     for (int r = 0; r < dc.n_chunks; ++r) {
-        cudaError_t e = launch_flux<T>(dc.D, dc.nf, dc.vtile, dc.nth, flux_blocks(dc, r), r, st, &dc, nullptr, nullptr, 0);
+        cudaError_t e = launch_flux<T>(dc.D, dc.nf, dc.vtile, flux_blocks(dc, r), r, st, &dc, nullptr, nullptr, 0);
         if (e == cudaSuccess)
             e = launch_stage1<T>(dc.D, dc.nf, stage1_blocks(dc, r), r, st, &dc, nullptr, nullptr, 0);
         if (e != cudaSuccess) return e;
@@ -2702,7 +2703,7 @@ template cudaError_t launch_small_batch<double>(int, int, const DevCase<double> 
 template cudaError_t launch_small_batch<float>(int, int, const DevCase<float> *, const int *, int, int, int, size_t,
                                                cudaStream_t);
 #define UGKS_GATHER(T)                                                                                        \
-    template cudaError_t launch_flux<T>(int, int, int, int, int, int, cudaStream_t, const DevCase<T> *,       \
+    template cudaError_t launch_flux<T>(int, int, int, int, int, cudaStream_t, const DevCase<T> *,            \
                                         const DevCase<T> *, const int *, int);                                \
     template cudaError_t launch_stage1<T>(int, int, int, int, cudaStream_t, const DevCase<T> *,               \
                                           const DevCase<T> *, const int *, int);                              \

@@ -16,12 +16,11 @@ template <typename T> cudaError_t launch_pre_gather(const DevCase<T> &dc, cudaSt
 // the flux and stage-1 passes over all chunks of a case
 template <typename T> cudaError_t launch_gather(const DevCase<T> &dc, cudaStream_t st);
 // one chunk's flux or stage-1 kernel, for one case (dc) or for n cases in one
-// launch: cases[] a device array of their DevCase with the same D, nf, vtile and
-// threads per CTA, off[0..n] the device prefix sums of their block counts,
-// blocks = off[n]
+// launch: cases[] a device array of their DevCase with the same D, nf and vtile,
+// off[0..n] the device prefix sums of their block counts, blocks = off[n]
 template <typename T>
-cudaError_t launch_flux(int D, int nf, int vtile, int nth, int blocks, int chunk, cudaStream_t st,
-                        const DevCase<T> *dc, const DevCase<T> *cases, const int *off, int n);
+cudaError_t launch_flux(int D, int nf, int vtile, int blocks, int chunk, cudaStream_t st, const DevCase<T> *dc,
+                        const DevCase<T> *cases, const int *off, int n);
 template <typename T>
 cudaError_t launch_stage1(int D, int nf, int blocks, int chunk, cudaStream_t st, const DevCase<T> *dc,
                           const DevCase<T> *cases, const int *off, int n);
