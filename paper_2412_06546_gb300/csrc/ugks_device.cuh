@@ -1043,7 +1043,7 @@ template <typename T, int D, typename P>
 __device__ __forceinline__ P poly_eval(const T *__restrict__ a, const P (&c)[D], const P c2)
 {
     constexpr int NB = Poly<D>::NB;
-    P p = pbc<P>(a[0]), q, g;
+    P p = pbc<P>(a[0]);
     if constexpr (std::is_same<T, double>::value) {
 #pragma unroll
         for (int e = 0; e < D; ++e) {
@@ -1053,17 +1053,20 @@ __device__ __forceinline__ P poly_eval(const T *__restrict__ a, const P (&c)[D],
             p = pfma(r, c[e], p);
         }
         return p;
-    }
+    } else {
+        P q, g;
 #pragma unroll
-    for (int e = 0; e < D; ++e) {
-        p = pfma(pbc<P>(a[1 + e]), c[e], p);
-        P r = pmul(pbc<P>(a[1 + D + (e * (2 * D - e + 1)) / 2]), c[e]);
+        for (int e = 0; e < D; ++e) {
+            p = pfma(pbc<P>(a[1 + e]), c[e], p);
+            P r = pmul(pbc<P>(a[1 + D + (e * (2 * D - e + 1)) / 2]), c[e]);
 #pragma unroll
-        for (int f = e + 1; f < D; ++f) r = pfma(pbc<P>(a[1 + D + (e * (2 * D - e + 1)) / 2 + (f - e)]), c[f], r);
-        q = e == 0 ? pmul(r, c[0]) : pfma(r, c[e], q);
-        g = e == 0 ? pmul(pbc<P>(a[1 + D + NB]), c[0]) : pfma(pbc<P>(a[1 + D + NB + e]), c[e], g);
+            for (int f = e + 1; f < D; ++f)
+                r = pfma(pbc<P>(a[1 + D + (e * (2 * D - e + 1)) / 2 + (f - e)]), c[f], r);
+            q = e == 0 ? pmul(r, c[0]) : pfma(r, c[e], q);
+            g = e == 0 ? pmul(pbc<P>(a[1 + D + NB]), c[0]) : pfma(pbc<P>(a[1 + D + NB + e]), c[e], g);
+        }
+        return pfma(g, c2, padd(p, q));
     }
-    return pfma(g, c2, padd(p, q));
 }
 
 }  // namespace ugks

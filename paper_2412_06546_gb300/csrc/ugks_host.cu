@@ -745,16 +745,17 @@ int kDefaultVtile(int prec) { return prec == UGKS_FP64 ? 32 : 64; }
 // A warp of stage 1 ends its group of velocities with a reduction over its lanes
 // that costs as much as about 250 velocities of the pass itself: groups of 1024,
 // fewer where the mesh has too few cells to fill the chip with one warp per cell
-// and group, or where the flux buffer of a group would exceed a copy of f.  (The
+// and group, or where the flux buffer of a group would exceed 9/8 of a copy of f.  (The
 // 107k-cell tetrahedral mesh x 4,568 velocities in FP32, flux and stage-1 passes:
 // 9.10, 8.30 and 7.95 ms at 256, 512 and 1024.)  The buffer holds as many
-// groups as fit 64 MB or a copy of f, whichever is smaller (4 MB are always
-// taken): fewer launches for small cases, little memory for large ones.
+// groups as fit 64 MB or 9/8 of a copy of f, whichever is smaller (4 MB are always
+// taken): fewer launches for small cases (the 1/8 lets quadrilaterals, 2.1 faces
+// per cell, do with two chunks), little memory for large ones.
 void set_chunks(ugks_case *c, int tile_group)
 {
     const int nvp = (int)c->nvp;
     const size_t per_vel = (size_t)std::max<int64_t>(c->F, 1) * c->NC * (c->prec == UGKS_FP64 ? 8 : 4);
-    const size_t most = std::max((size_t)c->f_bytes, (size_t)4 << 20);
+    const size_t most = std::max((size_t)c->f_bytes + c->f_bytes / 8, (size_t)4 << 20);
     const int64_t warps = 152 * 32;
     int groups = (nvp + 1023) / 1024, step = 128;
     auto vel = [&] { return ((nvp + groups - 1) / groups + step - 1) / step * step; };
@@ -1395,8 +1396,11 @@ struct ugks_batch {
         int vtile = 0, nf = 0, n_chunks = 0;
         int *off = nullptr;                  // [n_chunks][2][n + 1]
         std::vector<int> blocks;             // [n_chunks][2]
+        cudaStream_t branch = nullptr;       // capture stream of the group's branch (but the first's)
+        cudaEvent_t join = nullptr;
     };
     std::vector<Group> groups;
+    cudaEvent_t fork = nullptr;
     // the other kernels of a step, one launch each over all cases: block offsets
     // off[k][0..n] (device, prefix sums of the cases' block counts), total
     // blocks and dynamic shared memory per kernel
@@ -1468,6 +1472,10 @@ void batch_build(ugks_batch *b)
             }
         cuda_ok(cudaMalloc((void **)&g.off, goff.size() * sizeof(int)), "batch alloc");
         b->groups.push_back(g);      // owned by the batch from here on
+        if (b->groups.size() > 1) {
+            cuda_ok(cudaStreamCreateWithFlags(&b->groups.back().branch, cudaStreamNonBlocking), "branch stream");
+            cuda_ok(cudaEventCreateWithFlags(&b->groups.back().join, cudaEventDisableTiming), "branch event");
+        }
         cuda_ok(cudaMemcpy(g.off, goff.data(), goff.size() * sizeof(int), cudaMemcpyHostToDevice), "batch upload");
     }
 }
@@ -1485,14 +1493,25 @@ void batch_capture(ugks_batch *b)
     };
     cuda_ok(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal), "begin capture");
     for (int k = ugks::SK_PREP; k <= ugks::SK_WALL_SUM; ++k) small(k);
-    for (const auto &g : b->groups)
+    // the groups' passes touch different cases: branches of the graph, so that the
+    // last blocks of one run beside the first of another
+    cuda_ok(cudaEventRecord(b->fork, st), "fork");
+    for (size_t gi = 0; gi < b->groups.size(); ++gi) {
+        const auto &g = b->groups[gi];
+        cudaStream_t sg = gi == 0 ? st : g.branch;
+        if (gi > 0) cuda_ok(cudaStreamWaitEvent(sg, b->fork, 0), "fork");
         for (int r = 0; r < g.n_chunks; ++r) {
             const int *off = g.off + (size_t)r * 2 * (n + 1);
-            cuda_ok(ugks::launch_flux<T>(b->D, g.nf, g.vtile, g.blocks[2 * r], r, st, nullptr, dcs, off, n),
+            cuda_ok(ugks::launch_flux<T>(b->D, g.nf, g.vtile, g.blocks[2 * r], r, sg, nullptr, dcs, off, n),
                     "batched flux pass");
-            cuda_ok(ugks::launch_stage1<T>(b->D, g.nf, g.blocks[2 * r + 1], r, st, nullptr, dcs, off + n + 1, n),
+            cuda_ok(ugks::launch_stage1<T>(b->D, g.nf, g.blocks[2 * r + 1], r, sg, nullptr, dcs, off + n + 1, n),
                     "batched stage 1");
         }
+        if (gi > 0) {
+            cuda_ok(cudaEventRecord(g.join, sg), "join");
+            cuda_ok(cudaStreamWaitEvent(st, g.join, 0), "join");
+        }
+    }
     small(ugks::SK_UPDATE_W);
     small(ugks::SK_COLLIDE);
     cuda_ok(cudaStreamEndCapture(st, &b->graph), "end capture");
@@ -1505,12 +1524,16 @@ void batch_free(ugks_batch *b)
     if (b->exec) cudaGraphExecDestroy(b->exec);
     if (b->graph) cudaGraphDestroy(b->graph);
     if (b->dcases) cudaFree(b->dcases);
-    for (auto &g : b->groups)
-        if (g.off) cudaFree(g.off);
+    for (auto &g : b->groups) {
+            if (g.off) cudaFree(g.off);
+            if (g.join) cudaEventDestroy(g.join);
+            if (g.branch) cudaStreamDestroy(g.branch);
+        }
     if (b->small_off) cudaFree(b->small_off);
     for (auto e : b->case_ev)
         if (e) cudaEventDestroy(e);
     if (b->done) cudaEventDestroy(b->done);
+    if (b->fork) cudaEventDestroy(b->fork);
     if (b->own_stream && b->stream) cudaStreamDestroy(b->stream);
 }
 
@@ -1545,6 +1568,7 @@ ugks_status ugks_batch_create(ugks_case *const *cases, int32_t n, void *stream, 
             b->own_stream = true;
         }
         cuda_ok(cudaEventCreateWithFlags(&b->done, cudaEventDisableTiming), "event");
+        cuda_ok(cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming), "event");
         b->case_ev.assign(b->cases.size(), nullptr);
         for (auto &e : b->case_ev) cuda_ok(cudaEventCreateWithFlags(&e, cudaEventDisableTiming), "event");
         // the cases' own streams must have finished their queued work
