@@ -132,6 +132,36 @@ __device__ __forceinline__ void time_integrals(double dt, double x, double q[5])
     }
 }
 
+// ------------------------------------------------------------ launches
+// The kernels of a step are launched with programmatic stream serialisation: a
+// kernel is set up while the one before it drains, and waits here, before its
+// first access to what that one wrote, until the one before has ended and its
+// writes are visible.  Every kernel of the step waits, so the order of the whole
+// step is kept.  Step times on 13 and more kernels: 20x20 squares x 24^2 119 ->
+// 88 us, 2,183 triangles x 30x25 153 -> 117, 2,145 hexahedra x 4,080 446 -> 405.
+// Releasing the next kernel's blocks earlier (launch_dependents at a kernel's
+// start) was slower, 95, 123 and 416 us: they take the SMs' slots to wait in.
+__device__ __forceinline__ void dependency_wait()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+template <typename... P, typename... A>
+static cudaError_t launch(void (*kernel)(P...), int blocks, int threads, size_t smem, cudaStream_t st, const A &...args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)blocks);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
 // ------------------------------------------------------------ batched launches
 // The per-case kernels of a step (all but the gather) are written as bodies of
 // a block index.  k_X runs them for one case (block index = blockIdx.x);
@@ -257,6 +287,7 @@ __device__ __forceinline__ void prep_body(const DevCase<T> &dc, const int bx)
 template <typename T, int D, int NC>
 __global__ void k_prep(DevCase<T> dc)
 {
+    dependency_wait();
     prep_body<T, D, NC>(dc, blockIdx.x);
 }
 
@@ -265,6 +296,7 @@ __global__ void k_prep_batch(const DevCase<T> *__restrict__ cases, const int *__
 {
     int bx;
     const DevCase<T> &dc = batch_case(cases, off, n, bx);
+    dependency_wait();
     prep_body<T, D, NC>(dc, bx);
 }
 
@@ -358,6 +390,7 @@ __device__ __forceinline__ void macro_grad_body(const DevCase<T> &dc, const int 
 template <typename T, int D, int NC>
 __global__ void k_macro_grad(DevCase<T> dc)
 {
+    dependency_wait();
     macro_grad_body<T, D, NC>(dc, blockIdx.x);
 }
 
@@ -366,6 +399,7 @@ __global__ void k_macro_grad_batch(const DevCase<T> *__restrict__ cases, const i
 {
     int bx;
     const DevCase<T> &dc = batch_case(cases, off, n, bx);
+    dependency_wait();
     macro_grad_body<T, D, NC>(dc, bx);
 }
 
@@ -484,6 +518,7 @@ __device__ __forceinline__ void face_pre_body(const DevCase<T> &dc, const int bx
 template <typename T, int D, int NC>
 __global__ void k_face_pre(DevCase<T> dc)
 {
+    dependency_wait();
     face_pre_body<T, D, NC>(dc, blockIdx.x);
 }
 
@@ -492,6 +527,7 @@ __global__ void k_face_pre_batch(const DevCase<T> *__restrict__ cases, const int
 {
     int bx;
     const DevCase<T> &dc = batch_case(cases, off, n, bx);
+    dependency_wait();
     face_pre_body<T, D, NC>(dc, bx);
 }
 
@@ -577,6 +613,7 @@ __device__ __forceinline__ void face_sum1_body(const DevCase<T> &dc, const int b
 template <typename T, int D, int NC>
 __global__ void k_face_sum1(DevCase<T> dc)
 {
+    dependency_wait();
     face_sum1_body<T, D, NC>(dc, blockIdx.x);
 }
 
@@ -585,6 +622,7 @@ __global__ void k_face_sum1_batch(const DevCase<T> *__restrict__ cases, const in
 {
     int bx;
     const DevCase<T> &dc = batch_case(cases, off, n, bx);
+    dependency_wait();
     face_sum1_body<T, D, NC>(dc, bx);
 }
 
@@ -742,6 +780,7 @@ __device__ __forceinline__ void face_sum1_sep_body(const DevCase<T> &dc, const i
 template <typename T, int D, int NC>
 __global__ void __launch_bounds__(32 * SUM1_SEP_WARPS) k_face_sum1_sep(DevCase<T> dc)
 {
+    dependency_wait();
     face_sum1_sep_body<T, D, NC>(dc, blockIdx.x);
 }
 
@@ -750,6 +789,7 @@ __global__ void __launch_bounds__(32 * SUM1_SEP_WARPS) k_face_sum1_sep_batch(con
 {
     int bx;
     const DevCase<T> &dc = batch_case(cases, off, n, bx);
+    dependency_wait();
     face_sum1_sep_body<T, D, NC>(dc, bx);
 }
 
@@ -787,6 +827,7 @@ __device__ __forceinline__ void face_fin1_body(const DevCase<T> &dc, const int b
 template <typename T, int D, int NC>
 __global__ void k_face_fin1(DevCase<T> dc)
 {
+    dependency_wait();
     face_fin1_body<T, D, NC>(dc, blockIdx.x);
 }
 
@@ -795,6 +836,7 @@ __global__ void k_face_fin1_batch(const DevCase<T> *__restrict__ cases, const in
 {
     int bx;
     const DevCase<T> &dc = batch_case(cases, off, n, bx);
+    dependency_wait();
     face_fin1_body<T, D, NC>(dc, bx);
 }
 
@@ -980,6 +1022,7 @@ __device__ __forceinline__ void face_sum2_body(const DevCase<T> &dc, const int b
 template <typename T, int D, int NC>
 __global__ void k_face_sum2(DevCase<T> dc)
 {
+    dependency_wait();
     face_sum2_body<T, D, NC>(dc, blockIdx.x);
 }
 
@@ -988,6 +1031,7 @@ __global__ void k_face_sum2_batch(const DevCase<T> *__restrict__ cases, const in
 {
     int bx;
     const DevCase<T> &dc = batch_case(cases, off, n, bx);
+    dependency_wait();
     face_sum2_body<T, D, NC>(dc, bx);
 }
 
@@ -1051,6 +1095,7 @@ __device__ __forceinline__ void face_sum2_sep_body(const DevCase<T> &dc, const i
 template <typename T, int D, int NC>
 __global__ void k_face_sum2_sep(DevCase<T> dc)
 {
+    dependency_wait();
     face_sum2_sep_body<T, D, NC>(dc, blockIdx.x);
 }
 
@@ -1059,6 +1104,7 @@ __global__ void k_face_sum2_sep_batch(const DevCase<T> *__restrict__ cases, cons
 {
     int bx;
     const DevCase<T> &dc = batch_case(cases, off, n, bx);
+    dependency_wait();
     face_sum2_sep_body<T, D, NC>(dc, bx);
 }
 
@@ -1290,6 +1336,7 @@ __device__ __forceinline__ void face_fin2_body(const DevCase<T> &dc, const int b
 template <typename T, int D, int NC>
 __global__ void k_face_fin2(DevCase<T> dc)
 {
+    dependency_wait();
     face_fin2_body<T, D, NC>(dc, blockIdx.x);
 }
 
@@ -1298,6 +1345,7 @@ __global__ void k_face_fin2_batch(const DevCase<T> *__restrict__ cases, const in
 {
     int bx;
     const DevCase<T> &dc = batch_case(cases, off, n, bx);
+    dependency_wait();
     face_fin2_body<T, D, NC>(dc, bx);
 }
 
@@ -1441,6 +1489,7 @@ __device__ __forceinline__ void wall_sum_body(const DevCase<T> &dc, const int bx
 template <typename T, int D, int NC>
 __global__ void __launch_bounds__(256) k_wall_sum(DevCase<T> dc)
 {
+    dependency_wait();
     wall_sum_body<T, D, NC>(dc, blockIdx.x);
 }
 
@@ -1449,6 +1498,7 @@ __global__ void __launch_bounds__(256) k_wall_sum_batch(const DevCase<T> *__rest
 {
     int bx;
     const DevCase<T> &dc = batch_case(cases, off, n, bx);
+    dependency_wait();
     wall_sum_body<T, D, NC>(dc, bx);
 }
 
@@ -1745,6 +1795,7 @@ template <typename T, int D, int TV> constexpr int flux_min_ctas() { return size
 template <typename T, int D, int NC, int TV, int NF>
 __global__ void __launch_bounds__(FLUX_THREADS, flux_min_ctas<T, D, TV>()) k_flux(DevCase<T> dc, int chunk)
 {
+    dependency_wait();
     flux_body<T, D, NC, TV, NF>(dc, blockIdx.x, chunk);
 }
 
@@ -1754,6 +1805,7 @@ __global__ void __launch_bounds__(FLUX_THREADS, flux_min_ctas<T, D, TV>())
 {
     int bx;
     const DevCase<T> &dc = batch_case(cases, off, n, bx);
+    dependency_wait();
     flux_body<T, D, NC, TV, NF>(dc, bx, chunk);
 }
 
@@ -1961,6 +2013,7 @@ __device__ __forceinline__ void stage1_body(const DevCase<T> &dc, const int bx, 
 template <typename T, int D, int NC, int NF>
 __global__ void __launch_bounds__(256) k_stage1(DevCase<T> dc, int chunk)
 {
+    dependency_wait();
     stage1_body<T, D, NC, NF>(dc, blockIdx.x, chunk);
 }
 
@@ -1970,6 +2023,7 @@ __global__ void __launch_bounds__(256) k_stage1_batch(const DevCase<T> *__restri
 {
     int bx;
     const DevCase<T> &dc = batch_case(cases, off, n, bx);
+    dependency_wait();
     stage1_body<T, D, NC, NF>(dc, bx, chunk);
 }
 
@@ -2011,6 +2065,7 @@ __device__ __forceinline__ void update_W_body(const DevCase<T> &dc, const int bx
 template <typename T, int D, int NC>
 __global__ void __launch_bounds__(256) k_update_W(DevCase<T> dc)
 {
+    dependency_wait();
     update_W_body<T, D, NC>(dc, blockIdx.x);
 }
 
@@ -2019,6 +2074,7 @@ __global__ void __launch_bounds__(256) k_update_W_batch(const DevCase<T> *__rest
 {
     int bx;
     const DevCase<T> &dc = batch_case(cases, off, n, bx);
+    dependency_wait();
     update_W_body<T, D, NC>(dc, bx);
 }
 
@@ -2177,6 +2233,7 @@ __device__ __forceinline__ void collide_body(const DevCase<T> &dc, const int bx)
 template <typename T, int D, int NC>
 __global__ void __launch_bounds__(256, sizeof(T) == 4 && D == 2 ? 4 : 0) k_collide(DevCase<T> dc)
 {
+    dependency_wait();
     collide_body<T, D, NC>(dc, blockIdx.x);
 }
 
@@ -2186,6 +2243,7 @@ __global__ void __launch_bounds__(256) k_collide_batch(const DevCase<T> *__restr
 {
     int bx;
     const DevCase<T> &dc = batch_case(cases, off, n, bx);
+    dependency_wait();
     collide_body<T, D, NC>(dc, bx);
 }
 
@@ -2365,9 +2423,8 @@ static cudaError_t flux_launch(int blocks, int chunk, cudaStream_t st, const Dev
                   : cudaFuncSetAttribute(k_flux<T, D, NC, TV, NF>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (e != cudaSuccess) return e;
     }
-    if (cases) k_flux_batch<T, D, NC, TV, NF><<<blocks, FLUX_THREADS, smem, st>>>(cases, off, n, chunk);
-    else k_flux<T, D, NC, TV, NF><<<blocks, FLUX_THREADS, smem, st>>>(*dc, chunk);
-    return cudaGetLastError();
+    return cases ? launch(k_flux_batch<T, D, NC, TV, NF>, blocks, FLUX_THREADS, smem, st, cases, off, n, chunk)
+                 : launch(k_flux<T, D, NC, TV, NF>, blocks, FLUX_THREADS, smem, st, *dc, chunk);
 }
 
 template <typename T, int D, int NC, int NF>
@@ -2411,9 +2468,8 @@ static cudaError_t stage1_launch(int blocks, int chunk, cudaStream_t st, const D
                                                            cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (e != cudaSuccess) return e;
     }
-    if (cases) k_stage1_batch<T, D, NC, NF><<<blocks, 256, smem, st>>>(cases, off, n, chunk);
-    else k_stage1<T, D, NC, NF><<<blocks, 256, smem, st>>>(*dc, chunk);
-    return cudaGetLastError();
+    return cases ? launch(k_stage1_batch<T, D, NC, NF>, blocks, 256, smem, st, cases, off, n, chunk)
+                 : launch(k_stage1<T, D, NC, NF>, blocks, 256, smem, st, *dc, chunk);
 }
 
 template <typename T>
@@ -2532,9 +2588,8 @@ static cudaError_t sk_launch(int k, int blocks, int nt, size_t smem, cudaStream_
     if (blocks <= 0) return cudaSuccess;
 #define UGKS_SK(ID, K)                                                                                  \
     case ID:                                                                                            \
-        if (cases) K##_batch<T, D, NC><<<blocks, nt, smem, st>>>(cases, off, n);                        \
-        else K<T, D, NC><<<blocks, nt, smem, st>>>(*dc);                                                \
-        break;
+        return cases ? launch(K##_batch<T, D, NC>, blocks, nt, smem, st, cases, off, n)                 \
+                     : launch(K<T, D, NC>, blocks, nt, smem, st, *dc);
     if (k == SK_FACE_SUM1_SEP && smem > 48 * 1024) {
         cudaError_t e = cases ? cudaFuncSetAttribute(k_face_sum1_sep_batch<T, D, NC>,
                                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)
@@ -2558,7 +2613,6 @@ static cudaError_t sk_launch(int k, int blocks, int nt, size_t smem, cudaStream_
     default: return cudaErrorInvalidValue;
     }
 #undef UGKS_SK
-    return cudaGetLastError();
 }
 
 template <typename T, int D, int NC>
