@@ -36,10 +36,10 @@ CYLINDER = "cylinder_Ma5_Kn0.1_tri30k_v60x50"
 E2E_MAX_BYTES = 32e9      # largest host copy of f the e2e leg stages in pinned memory
 LARGE_CVU = 2e9           # cases above this many cell-velocities get a fixed FP64 tiling
 X38_SMALL_H0 = 0.2        # first layer of the X38-like mesh for the ~100k-cell profiling instance
-# gather tiling (patch cells, velocity tile, threads per CTA, tile group) of the benchmark's workloads:
-# the autotuner's choice on GB300 (it varies between near-equal tile groups from run to run), fixed so
-# that the committed ncu traffic figure applies and no trial launches run before the timed steps
-BENCH_TILING = {WORKLOAD: (48, 64, 512, 64), CYLINDER: (48, 64, 512, 8)}
+# tiling of the flux pass (patch cells, velocity tile, threads per patch, tile group) of the benchmark's
+# workloads: the autotuner's choice on GB300, fixed so that the committed ncu traffic figure applies and
+# no trial launches run before the timed steps
+BENCH_TILING = {WORKLOAD: (64, 128, 256, 8), CYLINDER: (64, 128, 256, 8)}
 
 
 def _peaks():
@@ -526,9 +526,9 @@ def main():
     ap.add_argument("--no-serving", action="store_true")
     ap.add_argument("--patch", type=int, default=0)
     ap.add_argument("--vtile", type=int, default=0)
-    ap.add_argument("--threads", type=int, default=0, help="gather CTA size, 256 or 512 (0: autotuned)")
+    ap.add_argument("--threads", type=int, default=0, help="threads per patch of the flux pass, 256 or 512 (0: 256)")
     ap.add_argument("--tile-group", type=int, default=0,
-                    help="velocity tiles per group of the gather grid order (0: autotuned)")
+                    help="velocity tiles per moment group of stage 1 (0: from the sizes of the case)")
     ap.add_argument("--w0-analytic", action="store_true",
                     help="interface W0 from the analytic half-range moments (the variant of the N4 row)")
     args = ap.parse_args()
