@@ -110,8 +110,9 @@ typedef struct {
                                vtile <= 64; 0: 256), in CTAs of 128 */
     int32_t gather_tile_group; /* velocity tiles per moment group of stage 1: the moments of a cell's flux
                                residual are summed over groups of this many tiles, the groups in FP64
-                               (1 .. 1024, larger values are clamped to the number of tiles, and to what
-                               the flux buffer may hold; 0: chosen from the sizes of the case) */
+                               (1 .. 1024, larger values are clamped to the number of tiles; 0: chosen
+                               from the velocity count where patch_cells is given, else from the sizes of
+                               the case) */
     int32_t w0_analytic;    /* interface equilibrium W0 (Sec. 2.4) from: 0 the discrete half-range
                                sums over the velocity set (default), 1 the analytic half-range
                                moments of the face-state Maxwellians over the continuous velocity
@@ -309,7 +310,9 @@ void ugks_server_destroy(ugks_server *s);
  * slopes of the face neighbours, whose limited gradients read the second
  * ring), with every face of its own cells and of the first ring.  One step of
  * the subdomain updates its own cells exactly as a step of the whole mesh
- * would, given the same time step; the halo's values come out wrong and are
+ * would, given the same time step and a fixed tiling (the same patch_cells,
+ * vtile and gather_tile_group; automatic ones depend on the size of the case
+ * and change the order of the moment sums); the halo's values come out wrong and are
  * replaced before the next step by the owners' values (f^{n+1}, W^{n+1} and the
  * heat flux q^{n+1}): pack the cells another subdomain needs into a device
  * buffer, move the buffer (a device copy on one GPU, NCCL send/receive or a

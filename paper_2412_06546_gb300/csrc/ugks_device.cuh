@@ -154,9 +154,29 @@ struct DevCase {
     // tiling of the flux and stage-1 passes
     int P, n_patches, vtile;      // cells per patch and velocities per warp of the flux pass
     int nth;                      // threads per patch (256, or 512 for FP32 at vtile <= 64), in CTAs of 128
-    int chunk, n_chunks;          // velocities per chunk (a multiple of gvel), chunks
-    int gvel, n_groups;           // velocities of a cell per warp of stage 1 (a multiple of vtile), groups per cell
+    int chunk, n_chunks;          // velocities per chunk, chunks (see chunk_span)
+    int gvel, n_groups;           // velocities of a cell per warp of stage 1, groups per cell
+    int parts;                    // chunks per group: 1 (a chunk holds one group or several), or more
+    T *carry;                     // parts > 1: lane sums of a group between its chunks, [C][D+2][32] of MomentSum
 };
+
+// First velocity of chunk r and the number of its velocities (<= 0: the case
+// has no such chunk).  A chunk holds whole groups of gvel velocities, or, where
+// the flux buffer cannot hold a group, is one of the parts of a group (multiples
+// of 128 velocities, so that a lane of stage 1 keeps its velocities).
+template <typename T>
+__host__ __device__ __forceinline__ void chunk_span(const DevCase<T> &dc, int r, int &kb, int &len)
+{
+    kb = r * dc.chunk;
+    int end = kb + dc.chunk;
+    if (dc.parts > 1) {
+        const int g = r / dc.parts;
+        kb += g * (dc.gvel - dc.parts * dc.chunk);
+        end = kb + dc.chunk < (g + 1) * dc.gvel ? kb + dc.chunk : (g + 1) * dc.gvel;
+    }
+    if (end > dc.nvp) end = dc.nvp;
+    len = end - kb;
+}
 
 // ------------------------------------------------------------------ math
 // 2^x with the hardware approximation (relative error ~2^-22); FP32 only

@@ -60,7 +60,7 @@ struct ugks_case {
     ugks::DevCase<double> d64{};
     ugks::DevCase<float> d32{};
     int P = 0, vtile = 0, nth = 256, n_patches = 0, vt_group = 1;
-    int nf = 0, gvel = 0, n_groups = 1, chunk = 0, n_chunks = 1;
+    int nf = 0, gvel = 0, n_groups = 1, chunk = 0, n_chunks = 1, parts = 1;
     long long *perm_d = nullptr;   // caller cell i -> internal cell
     std::vector<long long> perm_h; // the same on the host
     std::vector<long long> wall_face_h;   // face id of every wall slot
@@ -512,6 +512,13 @@ std::vector<T> cast(const std::vector<double> &v)
     return std::vector<T>(v.begin(), v.end());
 }
 
+// lane sums of stage 1 between the chunks of a group (DevCase::carry): per cell,
+// moment and lane 16 bytes (two pairs) in the FP32 form, 8 in the FP64 form
+size_t carry_bytes(const ugks_case *c)
+{
+    return (size_t)c->C * (c->D + 2) * 32 * (c->prec == UGKS_FP64 ? 8 : 16);
+}
+
 template <typename T>
 void fill_case(ugks_case *c, ugks::DevCase<T> &dc, const ugks_mesh *m, const ugks_vgrid *v, const ugks_params *p,
                const Host &h)
@@ -728,6 +735,8 @@ void fill_case(ugks_case *c, ugks::DevCase<T> &dc, const ugks_mesh *m, const ugk
     dc.n_groups = c->n_groups;
     dc.chunk = c->chunk;
     dc.n_chunks = c->n_chunks;
+    dc.parts = c->parts;
+    dc.carry = c->parts > 1 ? (T *)c->dalloc(carry_bytes(c)) : nullptr;
     dc.P = c->P;
     dc.nth = c->nth;
     dc.n_patches = c->n_patches;
@@ -751,7 +760,12 @@ int kDefaultVtile(int prec) { return prec == UGKS_FP64 ? 32 : 64; }
 // groups as fit 64 MB or 9/8 of a copy of f, whichever is smaller (4 MB are always
 // taken): fewer launches for small cases (the 1/8 lets quadrilaterals, 2.1 faces
 // per cell, do with two chunks), little memory for large ones.
-void set_chunks(ugks_case *c, int tile_group)
+// With a tiling of the caller's (patch_cells or the group given) the group depends on
+// the velocities alone, so that a cell's moments are summed alike on any mesh that
+// holds it, a subdomain's or the whole one.  Where the fluxes of such a group exceed
+// 9/8 of a copy of f by more than the lane sums that stage 1 then keeps
+// (carry_bytes), it is cut into several chunks.
+void set_chunks(ugks_case *c, int tile_group, bool fixed)
 {
     const int nvp = (int)c->nvp;
     const size_t per_vel = (size_t)std::max<int64_t>(c->F, 1) * c->NC * (c->prec == UGKS_FP64 ? 8 : 4);
@@ -759,14 +773,19 @@ void set_chunks(ugks_case *c, int tile_group)
     const int64_t warps = 152 * 32;
     int groups = (nvp + 1023) / 1024, step = 128;
     auto vel = [&] { return ((nvp + groups - 1) / groups + step - 1) / step * step; };
-    while (vel() > step && (c->C * groups < warps || vel() * per_vel > most)) ++groups;
+    while (!fixed && vel() > step && (c->C * groups < warps || vel() * per_vel > most)) ++groups;
     c->gvel = std::min(vel(), nvp);
-    if (tile_group > 0) {
-        // the caller's group, as far as the buffer may hold it
-        const int64_t fit = std::max<int64_t>(1, (int64_t)(most / (per_vel * c->vtile)));
-        c->gvel = (int)std::min<int64_t>(std::min(tile_group, nvp / c->vtile), fit) * c->vtile;
-    }
+    if (tile_group > 0) c->gvel = (int)std::min<int64_t>((int64_t)tile_group * c->vtile, nvp);
     c->n_groups = (nvp + c->gvel - 1) / c->gvel;
+    if (fixed && c->gvel > 128 && per_vel * c->gvel > most + carry_bytes(c)) {
+        const int fit = (int)std::max<size_t>(1, most / (per_vel * 128)) * 128;
+        c->parts = (c->gvel + fit - 1) / fit;
+        c->chunk = ((c->gvel + c->parts - 1) / c->parts + 127) / 128 * 128;
+        c->parts = (c->gvel + c->chunk - 1) / c->chunk;
+        const int last = nvp - (c->n_groups - 1) * c->gvel;
+        c->n_chunks = (c->n_groups - 1) * c->parts + (last + c->chunk - 1) / c->chunk;
+        return;
+    }
     const size_t in = std::max<size_t>(1, std::min(most, (size_t)64 << 20) / (per_vel * c->gvel));
     c->n_chunks = (int)((c->n_groups + in - 1) / in);
     c->chunk = std::min((c->n_groups + c->n_chunks - 1) / c->n_chunks * c->gvel, nvp);
@@ -1012,7 +1031,7 @@ ugks_status ugks_create(const ugks_mesh *mesh, const ugks_vgrid *vgrid, const ug
         c->n_patches = (int)((c->C + c->P - 1) / c->P);
         c->nvp = (c->Nv + vpad - 1) / vpad * vpad;
         c->f_bytes = (size_t)c->C * c->NC * c->nvp * (c->prec == UGKS_FP64 ? 8 : 4);
-        set_chunks(c.get(), params->gather_tile_group);
+        set_chunks(c.get(), params->gather_tile_group, params->patch_cells > 0 || params->gather_tile_group > 0);
         c->G = (int)h.gface.size();
         c->NW = (int)h.wface.size();
         // upwind CFL bound (the CFL step of Algorithm 1)
@@ -1033,9 +1052,7 @@ ugks_status ugks_create(const ugks_mesh *mesh, const ugks_vgrid *vgrid, const ug
                 autotune(c.get(), dc, params->vtile == 0);
                 cuda_ok(ugks::launch_init(dc, c->stream), "init");
             }
-            c->vt_group = params->gather_tile_group > 0
-                              ? (int)std::min<int64_t>(params->gather_tile_group, c->nvp / c->vtile)
-                              : std::max(1, c->gvel / c->vtile);
+            c->vt_group = (c->gvel + c->vtile - 1) / c->vtile;
         });
         cuda_ok(c->stream ? cudaStreamSynchronize(c->stream) : cudaDeviceSynchronize(), "create sync");
     });

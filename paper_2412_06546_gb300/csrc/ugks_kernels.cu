@@ -1568,9 +1568,11 @@ __device__ __forceinline__ void flux_body(const DevCase<T> &dc, const int bx, co
     const int warp = mine + (bx - tile * ncta - p * split) * (FLUX_THREADS / 32);   // on the patch
     // the lane's first velocity in the chunk and of all; the last tile may be
     // short: its lanes beyond the end repeat the tile's start and store nothing
+    int kb, kn;
+    chunk_span(dc, chunk, kb, kn);
     const int kl = tile * V + TV * lane;
-    const bool live = kl < dc.chunk && chunk * dc.chunk + kl < dc.nvp;
-    const int kc = live ? kl : tile * V, k = chunk * dc.chunk + kc;
+    const bool live = kl < kn;
+    const int kc = live ? kl : tile * V, k = kb + kc;
     const unsigned all = live ? (1u << TV) - 1 : 0u;
     const int cb = p * dc.P, ce = min(dc.C, cb + dc.P);
     const T *__restrict__ fl = dc.f_cur + k;
@@ -1828,6 +1830,9 @@ template <> struct MomentSum<double> {
     double s;
     __device__ __forceinline__ void zero() { s = 0.0; }
     __device__ __forceinline__ void add(double x, double) { s = __dadd_rn(s, x); }
+    // between the chunks of a group: slot i of the carry buffer
+    __device__ __forceinline__ void load(const double *carry, size_t i) { s = carry[i]; }
+    __device__ __forceinline__ void store(double *carry, size_t i) const { carry[i] = s; }
 };
 template <> struct MomentSum<float2> {
     float2 h, l;
@@ -1839,6 +1844,16 @@ template <> struct MomentSum<float2> {
         const float2 s = psum(x, h, one), v = pfma(h, m1, s);     // s - h
         l = padd(l, padd(pfma(pfma(v, m1, s), m1, h), pfma(v, m1, x)));   // (h - (s - v)) + (x - v)
         h = s;
+    }
+    __device__ __forceinline__ void load(const float *carry, size_t i)
+    {
+        const float4 v = reinterpret_cast<const float4 *>(carry)[i];
+        h = make_float2(v.x, v.y);
+        l = make_float2(v.z, v.w);
+    }
+    __device__ __forceinline__ void store(float *carry, size_t i) const
+    {
+        reinterpret_cast<float4 *>(carry)[i] = make_float4(h.x, h.y, l.x, l.y);
     }
 };
 
@@ -1872,8 +1887,10 @@ __device__ __forceinline__ void stage1_body(const DevCase<T> &dc, const int bx, 
     const int ncb = (dc.C + 7) >> 3, grp = bx / ncb;
     const int c = (bx - grp * ncb) * 8 + (threadIdx.x >> 5);
     if (c >= dc.C) return;
-    const int kb = chunk * dc.chunk, kg = grp * dc.gvel;              // chunk start; group start in the chunk
-    const int kn = min(min(dc.chunk, dc.nvp - kb), kg + dc.gvel);     // end in the chunk
+    int kb, kn;                                                        // chunk start, velocities
+    chunk_span(dc, chunk, kb, kn);
+    const int kg = grp * dc.gvel;                                      // group start in the chunk
+    kn = min(kn, kg + dc.gvel);                                        // end in the chunk
     if (kg >= kn) return;                                              // the last chunk may be short
     int e0 = c * NF, ne = NF;
     if (NF == 0) entry_range(dc, c, e0, ne);
@@ -1915,6 +1932,10 @@ __device__ __forceinline__ void stage1_body(const DevCase<T> &dc, const int bx, 
     MomentSum<P> acc[M];
 #pragma unroll
     for (int i = 0; i < M; ++i) acc[i].zero();
+    // a group in several chunks: the lane's sums go on where the chunk before left them
+    if (dc.parts > 1 && chunk % dc.parts > 0)
+#pragma unroll
+        for (int i = 0; i < M; ++i) acc[i].load(dc.carry, ((size_t)c * M + i) * 32 + lane);
     int slot = 0;
     for (int kc = kg + 4 * lane; kc < kn; kc += 128) {
         P fs[NC][NP], R[NC][NP];
@@ -1994,6 +2015,12 @@ __device__ __forceinline__ void stage1_body(const DevCase<T> &dc, const int bx, 
             stv<T, 4>(frow + (size_t)m * dc.nvp + kc, v);
         }
     }
+    const int group = (kb + kg) / dc.gvel;
+    if (dc.parts > 1 && kb + kn < min(dc.nvp, (group + 1) * dc.gvel)) {
+#pragma unroll
+        for (int i = 0; i < M; ++i) acc[i].store(dc.carry, ((size_t)c * M + i) * 32 + lane);
+        return;
+    }
     // across the warp
     constexpr int NR = M <= 4 ? 4 : 8;
     const int vi = lane >> (NR == 4 ? 3 : 2);
@@ -2018,7 +2045,7 @@ __device__ __forceinline__ void stage1_body(const DevCase<T> &dc, const int bx, 
         sum = warp_transpose_sum<T, NR>(v);
     }
     if ((lane & (NR == 4 ? 7 : 3)) == 0 && vi < M)
-        dc.dW_part[((size_t)c * dc.n_groups + (kb + kg) / dc.gvel) * M + vi] = sum;
+        dc.dW_part[((size_t)c * dc.n_groups + group) * M + vi] = sum;
 }
 
 template <typename T, int D, int NC, int NF>
@@ -2500,14 +2527,16 @@ cudaError_t launch_stage1(int D, int nf, int blocks, int chunk, cudaStream_t st,
 
 template <typename T> int flux_blocks(const DevCase<T> &dc, int chunk)
 {
-    const int left = dc.nvp - chunk * dc.chunk;
-    return left > 0 ? dc.n_patches * (dc.nth / FLUX_THREADS) * cdiv(std::min(left, dc.chunk), dc.vtile) : 0;
+    int kb, len;
+    chunk_span(dc, chunk, kb, len);
+    return len > 0 ? dc.n_patches * (dc.nth / FLUX_THREADS) * cdiv(len, dc.vtile) : 0;
 }
 
 template <typename T> int stage1_blocks(const DevCase<T> &dc, int chunk)
 {
-    const int left = dc.nvp - chunk * dc.chunk;
-    return left > 0 ? cdiv(dc.C, 8) * cdiv(std::min(left, dc.chunk), dc.gvel) : 0;
+    int kb, len;
+    chunk_span(dc, chunk, kb, len);
+    return len > 0 ? cdiv(dc.C, 8) * cdiv(len, dc.gvel) : 0;
 }
 
 // the flux and stage-1 passes of one case over its chunks

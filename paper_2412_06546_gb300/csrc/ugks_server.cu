@@ -58,9 +58,10 @@ struct Request {
 };
 
 // Device bytes a case will hold, from its sizes (an upper bound of what
-// ugks_create allocates: f and the flux buffer, which is at most a copy of f, or
-// up to 4 MB or 128 velocities where that is more, FP64 cell / face arrays and
-// records).
+// ugks_create allocates: f, the flux buffer, which is at most 9/8 of a copy of f, or
+// up to 4 MB or 128 velocities where that is more, with a fixed tiling also the
+// lane sums of stage 1 or as many bytes more of the buffer, FP64 cell / face arrays
+// and records).
 size_t footprint_estimate(const Request &r)
 {
     const int D = r.D, M = D + 2, NC = D == 2 ? 2 : 1;
@@ -68,7 +69,8 @@ size_t footprint_estimate(const Request &r)
     const size_t nvp = (size_t)((r.Nv + 127) / 128 * 128);
     const size_t C = (size_t)r.C, F = (size_t)std::max<int64_t>(r.F, 1);
     const size_t f = C * NC * nvp * s, vel = F * NC * s;
-    size_t b = f + std::max({f, std::min<size_t>((size_t)4 << 20, vel * nvp), vel * 128});   // f, fluxes
+    size_t b = f + std::max({f + f / 8, std::min<size_t>((size_t)4 << 20, vel * nvp), vel * 128});   // f, fluxes
+    if (r.params.patch_cells > 0 || r.params.gather_tile_group > 0) b += C * M * 32 * (s == 8 ? 8 : 16);
     b += C * (size_t)(M * 2 + D + D * M * 2 + 8) * 8;                  // W, q, prim, gradients, vol
     b += C * 2 * 12 * s + C * (nvp / 32 + 1) * M * s;                  // records, residual partials
     b += F * (size_t)(40 * s + 24 * s + 16 * s + (D * M + D + D + M + M + 5) * 8 + 60 * 8 + 64);

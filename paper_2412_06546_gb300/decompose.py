@@ -140,8 +140,8 @@ class DecomposedCase:
     steps every subdomain once, then moves the halo rows by device copies
     (ugks_halo_pack into a buffer, ugks_halo_unpack from it).  All
     subdomains share one stream, so the moves are ordered after the steps.
-    ``tiling`` fixes the gather tiling of every subdomain (it must match the
-    undivided case's for bit-identical results)."""
+    ``tiling`` fixes the tiling of every subdomain: bit-identical results need
+    the undivided case's ``patch_cells``, ``vtile`` and ``tile_group``."""
 
     def __init__(self, case, nparts, precision, stream=None, **tiling):
         import torch
