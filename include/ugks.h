@@ -112,7 +112,8 @@ typedef struct {
                                residual are summed over groups of this many tiles, the groups in FP64
                                (1 .. 1024, larger values are clamped to the number of tiles; 0: chosen
                                from the velocity count where patch_cells is given, else from the sizes of
-                               the case) */
+                               the case).  With vtile 0 the tiles meant are of 64 velocities (UGKS_FP64:
+                               32), and the autotuner takes a tile that divides the group. */
     int32_t w0_analytic;    /* interface equilibrium W0 (Sec. 2.4) from: 0 the discrete half-range
                                sums over the velocity set (default), 1 the analytic half-range
                                moments of the face-state Maxwellians over the continuous velocity
@@ -142,7 +143,8 @@ typedef struct {
     int64_t kernel_launches_per_step;
     int64_t n_wall_faces;               /* faces of type UGKS_FACE_WALL */
     int32_t gather_threads;             /* threads per patch of the flux pass in use */
-    int32_t gather_tile_group;          /* velocity tiles per moment group of stage 1 in use */
+    int32_t gather_tile_group;          /* velocity tiles (of vtile) per moment group of stage 1 in use: a
+                                           case created with the reported tiling has the same groups */
 } ugks_info_t;
 
 /* Create a case: validates and copies the inputs, orders cells for locality,

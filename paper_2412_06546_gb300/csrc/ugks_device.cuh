@@ -155,7 +155,7 @@ struct DevCase {
     int P, n_patches, vtile;      // cells per patch and velocities per warp of the flux pass
     int nth;                      // threads per patch (256, or 512 for FP32 at vtile <= 64), in CTAs of 128
     int chunk, n_chunks;          // velocities per chunk, chunks (see chunk_span)
-    int gvel, n_groups;           // velocities of a cell per warp of stage 1, groups per cell
+    int gvel, n_groups;           // velocities of a cell per warp of stage 1 (whole tiles, or all), groups per cell
     int parts;                    // chunks per group: 1 (a chunk holds one group or several), or more
     T *carry;                     // parts > 1: lane sums of a group between its chunks, [C][D+2][32] of MomentSum
 };

@@ -832,7 +832,9 @@ void autotune(ugks_case *c, ugks::DevCase<T> &dc, bool tune_vtile)
         cuda_ok(cudaEventCreate(&e1), "event");
         float best_ms = 0.f;
         for (int vt : vc) {
-            if ((c->chunk % vt && c->n_chunks > 1) || (c->nth == 512 && vt > 64)) continue;
+            // whole tiles per group, so that the reported tiling gives the same groups again;
+            // the key holds all that this depends on
+            if ((c->gvel % vt && c->gvel != c->nvp) || (c->nth == 512 && vt > 64)) continue;
             for (int P : {8, 16, 32, 64}) {
                 if (P > 8 && (P < c->nth / 32 || P > std::max<int64_t>(16, c->C / 64))) continue;
                 set_tiling(c, dc, P, vt);

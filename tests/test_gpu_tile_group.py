@@ -64,6 +64,31 @@ def test_group_is_used_on_every_mesh(name, precision, vtile, group, chunks):
 
 
 @pytest.mark.parametrize("precision", [_lib.FP32, _lib.FP64])
+@pytest.mark.parametrize("nv,group", [((24, 24), 0), ((24, 24), 3), ((41, 37), 0), ((41, 37), 1), ((41, 37), 5)])
+def test_reported_tiling_gives_the_same_groups(precision, nv, group):
+    """The autotuned tiling that ugks_info reports, fed back, gives the same moment
+    groups: W after three steps is bitwise the same.  A caller's group is of
+    default tiles whatever tile the autotuner takes."""
+    case = cs.cylinder_case(n_cells=3000, nvx=nv[0], nvy=nv[1], mach=3.0)
+    f, W = _perturbed(case, precision)
+    out = []
+    tiling = {"tile_group": group}
+    for _ in range(2):
+        g = _lib.Case(case["mesh"], case["vgrid"], case["params"], case["init"], precision=precision, **tiling)
+        i = g.info()
+        if group:
+            assert i["gather_tile_group"] * i["vtile"] == group * (64 if precision == _lib.FP32 else 32)
+        tiling = {"patch_cells": i["patch_cells"], "vtile": i["vtile"], "threads": i["gather_threads"],
+                  "tile_group": i["gather_tile_group"]}
+        g.set_state(f, W)
+        g.step(3)
+        out.append(g.state())
+        g.close()
+    assert np.array_equal(out[0][1], out[1][1]), np.abs(out[0][1] - out[1][1]).max()
+    assert np.array_equal(out[0][0], out[1][0])
+
+
+@pytest.mark.parametrize("precision", [_lib.FP32, _lib.FP64])
 @pytest.mark.parametrize("tiling", [{}, {"patch_cells": 16, "vtile": 32, "tile_group": 1024},
                                     {"patch_cells": 16, "vtile": 32, "tile_group": 1}])
 def test_footprint_estimate_bounds_the_device_bytes(precision, tiling):
