@@ -728,7 +728,8 @@ void fill_case(ugks_case *c, ugks::DevCase<T> &dc, const ugks_mesh *m, const ugk
     dc.fprim0 = (double *)c->dalloc(Fm * M * sizeof(double));
     dc.fqs = (double *)c->dalloc(Fm * 5 * sizeof(double));
     dc.dW_part = (double *)c->dalloc((size_t)c->C * c->n_groups * M * sizeof(double));
-    dc.res_part = (double *)c->dalloc((size_t)c->n_res_parts * 2 * M * sizeof(double));
+    // the partials, then the folded ones (residual_parts)
+    dc.res_part = (double *)c->dalloc((size_t)(c->n_res_parts + c->n_res_parts / ugks::RES_FOLD + 1) * 2 * M * sizeof(double));
     dc.flags = c->flags_d;
     dc.owned = nullptr;
     dc.gvel = c->gvel;
@@ -967,6 +968,21 @@ void export_W(ugks_case *c, double *W)
     cuda_ok(cudaStreamSynchronize(c->stream), "sync");
 }
 
+// the partial sums of the last step's residual and their number: folded by
+// RES_FOLD above 65,536 cells, where copying or adding up the 32-cell partials takes
+// longer than the launch (a million cells: ugks_residual_sums 0.162 -> 0.046 ms,
+// ugks_residual 0.111 -> 0.052 ms; 30k cells unfolded 0.023, folded 0.027)
+const double *residual_parts(ugks_case *c, int &n)
+{
+    double *rp = c->prec == UGKS_FP64 ? c->d64.res_part : c->d32.res_part;
+    n = c->n_res_parts;
+    if (n <= 2048) return rp;
+    double *folded = rp + (size_t)n * 2 * (c->D + 2);
+    cuda_ok(ugks::launch_residual_fold(rp, n, c->D, folded, c->stream), "residual launch");
+    n = (n + ugks::RES_FOLD - 1) / ugks::RES_FOLD;
+    return folded;
+}
+
 template <typename S>
 ugks_status get_state(ugks_case *c, S *f, double *W)
 {
@@ -1149,8 +1165,9 @@ ugks_status ugks_residual(ugks_case *c, double *res)
             for (int m = 0; m < M; ++m) res[m] = 0.0;
             return;
         }
-        const double *rp = c->prec == UGKS_FP64 ? c->d64.res_part : c->d32.res_part;
-        cuda_ok(ugks::launch_residual(rp, c->n_res_parts, c->D, c->res_d, c->stream), "residual launch");
+        int n;
+        const double *rp = residual_parts(c, n);
+        cuda_ok(ugks::launch_residual(rp, n, c->D, c->res_d, c->stream), "residual launch");
         cuda_ok(cudaMemcpyAsync(res, c->res_d, M * sizeof(double), cudaMemcpyDeviceToHost, c->stream), "residual copy");
         cuda_ok(cudaStreamSynchronize(c->stream), "residual sync");
     });
@@ -1334,12 +1351,13 @@ ugks_status ugks_residual_sums(ugks_case *c, double *sums)
         const int M = c->D + 2;
         for (int i = 0; i < 2 * M; ++i) sums[i] = 0.0;
         if (!c->stepped) return;
-        std::vector<double> part((size_t)c->n_res_parts * 2 * M);
-        const double *rp = c->prec == UGKS_FP64 ? c->d64.res_part : c->d32.res_part;
+        int n;
+        const double *rp = residual_parts(c, n);
+        std::vector<double> part((size_t)n * 2 * M);
         cuda_ok(cudaMemcpyAsync(part.data(), rp, part.size() * sizeof(double), cudaMemcpyDeviceToHost, c->stream),
                 "residual copy");
         cuda_ok(cudaStreamSynchronize(c->stream), "residual sync");
-        for (int b = 0; b < c->n_res_parts; ++b)
+        for (int b = 0; b < n; ++b)
             for (int i = 0; i < 2 * M; ++i) sums[i] += part[(size_t)b * 2 * M + i];
     });
 }

@@ -2116,18 +2116,25 @@ __global__ void __launch_bounds__(256) k_update_W_batch(const DevCase<T> *__rest
     update_W_body<T, D, NC>(dc, bx);
 }
 
-// one block of RES_THREADS threads: lane sums of the partials, then the lanes in order
+// one block of RES_THREADS threads: thread sums of the partials, all values of a
+// partial requested together, then the lanes in order
 constexpr int RES_THREADS = 512;
 template <int M>
 __global__ void __launch_bounds__(RES_THREADS) k_residual(const double *res_part, int nparts, double *res)
 {
     __shared__ double acc[2 * M][RES_THREADS / 32];
     const int t = threadIdx.x;
+    double s[2 * M];
+#pragma unroll
+    for (int i = 0; i < 2 * M; ++i) s[i] = 0.0;
+#pragma unroll 4
+    for (int b = t; b < nparts; b += RES_THREADS)
+#pragma unroll
+        for (int i = 0; i < 2 * M; ++i) s[i] += res_part[(size_t)b * 2 * M + i];
+#pragma unroll
     for (int i = 0; i < 2 * M; ++i) {
-        double s = 0.0;
-        for (int b = t; b < nparts; b += RES_THREADS) s += res_part[(size_t)b * 2 * M + i];
-        s = warp_sum(s);
-        if ((t & 31) == 0) acc[i][t >> 5] = s;
+        const double v = warp_sum(s[i]);
+        if ((t & 31) == 0) acc[i][t >> 5] = v;
     }
     __syncthreads();
     if (t < M) {
@@ -2138,6 +2145,16 @@ __global__ void __launch_bounds__(RES_THREADS) k_residual(const double *res_part
         }
         res[t] = b > 0.0 ? sqrt(a) / sqrt(b) : sqrt(a);
     }
+}
+
+// sums of RES_FOLD consecutive partials (of 32 cells each), a thread per value
+__global__ void __launch_bounds__(256) k_residual_fold(const double *res_part, int nparts, int nvals, double *out)
+{
+    const int t = blockIdx.x * 256 + threadIdx.x, j = t / nvals, i = t - j * nvals;
+    if (j * RES_FOLD >= nparts) return;
+    double s = 0.0;
+    for (int b = j * RES_FOLD; b < min(nparts, (j + 1) * RES_FOLD); ++b) s += res_part[(size_t)b * nvals + i];
+    out[t] = s;
 }
 
 // ------------------------------------------------------------ stage 2
@@ -2804,6 +2821,13 @@ cudaError_t launch_residual(const double *res_part, int nparts, int D, double *r
 {
     if (D == 2) k_residual<4><<<1, RES_THREADS, 0, st>>>(res_part, nparts, res);
     else k_residual<5><<<1, RES_THREADS, 0, st>>>(res_part, nparts, res);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_residual_fold(const double *res_part, int nparts, int D, double *out, cudaStream_t st)
+{
+    const int nvals = 2 * (D + 2), n = cdiv(nparts, RES_FOLD) * nvals;
+    if (n > 0) k_residual_fold<<<cdiv(n, 256), 256, 0, st>>>(res_part, nparts, nvals, out);
     return cudaGetLastError();
 }
 
