@@ -447,7 +447,12 @@ __device__ __forceinline__ void shakhov_fplus(const T *rec, const T u[3], T fp[N
 }
 
 // TV consecutive values at a TV*sizeof(T)-aligned address, moved in chunks
-// of at most 16 bytes (read-only data through the non-coherent path)
+// of at most 16 bytes.  Two kinds of loads: *_const through the non-coherent
+// path, for what no kernel of a step writes (velocities, weights, geometry), and
+// ordinary ones for what an earlier kernel of the step wrote (f, the fluxes, the
+// records).  A kernel of a step starts before its predecessor has ended
+// (dependency_wait), and a non-coherent load may be moved ahead of the wait: it
+// asks for memory that is read-only as long as the kernel lives.
 template <typename T, int N> struct VecOf;
 template <> struct VecOf<float, 1> { using type = float; };
 template <> struct VecOf<float, 2> { using type = float2; };
@@ -456,19 +461,25 @@ template <> struct VecOf<double, 1> { using type = double; };
 template <> struct VecOf<double, 2> { using type = double2; };
 template <typename T, int TV> constexpr int vec_chunk() { return TV * (int)sizeof(T) <= 16 ? TV : 16 / (int)sizeof(T); }
 
-template <typename T, int TV>
-__device__ __forceinline__ void ldv(const T *__restrict__ p, T (&x)[TV])
+template <bool CONST, typename V> __device__ __forceinline__ V ld(const V *p)
+{
+    if constexpr (CONST) return __ldg(p);
+    else return *p;
+}
+template <bool CONST, typename T, int TV>
+__device__ __forceinline__ void ld_lane(const T *p, T (&x)[TV])
 {
     constexpr int CH = vec_chunk<T, TV>();
     using V = typename VecOf<T, CH>::type;
 #pragma unroll
     for (int i = 0; i < TV / CH; ++i) {
-        const V v = __ldg(reinterpret_cast<const V *>(p) + i);
+        const V v = ld<CONST>(reinterpret_cast<const V *>(p) + i);
         const T *e = reinterpret_cast<const T *>(&v);
 #pragma unroll
         for (int j = 0; j < CH; ++j) x[i * CH + j] = e[j];
     }
 }
+template <typename T, int TV> __device__ __forceinline__ void ldv_const(const T *p, T (&x)[TV]) { ld_lane<true>(p, x); }
 template <typename T, int TV>
 __device__ __forceinline__ void stv(T *p, const T (&x)[TV])
 {
@@ -485,30 +496,20 @@ __device__ __forceinline__ void stv(T *p, const T (&x)[TV])
 }
 
 // copy a 16-byte aligned record of N values into registers with vector loads
-template <int N>
-__device__ __forceinline__ void load_rec(const float *__restrict__ p, float (&r)[N])
+template <bool CONST, typename T, int N> __device__ __forceinline__ void ld_rec(const T *p, T (&r)[N])
 {
-    static_assert(N % 4 == 0, "record length");
+    constexpr int CH = 16 / (int)sizeof(T);
+    static_assert(N % CH == 0, "record length");
 #pragma unroll
-    for (int i = 0; i < N / 4; ++i) {
-        const float4 v = __ldg(reinterpret_cast<const float4 *>(p) + i);
-        r[4 * i] = v.x;
-        r[4 * i + 1] = v.y;
-        r[4 * i + 2] = v.z;
-        r[4 * i + 3] = v.w;
+    for (int i = 0; i < N / CH; ++i) {
+        const typename VecOf<T, CH>::type v = ld<CONST>(reinterpret_cast<const typename VecOf<T, CH>::type *>(p) + i);
+        const T *e = reinterpret_cast<const T *>(&v);
+#pragma unroll
+        for (int j = 0; j < CH; ++j) r[i * CH + j] = e[j];
     }
 }
-template <int N>
-__device__ __forceinline__ void load_rec(const double *__restrict__ p, double (&r)[N])
-{
-    static_assert(N % 2 == 0, "record length");
-#pragma unroll
-    for (int i = 0; i < N / 2; ++i) {
-        const double2 v = __ldg(reinterpret_cast<const double2 *>(p) + i);
-        r[2 * i] = v.x;
-        r[2 * i + 1] = v.y;
-    }
-}
+template <int N, typename T> __device__ __forceinline__ void load_rec(const T *p, T (&r)[N]) { ld_rec<false>(p, r); }
+template <int N, typename T> __device__ __forceinline__ void load_rec_const(const T *p, T (&r)[N]) { ld_rec<true>(p, r); }
 
 // velocity k and its weight from the packed array, one 16-byte (FP32) or two
 // 16-byte (FP64) loads
@@ -579,14 +580,18 @@ template <int W, typename P> __device__ __forceinline__ auto &pel(P *x, int j)
 }
 
 // TV consecutive values into packs
-template <typename T, int TV>
-__device__ __forceinline__ void ldp(const T *__restrict__ p, typename Pk<T, TV>::P (&x)[Pk<T, TV>::NP])
+template <bool CONST, typename T, int TV>
+__device__ __forceinline__ void ld_pack(const T *p, typename Pk<T, TV>::P (&x)[Pk<T, TV>::NP])
 {
     T v[TV];
-    ldv<T, TV>(p, v);
+    ld_lane<CONST>(p, v);
 #pragma unroll
     for (int j = 0; j < TV; ++j) pel<Pk<T, TV>::W>(x, j) = v[j];
 }
+template <typename T, int TV>
+__device__ __forceinline__ void ldp(const T *p, typename Pk<T, TV>::P (&x)[Pk<T, TV>::NP]) { ld_pack<false, T, TV>(p, x); }
+template <typename T, int TV>
+__device__ __forceinline__ void ldp_const(const T *p, typename Pk<T, TV>::P (&x)[Pk<T, TV>::NP]) { ld_pack<true, T, TV>(p, x); }
 
 // a + b where a is a product that must not be contracted into the sum.  ptxas
 // fuses a packed multiplication and addition even where both carry .rn (the
@@ -741,7 +746,7 @@ template <typename T, int D, int NC, int TV> struct GlobalCell {
     __device__ __forceinline__ int4 ids(int e) const { return __ldg(dc.gi + e0 + e); }
     __device__ __forceinline__ void values(int e, int at, T (&v)[4]) const
     {
-        load_rec<4>(dc.gf + (size_t)(e0 + e) * GEnt<D>::LEN + at, v);
+        load_rec_const<4>(dc.gf + (size_t)(e0 + e) * GEnt<D>::LEN + at, v);
     }
     __device__ __forceinline__ void row_of(int cell, P (&x)[NC][NP]) const
     {

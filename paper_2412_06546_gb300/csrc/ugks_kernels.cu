@@ -544,8 +544,8 @@ __device__ __forceinline__ void face_sum1_body(const DevCase<T> &dc, const int b
     T sL[GREC], sR[GREC];
 #pragma unroll
     for (int i = 0; i < GREC; ++i) {
-        sL[i] = __ldg(dc.fside + (size_t)f * 2 * GREC + i);
-        sR[i] = __ldg(dc.fside + (size_t)f * 2 * GREC + GREC + i);
+        sL[i] = dc.fside[(size_t)f * 2 * GREC + i];
+        sR[i] = dc.fside[(size_t)f * 2 * GREC + GREC + i];
     }
     T n[D], Ur[D];
     for (int d = 0; d < D; ++d) {
@@ -1395,13 +1395,13 @@ __device__ __forceinline__ void wall_sum_body(const DevCase<T> &dc, const int bx
     entry_range(dc, c, e0, ne);
     for (int k0 = TW * threadIdx.x; k0 < dc.nvp; k0 += TW * blockDim.x) {
         T u[3][TW], wk[TW], un[TW];
-        ldv<T, TW>(dc.u[0] + k0, u[0]);
-        ldv<T, TW>(dc.u[1] + k0, u[1]);
-        if (D == 3) ldv<T, TW>(dc.u[2] + k0, u[2]);
+        ldv_const<T, TW>(dc.u[0] + k0, u[0]);
+        ldv_const<T, TW>(dc.u[1] + k0, u[1]);
+        if (D == 3) ldv_const<T, TW>(dc.u[2] + k0, u[2]);
         else
 #pragma unroll
             for (int j = 0; j < TW; ++j) u[2][j] = T(0);
-        ldv<T, TW>(dc.w + k0, wk);
+        ldv_const<T, TW>(dc.w + k0, wk);
         bool out = false;
 #pragma unroll
         for (int j = 0; j < TW; ++j) {
@@ -1575,12 +1575,12 @@ __device__ __forceinline__ void flux_body(const DevCase<T> &dc, const int bx, co
     const int kc = live ? kl : tile * V, k = kb + kc;
     const unsigned all = live ? (1u << TV) - 1 : 0u;
     const int cb = p * dc.P, ce = min(dc.C, cb + dc.P);
-    const T *__restrict__ fl = dc.f_cur + k;
+    const T *fl = dc.f_cur + k;
     P u[NP][D];
 #pragma unroll
     for (int d = 0; d < D; ++d) {
         P t[NP];
-        ldp<T, TV>(dc.u[d] + k, t);
+        ldp_const<T, TV>(dc.u[d] + k, t);
 #pragma unroll
         for (int i = 0; i < NP; ++i) u[i][d] = t[i];
     }
@@ -1978,8 +1978,8 @@ __device__ __forceinline__ void stage1_body(const DevCase<T> &dc, const int bx, 
         }
         P u[D][NP], wk[NP];
 #pragma unroll
-        for (int d = 0; d < D; ++d) ldp<T, 4>(dc.u[d] + kb + kc, u[d]);
-        ldp<T, 4>(dc.w + kb + kc, wk);
+        for (int d = 0; d < D; ++d) ldp_const<T, 4>(dc.u[d] + kb + kc, u[d]);
+        ldp_const<T, 4>(dc.w + kb + kc, wk);
 #pragma unroll
         for (int i = 0; i < NP; ++i) {
             // f+ of the cell (shakhov_fplus), stage 1
@@ -2174,7 +2174,7 @@ __device__ __forceinline__ void collide_body(const DevCase<T> &dc, const int bx)
     // the cell's record in registers: read once, not again after every store of f
     T kr[CREC];
 #pragma unroll
-    for (int i = 0; i < CREC; ++i) kr[i] = __ldg(dc.krec + (size_t)c * CREC + i);
+    for (int i = 0; i < CREC; ++i) kr[i] = dc.krec[(size_t)c * CREC + i];
     const T cc = kr[CR_C];
     const T inv = kr[CR_INV];
     T U[D];
@@ -2224,13 +2224,13 @@ __device__ __forceinline__ void collide_body(const DevCase<T> &dc, const int bx)
             // of four consecutive velocities per lane would touch four times the
             // cache lines per load)
             T uv[3][4], wv[4];
-            ldv<T, 4>(dc.u[0] + k0, uv[0]);
-            ldv<T, 4>(dc.u[1] + k0, uv[1]);
-            if (D == 3) ldv<T, 4>(dc.u[2] + k0, uv[2]);
+            ldv_const<T, 4>(dc.u[0] + k0, uv[0]);
+            ldv_const<T, 4>(dc.u[1] + k0, uv[1]);
+            if (D == 3) ldv_const<T, 4>(dc.u[2] + k0, uv[2]);
             else
 #pragma unroll
                 for (int j = 0; j < 4; ++j) uv[2][j] = T(0);
-            ldv<T, 4>(dc.w + k0, wv);
+            ldv_const<T, 4>(dc.w + k0, wv);
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 const T u[3] = {uv[0][j], uv[1][j], uv[2][j]};
@@ -2433,7 +2433,7 @@ __global__ void __launch_bounds__(256) k_halo_pack(DevCase<T> dc, const int *cel
 #pragma unroll
     for (int m = 0; m < NC; ++m) {
         T *__restrict__ fo = reinterpret_cast<T *>(r) + (size_t)m * dc.nv;
-        const T *__restrict__ fc = dc.f_cur + ((size_t)c * NC + m) * dc.nvp;
+        const T *fc = dc.f_cur + ((size_t)c * NC + m) * dc.nvp;
         copy_row(fc, fo, dc.nv);
     }
     double *tail = reinterpret_cast<double *>(r + row - (size_t)(M + D) * sizeof(double));
@@ -2453,7 +2453,7 @@ __global__ void __launch_bounds__(256) k_halo_unpack(DevCase<T> dc, const int *c
 #pragma unroll
     for (int m = 0; m < NC; ++m) {
         const T *__restrict__ fi = reinterpret_cast<const T *>(r) + (size_t)m * dc.nv;
-        T *__restrict__ fc = dc.f_cur + ((size_t)c * NC + m) * dc.nvp;
+        T *fc = dc.f_cur + ((size_t)c * NC + m) * dc.nvp;
         copy_row(fi, fc, dc.nv);
     }
     const double *tail = reinterpret_cast<const double *>(r + row - (size_t)(M + D) * sizeof(double));
