@@ -22,6 +22,7 @@
 // equilibrium parameters, the heat flux, the collision coefficients) are
 // formed in FP64.
 #include "ugks_device.cuh"
+#include "ugks_scalar.cuh"
 #include "ugks_kernels.h"
 
 #include <algorithm>
@@ -30,44 +31,7 @@
 
 namespace ugks {
 
-// ------------------------------------------------------------ FP64 helpers
-struct Prim {
-    double rho, U[MAXD], lam, T;
-};
-
-__device__ __forceinline__ Prim prim_of(const double *W, int D)
-{
-    Prim p;
-    p.rho = W[0];
-    const double ir = 1.0 / W[0];
-    double ke = 0.0;
-    for (int d = 0; d < MAXD; ++d) p.U[d] = 0.0;
-    for (int d = 0; d < D; ++d) {
-        p.U[d] = W[1 + d] * ir;
-        ke += p.U[d] * p.U[d];
-    }
-    p.T = (2.0 / 3.0) * (W[D + 1] * ir - 0.5 * ke);
-    p.lam = 0.5 / p.T;
-    return p;
-}
-
-// the same from a primitive row (rho, U, T)
-template <int D> __device__ __forceinline__ void set_prim(const double *P, Prim &p)
-{
-    p.rho = P[0];
-    for (int d = 0; d < MAXD; ++d) p.U[d] = d < D ? P[1 + d] : 0.0;
-    p.T = P[D + 1];
-    p.lam = 0.5 / p.T;
-}
-
-constexpr double LOG2E = 1.4426950408889634073599246810018921;
-
-__device__ __forceinline__ double pref_of(double rho, double lam, int D)
-{
-    const double a = lam * 0.31830988618379067153776752674502872;    // 1 / pi
-    return D == 2 ? rho * a : rho * a * sqrt(a);
-}
-
+// ------------------------------------------------------------ FP64 helpers (see ugks_scalar.cuh)
 // dt / tau of a state, tau = mu_ref T^omega / (rho T) (VHS viscosity, p = rho T)
 template <typename T>
 __device__ __forceinline__ double dt_over_tau(const DevCase<T> &dc, double rho, double Tmp)
@@ -91,45 +55,6 @@ __device__ __forceinline__ void cell_record(const DevCase<T> &dc, const Prim &p,
     r[CR_INV] = (T)(1.0 / (1.0 + cc));
     r[CR_NB] = (T)(dc.nxi * p.T);
     r[CR_NL2] = (T)(-p.lam * LOG2E);
-}
-
-// Time integrals of c1..c5 over [0, dt] (Sec. 2.4), written with x = dt/tau,
-// E = 1 - e^{-x}:  q1 = dt E/x, q2 = dt^2 (x e^{-x} - E)/x^2, q3 = dt (x - E)/x,
-// q4 = dt^2 (2E - x(1 + e^{-x}))/x^2, q5 = dt^2 (x^2/2 - x + E)/x^2.
-// Below x = 1/2 the brackets cancel; with phi_n = sum_i (-x)^i / (i + n)! they
-// are phi_1, phi_2 - phi_1, x phi_2, -x (phi_2 - 2 phi_3) and x phi_3, where
-// phi_3 is summed to rounding and phi_2 = 1/2 - x phi_3, phi_1 = 1 - x phi_2.
-// (Summing the five series term by term took about 500 FP64 operations; an SM
-// retires 1.6 of them per cycle and lane-wise that was half of k_face_fin1.)
-__device__ __forceinline__ void time_integrals(double dt, double x, double q[5])
-{
-    if (x < 0.5) {
-        double f = 1.0;                    // (i + 3)! upwards, folded at compile time
-        double c[14];
-#pragma unroll
-        for (int i = 0; i < 14; ++i) {
-            f *= i == 0 ? 6.0 : (double)(i + 3);
-            c[i] = (i & 1 ? -1.0 : 1.0) / f;
-        }
-        double p3 = c[13];
-#pragma unroll
-        for (int i = 12; i >= 0; --i) p3 = fma(p3, x, c[i]);
-        const double p2 = fma(-x, p3, 0.5), p1 = fma(-x, p2, 1.0);
-        q[0] = dt * p1;
-        q[1] = dt * dt * (p2 - p1);
-        q[2] = dt * x * p2;
-        q[3] = -dt * dt * x * fma(-2.0, p3, p2);
-        q[4] = dt * dt * x * p3;
-    } else {
-        const double e = exp(-x);
-        const double E = 1.0 - e;
-        const double ix = 1.0 / x, ix2 = ix * ix;
-        q[0] = dt * E * ix;
-        q[1] = dt * dt * (x * e - E) * ix2;
-        q[2] = dt * (x - E) * ix;
-        q[3] = dt * dt * (2.0 * E - x * (1.0 + e)) * ix2;
-        q[4] = dt * dt * (0.5 * x * x - x + E) * ix2;
-    }
 }
 
 // ------------------------------------------------------------ launches
@@ -1144,58 +1069,6 @@ __device__ __forceinline__ void sep_moments(const double (&m)[D][6], double pref
                 R[Mo::O3 + triple_index(D, d, e, g)] = Q(xe + (g == 0), ye + (g == 1), ze + (g == 2));
         }
     }
-}
-
-// A = L diag(d) L^T of a symmetric positive definite matrix (packed upper
-// triangle t(i, j), i <= j); inv[i] = 1 / d_i, L below the diagonal in place of
-// the entries.  Five divisions for the factor and none in the solves (the
-// Cholesky form took 5 square roots and 50 divisions for the four right-hand
-// sides, FP64 operations of about ten instructions each).
-template <int M> __device__ __forceinline__ constexpr int tri(int i, int j) { return i * M - i * (i - 1) / 2 + (j - i); }
-
-template <int M>
-__device__ __forceinline__ void ldl_factor(double *A, double (&inv)[M])
-{
-#pragma unroll
-    for (int j = 0; j < M; ++j) {
-        double dj = A[tri<M>(j, j)];
-        double w[M];                             // L_jk d_k
-#pragma unroll
-        for (int k = 0; k < j; ++k) {
-            w[k] = A[tri<M>(k, j)];
-            const double l = w[k] * inv[k];
-            dj -= l * w[k];
-        }
-        inv[j] = 1.0 / dj;
-        // A(j, i) for i > j: subtract sum_k L_jk d_k L_ik, kept as L_ij d_j
-#pragma unroll
-        for (int i = j + 1; i < M; ++i) {
-            double t = A[tri<M>(j, i)];
-#pragma unroll
-            for (int k = 0; k < j; ++k) t -= w[k] * inv[k] * A[tri<M>(k, i)];
-            A[tri<M>(j, i)] = t;
-        }
-    }
-    // entries (j, i) hold L_ij d_j: scale to L_ij
-#pragma unroll
-    for (int j = 0; j < M; ++j)
-#pragma unroll
-        for (int i = j + 1; i < M; ++i) A[tri<M>(j, i)] *= inv[j];
-}
-
-template <int M>
-__device__ __forceinline__ void ldl_solve(const double *A, const double (&inv)[M], double *x)
-{
-#pragma unroll
-    for (int i = 1; i < M; ++i)
-#pragma unroll
-        for (int k = 0; k < i; ++k) x[i] -= A[tri<M>(k, i)] * x[k];
-#pragma unroll
-    for (int i = 0; i < M; ++i) x[i] *= inv[i];
-#pragma unroll
-    for (int i = M - 2; i >= 0; --i)
-#pragma unroll
-        for (int k = i + 1; k < M; ++k) x[i] -= A[tri<M>(i, k)] * x[k];
 }
 
 // slopes of g0 in the centred basis: M0 = L Mc L^T, sum_k w u_d psi psi^T g0 =
