@@ -9,6 +9,16 @@ struct Prim {
     double rho, U[MAXD], lam, T;
 };
 
+// a / b with ib = 1 / b: the quotient's remainder corrects the product, which
+// rounds as the division does in all but rare cases, for a third of its operations
+__device__ __forceinline__ double quotient(double a, double b, double ib)
+{
+    const double q = a * ib;
+    return fma(fma(-q, b, a), ib, q);
+}
+
+// (with products by the reciprocal, U of random states was off by 0.64e-16 in the
+// root mean square, where divisions and this leave 0.43e-16)
 __device__ __forceinline__ Prim prim_of(const double *W, int D)
 {
     Prim p;
@@ -17,10 +27,10 @@ __device__ __forceinline__ Prim prim_of(const double *W, int D)
     double ke = 0.0;
     for (int d = 0; d < MAXD; ++d) p.U[d] = 0.0;
     for (int d = 0; d < D; ++d) {
-        p.U[d] = W[1 + d] * ir;
+        p.U[d] = quotient(W[1 + d], W[0], ir);
         ke += p.U[d] * p.U[d];
     }
-    p.T = (2.0 / 3.0) * (W[D + 1] * ir - 0.5 * ke);
+    p.T = (2.0 / 3.0) * (quotient(W[D + 1], W[0], ir) - 0.5 * ke);
     p.lam = 0.5 / p.T;
     return p;
 }
@@ -38,7 +48,7 @@ constexpr double LOG2E = 1.4426950408889634073599246810018921;
 
 __device__ __forceinline__ double pref_of(double rho, double lam, int D)
 {
-    const double a = lam * 0.31830988618379067153776752674502872;    // 1 / pi
+    const double a = fma(lam, 0.3183098861837907, lam * -1.9678676675182487e-17);     // lam / pi, 1 / pi in two parts
     return D == 2 ? rho * a : rho * a * sqrt(a);
 }
 

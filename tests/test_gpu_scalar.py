@@ -11,7 +11,7 @@ torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
 HERE = os.path.dirname(os.path.abspath(__file__))
-EXP_NEG, TIME_INTEGRALS = range(2)
+EXP_NEG, TIME_INTEGRALS, PRIM2, PRIM3 = range(4)
 LD = np.longdouble
 # a root mean square over 2e4 samples scatters by well under 1 %, and the CUDA and the
 # host library round exp and expm1 differently (0.25 units in the last place in the mean)
@@ -109,3 +109,32 @@ def test_exp_neg_beyond_its_range(probe):
     x = np.array([710.0, 1e300, np.inf])
     assert np.all(probe(EXP_NEG, x, 1) == np.inf)
     assert np.all(np.isnan(probe(EXP_NEG, np.array([np.nan, -np.nan]), 1)))
+
+
+def _primitive(W):
+    """U, T, lam and the prefactor of a Maxwellian, in the type of W."""
+    D = W.shape[1] - 2
+    pi = W.dtype.type("3.14159265358979323846264338327950288")
+    U = W[:, 1:-1] / W[:, :1]
+    ke = np.zeros_like(W[:, 0])
+    for d in range(D):
+        ke = ke + U[:, d] * U[:, d]
+    T = W.dtype.type(2) / 3 * (W[:, -1] / W[:, 0] - ke / 2)
+    lam = 1 / (2 * T)
+    a = lam / pi
+    return np.column_stack([U, T, lam, W[:, 0] * a if D == 2 else W[:, 0] * a * np.sqrt(a)])
+
+
+@pytest.mark.parametrize("D,what", [(2, PRIM2), (3, PRIM3)])
+def test_primitive_variables(probe, D, what):
+    """(rho, rho U, rho E) over six decades of density and three of temperature to
+    U, T, lambda and the prefactor: the root mean square errors of the formulas
+    with IEEE divisions, on the same states (3 % for what the contraction of a
+    product and a sum changes at either side)."""
+    rng = np.random.default_rng(7)
+    rho, T = np.exp(rng.uniform(-7, 7, 10 * SAMPLES)), np.exp(rng.uniform(np.log(0.1), np.log(100.0), 10 * SAMPLES))
+    U = rng.normal(size=(10 * SAMPLES, D)) * np.sqrt(T)[:, None]
+    W = np.column_stack([rho, rho[:, None] * U, rho * (0.5 * (U * U).sum(1) + 1.5 * T)])
+    exact = _primitive(W.astype(LD))
+    here, plain = _rms(probe(what, W, D + 3), exact), _rms(_primitive(W), exact)
+    assert np.all(here <= 1.03 * plain), (here, plain)
