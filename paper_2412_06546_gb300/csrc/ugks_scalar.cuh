@@ -100,7 +100,10 @@ __device__ __forceinline__ void time_integrals(double dt, double x, double q[5])
 // triangle t(i, j), i <= j); inv[i] = 1 / d_i, L below the diagonal in place of
 // the entries.  Five divisions for the factor and none in the solves (the
 // Cholesky form took 5 square roots and 50 divisions for the four right-hand
-// sides, FP64 operations of about ten instructions each).
+// sides, FP64 operations of about ten instructions each).  A pivot that is not
+// positive makes the solutions NaN, as its square root would: such a matrix is no
+// set of moments (a velocity set in one plane, a broken state), and the NaN is what
+// ugks_check finds.
 template <int M> __device__ __forceinline__ constexpr int tri(int i, int j) { return i * M - i * (i - 1) / 2 + (j - i); }
 
 template <int M>
@@ -116,7 +119,7 @@ __device__ __forceinline__ void ldl_factor(double *A, double (&inv)[M])
             const double l = w[k] * inv[k];
             dj -= l * w[k];
         }
-        inv[j] = 1.0 / dj;
+        inv[j] = dj > 0.0 ? 1.0 / dj : __longlong_as_double(0x7ff8000000000000ll);
         // A(j, i) for i > j: subtract sum_k L_jk d_k L_ik, kept as L_ij d_j
 #pragma unroll
         for (int i = j + 1; i < M; ++i) {
