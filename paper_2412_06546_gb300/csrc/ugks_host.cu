@@ -1037,11 +1037,11 @@ ugks_status ugks_create(const ugks_mesh *mesh, const ugks_vgrid *vgrid, const ug
             c->alloc = *alloc;
             c->user_alloc = true;
         }
-        // velocity rows are padded to a multiple of the widest tile the autotuner
-        // may choose (64 in 2D, 128 in 3D) unless the tile is fixed
+        // velocity rows are padded to whole tiles, in 2D of 64 velocities at most (a
+        // last tile of 128 may be short), as for the autotuner's choice of a tile
         c->vtile = params->vtile > 0 ? params->vtile : kDefaultVtile(c->prec);
         c->nth = params->gather_threads > 0 ? params->gather_threads : 256;
-        const int vpad = params->vtile > 0 ? params->vtile : (c->D == 3 ? 128 : 64);
+        const int most = c->D == 3 ? 128 : 64, vpad = params->vtile > 0 ? std::min(params->vtile, most) : most;
         c->P = params->patch_cells > 0 ? params->patch_cells : 16;
         Host h;
         preprocess(mesh, params, h);
