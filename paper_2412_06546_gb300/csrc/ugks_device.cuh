@@ -415,19 +415,6 @@ __device__ __forceinline__ double block_to_fp64(float (&blk)[N])
     return (double)warp_transpose_sum<float, N>(blk);
 }
 
-// Maxwellian H and the b-factor of a record (cell / ghost / side / wall)
-template <typename T, int D>
-__device__ __forceinline__ T maxwell_h(const T *rec, const T u[3])
-{
-    T c2 = 0;
-#pragma unroll
-    for (int d = 0; d < D; ++d) {
-        T c = u[d] - rec[GR_U + d];
-        c2 += c * c;
-    }
-    return rec[GR_PREF] * gauss<T>(rec[GR_LAM], rec[GR_NL2], c2);
-}
-
 // Shakhov equilibrium f+ = (H + H+, B + B+) of a cell record at velocity u:
 // H+ = kappa (c.q)(2 lam c^2 - D - 2) H,  B+ = kappa (c.q)(2 lam c^2 - D) nb H
 template <typename T, int D, int NC>
@@ -537,7 +524,8 @@ __device__ __forceinline__ void load_uw(const double *__restrict__ uw, int k, do
 // per issued instruction at the rounding of the scalar ones; measured on GB300
 // at 1.87 packed against 3.6 scalar instructions per cycle and SM, so the
 // arithmetic rate is the same but half of the issue slots are free for loads,
-// compares and selects), single values otherwise.  Every contraction is
+// compares and selects), single values otherwise.  Every contraction of the
+// formulas on packs, and of what is evaluated beside them per velocity, is
 // explicit, so all instantiations of a formula round alike.
 template <typename T, int TV> struct Pk {
     static constexpr int W = 1, NP = TV;
@@ -564,6 +552,19 @@ __device__ __forceinline__ float2 padd(float2 a, float2 b) { return __fadd2_rn(a
 __device__ __forceinline__ float pneg(float a) { return -a; }
 __device__ __forceinline__ double pneg(double a) { return -a; }
 __device__ __forceinline__ float2 pneg(float2 a) { return __fmul2_rn(a, make_float2(-1.f, -1.f)); }
+
+// Maxwellian H and the b-factor of a record (cell / ghost / side / wall)
+template <typename T, int D>
+__device__ __forceinline__ T maxwell_h(const T *rec, const T u[3])
+{
+    T c2 = 0;
+#pragma unroll
+    for (int d = 0; d < D; ++d) {
+        const T c = u[d] - rec[GR_U + d];
+        c2 = pfma(c, c, c2);
+    }
+    return rec[GR_PREF] * gauss<T>(rec[GR_LAM], rec[GR_NL2], c2);
+}
 
 // the same value in every element
 template <typename P> __device__ __forceinline__ P pbc(double v);

@@ -1500,7 +1500,7 @@ __device__ __forceinline__ void flux_body(const DevCase<T> &dc, const int bx, co
 #pragma unroll
                     for (int m = 0; m < NC; ++m) {
                         P s = at_face(m, i);
-                        const T out = dt * pel<W>(&s, j % W) - hdt2 * pel<W>(ug[m], j);
+                        const T out = pfma(dt, pel<W>(&s, j % W), -pmul(hdt2, pel<W>(ug[m], j)));
                         pel<W>(F[m], j) = (on >> j & 1) ? unj * out : (m == 0 ? unj * dt : unj * dt * wr[GR_NB]) * H;
                     }
                 }
