@@ -78,8 +78,7 @@ struct DevCase {
     double dt_mu;                 // dt / mu_ref (0: collisionless)
     int limiter;
     int w0_analytic;              // 1: W0 from the analytic half-range moments
-    // velocity grid (padded), FP64 and T copies
-    const double *ud[3], *wd;
+    // velocity grid (padded)
     const T *u[3], *w;
     const T *uw;                  // [nvp][4] (u_x, u_y, u_z or 0, w) packed for one vector load
     // distribution, updated in place: f^n, then f~ (stage 1), then f^{n+1}
@@ -88,18 +87,14 @@ struct DevCase {
     // chunk of velocities: [F][NC][chunk]
     T *flux;
     // macroscopic state
-    double *W, *q, *gradW, *vol;
+    double *W, *q, *gradW;
     double *prim, *primg, *gradprim;  // primitive (rho, U, T) of cells / ghosts, limited gradient
     // least squares (CSR over cells)
     const int *nb_ptr, *nb_id;    // id >= 0: cell, id < 0: ghost -(id+1)
     const double *nb_a_d;
-    const T *nb_a;
     // faces of each cell (CSR): limiter offsets and gather entries
-    const int *cf_ptr, *cf_face;
-    const signed char *cf_side;   // 0 owner, 1 neighbour
-    const double *cf_r_d;
-    const T *cf_r;                // x_f - x_c (periodic image on the neighbour side)
-    const T *cf_coef;             // -sigma S_f / |Omega_c|
+    const int *cf_ptr;
+    const double *cf_r_d;         // x_f - x_c (periodic image on the neighbour side)
     // entries, one per (cell, face) in cf order: gi = {row, face, type + 256
     // (cell owns the face), ghost or wall slot} with row the neighbour cell
     // (interior, periodic) or the cell itself; gf = GEnt<D> values.  nf > 0:
@@ -114,7 +109,7 @@ struct DevCase {
     const int *fL, *fR, *faux;    // owner, neighbour (-1 at boundaries), ghost or wall slot
     const signed char *ftype;
     const double *fn_d, *frL_d, *frR_d;
-    const T *fn, *frL, *frR;      // T copies used inside velocity loops
+    const T *fn, *frL;            // T copies used inside velocity loops
     T dtT;                        // dt in the arithmetic type
     T one;                        // 1 (see psum)
     // ghosts (one per far-field face)
@@ -256,11 +251,6 @@ __device__ __forceinline__ double exp_neg(double x)
 template <typename T> __device__ __forceinline__ T gauss(T lam, T nl2, T c2);
 template <> __device__ __forceinline__ double gauss<double>(double lam, double, double c2) { return exp_neg(-lam * c2); }
 template <> __device__ __forceinline__ float gauss<float>(float, float nl2, float c2) { return ex2_approx(nl2 * c2); }
-
-// a / b: IEEE in FP64, the fast reciprocal-based quotient in FP32
-template <typename T> __device__ __forceinline__ T fdiv(T a, T b);
-template <> __device__ __forceinline__ double fdiv<double>(double a, double b) { return a / b; }
-template <> __device__ __forceinline__ float fdiv<float>(float a, float b) { return __fdividef(a, b); }
 
 template <typename T> __device__ __forceinline__ T mul_rn(T a, T b);
 template <> __device__ __forceinline__ double mul_rn<double>(double a, double b) { return __dmul_rn(a, b); }

@@ -184,7 +184,7 @@ struct Host {
     std::vector<int> perm_i2u, perm_u2i;
     std::vector<int> cf_ptr, cf_face;
     std::vector<signed char> cf_side;
-    std::vector<double> cf_r, cf_coef;
+    std::vector<double> cf_r;
     std::vector<double> gf;          // entry values, GEnt<D>::LEN each
     std::vector<int> gi;             // entry ids, 4 each
     int nf = 0;                      // entries per cell (0: the cells' own counts)
@@ -390,7 +390,6 @@ void preprocess(const ugks_mesh *m, const ugks_params *p, Host &h)
     h.cf_face.resize(ncf);
     h.cf_side.resize(ncf);
     h.cf_r.resize((size_t)ncf * D);
-    h.cf_coef.resize(ncf);
     std::vector<int> fill(C, 0);
     for (int f = 0; f < F; ++f)
         for (int s = 0; s < 2; ++s) {
@@ -400,7 +399,6 @@ void preprocess(const ugks_mesh *m, const ugks_params *p, Host &h)
             h.cf_face[e] = f;
             h.cf_side[e] = (signed char)s;
             for (int d = 0; d < D; ++d) h.cf_r[(size_t)e * D + d] = s == 0 ? h.frL[(size_t)f * D + d] : h.frR[(size_t)f * D + d];
-            h.cf_coef[e] = (s == 0 ? -1.0 : 1.0) * m->face_S[f] / h.vol[c];
         }
 
     // ---- least squares: neighbours across non-wall faces, far-field ghosts
@@ -544,13 +542,11 @@ void fill_case(ugks_case *c, ugks::DevCase<T> &dc, const ugks_mesh *m, const ugk
     dc.w0_analytic = p->w0_analytic ? 1 : 0;
     // velocities, padded with u = 0, w = 0
     for (int d = 0; d < 3; ++d) {
-        dc.ud[d] = nullptr;
         dc.u[d] = nullptr;
     }
     for (int d = 0; d < D; ++d) {
         std::vector<double> ud(c->nvp, 0.0);
         for (int64_t k = 0; k < c->Nv; ++k) ud[k] = v->u[k * D + d];
-        dc.ud[d] = c->upload(ud);
         dc.u[d] = c->upload(cast<T>(ud));
     }
     // tensor-product grid: u_k = (x_i, y_j[, z_l]), k = i + nx (j + ny l), and
@@ -614,7 +610,6 @@ void fill_case(ugks_case *c, ugks::DevCase<T> &dc, const ugks_mesh *m, const ugk
     }
     std::vector<double> wd(c->nvp, 0.0);
     for (int64_t k = 0; k < c->Nv; ++k) wd[k] = v->w[k];
-    dc.wd = c->upload(wd);
     dc.w = c->upload(cast<T>(wd));
     {
         std::vector<T> uw((size_t)c->nvp * 4, T(0));
@@ -656,17 +651,11 @@ void fill_case(ugks_case *c, ugks::DevCase<T> &dc, const ugks_mesh *m, const ugk
     dc.gradprim = (double *)c->dalloc((size_t)c->C * D * M * sizeof(double));
     dc.prim = (double *)c->dalloc((size_t)c->C * M * sizeof(double));
     dc.primg = (double *)c->dalloc((size_t)std::max(c->G, 1) * M * sizeof(double));
-    dc.vol = c->upload(h.vol);
     dc.nb_ptr = c->upload(h.nb_ptr);
     dc.nb_id = c->upload(h.nb_id);
     dc.nb_a_d = c->upload(h.nb_a);
-    dc.nb_a = c->upload(cast<T>(h.nb_a));
     dc.cf_ptr = c->upload(h.cf_ptr);
-    dc.cf_face = c->upload(h.cf_face);
-    dc.cf_side = c->upload(h.cf_side);
     dc.cf_r_d = c->upload(h.cf_r);
-    dc.cf_r = c->upload(cast<T>(h.cf_r));
-    dc.cf_coef = c->upload(cast<T>(h.cf_coef));
     dc.gi = reinterpret_cast<const int4 *>(c->upload(h.gi));
     dc.gf = c->upload(cast<T>(h.gf));
     dc.nf = h.nf;
@@ -682,7 +671,6 @@ void fill_case(ugks_case *c, ugks::DevCase<T> &dc, const ugks_mesh *m, const ugk
     dc.frR_d = c->upload(h.frR);
     dc.fn = c->upload(cast<T>(h.fn));
     dc.frL = c->upload(cast<T>(h.frL));
-    dc.frR = c->upload(cast<T>(h.frR));
     dc.dtT = (T)c->dt;
     dc.one = T(1);
     dc.gface = c->upload(h.gface);
