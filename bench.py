@@ -457,13 +457,13 @@ def _measure(torch, lib, name, case, args, dist, ws, local, steps, warmup, strea
                    "l2": f"inputs larger than L2 (f {info['f_bytes'] / 1e9:.2f} GB per copy)",
                    "w0": "analytic half-range moments" if args.w0_analytic else "discrete half-range sums",
                    "parallelism": f"replicas x{ws}"},
-        "roofline": {"bound": "hbm", "kernel": "k_gather", "achieved": achieved, "peak": peak,
+        "roofline": {"bound": "hbm", "kernel": "k_flux + k_stage1", "achieved": achieved, "peak": peak,
                      "unit": "GB/s", "frac": (achieved / peak) if achieved else None,
                      "traffic": _gather_traffic(name, info["patch_cells"], info["vtile"],
                                                 info["gather_threads"], info["gather_tile_group"]),
                      "peak_kind": peak_kind, "algorithmic_bytes_per_launch": alg_bytes,
                      "launch_ms": g_ms, "group_share": share},
-        "alu_roofline": {"bound": "alu", "kernel": "k_gather", "achieved": alu_achieved, "peak": fp32_peak,
+        "alu_roofline": {"bound": "alu", "kernel": "k_flux + k_stage1", "achieved": alu_achieved, "peak": fp32_peak,
                          "unit": "TFLOP/s",
                          "frac": (alu_achieved / fp32_peak) if (alu_achieved and fp32_peak) else None,
                          "flops_per_cvu": round(flops_cvu, 1), "faces_per_cell": round(nf, 3),

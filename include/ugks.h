@@ -242,9 +242,9 @@ ugks_status ugks_profile_end(ugks_case *c, double *ms, int32_t n, int32_t *steps
 /* Batched stepping of several cases (one GPU).  The cases must share the
  * dimension and precision.  Each batch step runs every kernel once for all cases
  * (block offsets per case), the flux and stage-1 kernels once per velocity chunk
- * and per (velocity tile, faces per cell) present in the batch, so a
- * step is about a dozen launches whatever the number of cases.  The whole
- * step is captured once as a CUDA graph on `stream` (cudaStream_t, NULL: a
+ * and per (velocity tile, faces per cell) present in the batch, so a step is
+ * about ten launches and two per chunk and such group, whatever the number of
+ * cases.  The whole step is captured once as a CUDA graph on `stream` (cudaStream_t, NULL: a
  * stream of the batch's own) and replayed.  Results are bit-identical to
  * stepping each case alone with ugks_step.  The cases stay owned by the
  * caller and must outlive the batch; ugks_batch_step advances each case's

@@ -1,5 +1,5 @@
 // ugks_host.cu -- C ABI of the UGKS library: validation, host preprocessing
-// (cell ordering, least-squares coefficients, gather patches), device state and
+// (cell ordering, least-squares coefficients, face entries), device state and
 // the launch sequence of a time step.  The numerics live in ugks_kernels.cu.
 #include "../../include/ugks.h"
 #include "ugks_device.cuh"
@@ -110,7 +110,7 @@ struct ugks_case {
         return p;
     }
 
-    // frees one block of dalloc (the patch arrays of a tiling that is replaced)
+    // frees one block of dalloc (a halo list that is replaced)
     void dfree(const void *p)
     {
         if (!p) return;

@@ -1403,12 +1403,12 @@ __global__ void __launch_bounds__(256) k_wall_sum_batch(const DevCase<T> *__rest
 // most of its instructions on slopes recomputed for the neighbours of a patch
 // (2.2 evaluations per cell of 48-cell patches), on fluxes evaluated from both
 // sides of a face and on selects between the sides: 897 thread instructions
-// per cell-velocity for tetrahedra against 286 of the two kernels here
-// (k_flux 194, k_stage1 92 at 256-velocity groups).  The price is the flux
+// per cell-velocity for tetrahedra against 295 of the two kernels here
+// (k_flux 227, k_stage1 68 at 1,024-velocity groups).  The price is the flux
 // buffer, F/C values per cell and velocity written once and read twice, which
 // L2 and HBM have room for.  107k-cell tetrahedral mesh x 4,568 velocities,
 // FP32: 17.2 -> 7.95 ms; 24k cells x 28^3: 18.4 -> 8.2 ms; 30k triangles x
-// 60x50: 3.18 -> 1.55 ms; FP64, 8k triangles x 60x50: 21.0 -> 13.4 ms.
+// 60x50: 3.18 -> 1.55 ms; FP64, 8k triangles x 60x50: 21.0 -> 14.8 ms.
 // A chunk bounds the buffer; velocities of different chunks do not meet, so
 // the update is in place.
 
@@ -1419,9 +1419,10 @@ __global__ void __launch_bounds__(256) k_wall_sum_batch(const DevCase<T> *__rest
 // 9.1 against 12.4 ms of both kernels).  The next cell's rows, entries and
 // records are copied to shared memory while a cell is worked on (StagedCell):
 // with loads at their use the 16 warps of an SM waited for memory in 3.8 of 8.9
-// cycles per instruction, now in 1.3 of 7.1, and both kernels went from 8.14 to
-// 7.35 ms on that mesh and from 0.266 to 0.215 on 2,145 hexahedra x 4,080.
-// Bound: instruction issue (54 % of the issue slots, FMA pipe 51 %, DRAM 14 %).
+// cycles per instruction, now its 19 in 1.5 of 8.2, and both kernels went from 8.14
+// to 7.35 ms on that mesh and from 0.266 to 0.215 on 2,145 hexahedra x 4,080.
+// Bound: instruction issue (45,796 tetrahedra x 1,024 velocities: 58 % of the issue
+// slots, FMA pipe 55 %, DRAM 18 %; 15,081 triangles: 54, 50 and 19 %).
 constexpr int FLUX_THREADS = 128;
 
 template <typename T, int D, int NC, int TV, int NF>
@@ -1673,8 +1674,8 @@ template <typename T, int D, int NC, int TV, int NF> constexpr int flux_smem()
 // CTAs of four warps: 20 warps fit an SM at 96 registers (tetrahedra and
 // hexahedra, FP32 at TV = 4) and 16 at the 120 of the 2D kernels, against 16 in
 // CTAs of eight, and the last wave ends sooner.  Both kernels, 107k-cell
-// tetrahedral mesh 7.12 -> 6.59 ms (6.88 at four CTAs per SM), 24k cells x 28^3 7.73 -> 7.32,
-// 30k-cell triangulation 1.52 -> 1.47 (1.56 at five CTAs per SM, which spill in
+// tetrahedral mesh 7.12 -> 6.63 ms (6.88 at four CTAs per SM), 24k cells x 28^3 7.73 -> 7.38,
+// 30k-cell triangulation 1.52 -> 1.49 (1.56 at five CTAs per SM, which spill in
 // 2D); CTAs of six warps 7.11, 7.84 and 1.57, of two 6.62, 7.34 and 1.55.
 template <typename T, int D, int TV> constexpr int flux_min_ctas() { return sizeof(T) == 4 && TV == 4 ? (D == 3 ? 5 : 4) : 0; }
 
@@ -1739,7 +1740,9 @@ template <> struct MomentSum<float2> {
 // iterations ahead by asynchronous copies (a lane reads back what it copied, so
 // no barrier): without it a warp had the loads of one iteration in flight and
 // waited for them in 11 of 15 cycles per instruction (7.35 -> 7.12 ms of both
-// kernels on the 107k-cell mesh, 1.56 -> 1.52 on the 30k-cell triangulation).
+// kernels on the 107k-cell mesh, 1.56 -> 1.52 on the 30k-cell triangulation); now it
+// waits in 2.9 of 8.0 cycles for tetrahedra (DRAM 55 %) and 4.8 of 9.5 for triangles
+// (65 %).
 template <typename T, int NC, int NF> constexpr int stage1_stages()
 {
     return (NF + 1) * NC * 4 * (int)sizeof(T) * 32 * 8 * 3 <= 64 * 1024 ? 3 : 2;

@@ -2,6 +2,8 @@
 a group depends on the velocity set alone, whatever the flux buffer of the mesh can hold,
 so that subdomains sum the moments of a cell as the whole mesh does, and
 ugks_info reports the group that is used."""
+import functools
+
 import numpy as np
 import pytest
 
@@ -19,6 +21,16 @@ def _built():
     build.build()
 
 
+@functools.lru_cache(maxsize=None)
+def _case(name):
+    if name == "cylinder":
+        return cs.cylinder_case(n_cells=5000, nvx=32, nvy=30, mach=3.0)
+    n, nv = {"box": ((14, 13, 14), 12), "box 3": ((20, 20, 20), 3), "box 8": ((20, 20, 20), 8)}[name]
+    mesh = cs.hex_mesh(*n)
+    return {"mesh": mesh, "vgrid": cs.cartesian_vgrid((nv,) * 3, (-4.0,) * 3, (4.0,) * 3),
+            "params": cs.params(0.1, walls=[{"T": 1.1, "U": [0.2, 0.0, 0.0]}]), "init": cs.smooth_state(mesh, 3, 0.1)}
+
+
 def _perturbed(case, precision):
     g = _lib.Case(case["mesh"], case["vgrid"], case["params"], case["init"], precision=precision, patch_cells=16)
     f, W = g.state()
@@ -29,17 +41,16 @@ def _perturbed(case, precision):
 
 @pytest.mark.parametrize("name,precision,vtile,group,chunks", [
     ("cylinder", _lib.FP32, 64, 15, 2), ("cylinder", _lib.FP32, 32, 28, 3), ("cylinder", _lib.FP64, 32, 1024, 2),
-    ("cylinder", _lib.FP64, 64, 14, 3), ("cylinder", _lib.FP32, 64, 0, 2), ("sphere", _lib.FP64, 32, 0, 2),
-    ("sphere", _lib.FP32, 64, 1024, 2), ("sphere", _lib.FP32, 128, 12, 3),
-    ("sphere", _lib.FP64, 32, 50, 3), ("sphere", _lib.FP64, 64, 1024, 2)])
+    ("cylinder", _lib.FP64, 64, 14, 3), ("cylinder", _lib.FP32, 64, 0, 2), ("box", _lib.FP64, 32, 0, 4),
+    ("box", _lib.FP32, 64, 1024, 4), ("box", _lib.FP32, 128, 12, 4), ("box", _lib.FP64, 32, 50, 5),
+    ("box", _lib.FP64, 64, 1024, 4)])
 def test_group_is_used_on_every_mesh(name, precision, vtile, group, chunks):
     """Groups of which the whole mesh's flux buffer holds a part (``chunks`` per
     step in all, the last group shorter in some) and a subdomain's a part or
     all: three decomposed steps bitwise equal the undivided ones, also in W,
     and the reported group is the caller's, at most all tiles (0: up to 1,024
     velocities, equal groups in multiples of 128)."""
-    case = (cs.cylinder_case(n_cells=5000, nvx=32, nvy=30, mach=3.0) if name == "cylinder" else
-            cs.sphere_case(n_cells=4000, nv=12, vmax=6.0, mach=2.0))
+    case = _case(name)
     mesh, vg, pr = case["mesh"], case["vgrid"], case["params"]
     case = dict(case, params=dict(pr, dt=_lib.cfl_dt(mesh, vg, pr["cfl"])))
     tiling = {"patch_cells": 32, "vtile": vtile, "threads": 256, "tile_group": group}
@@ -48,7 +59,7 @@ def test_group_is_used_on_every_mesh(name, precision, vtile, group, chunks):
     info = full.info()
     assert info["kernel_launches_per_step"] == 10 + 2 * chunks
     tiles = -(-info["nv_pad"] // vtile)
-    used = min(group, tiles) if group else {"cylinder": 960, "sphere": 896}[name] // vtile
+    used = min(group, tiles) if group else {"cylinder": 960, "box": 896}[name] // vtile
     for c in [full] + dec.cases:
         assert c.info()["gather_tile_group"] == used
     f, W = _perturbed(case, precision)
@@ -95,13 +106,8 @@ def test_footprint_estimate_bounds_the_device_bytes(precision, tiling):
     """The server admits by an estimate that is no less than what a case holds:
     two- and three-dimensional requests of few and of many velocities."""
     import ctypes as ct
-    box = cs.hex_mesh(20, 20, 20)
-    boxes = [{"mesh": box, "vgrid": cs.cartesian_vgrid((n,) * 3, (-4.0,) * 3, (4.0,) * 3),
-              "params": cs.params(0.1, walls=[{"T": 1.0, "U": [0.0, 0.0, 0.0]}] * 6),
-              "init": cs.smooth_state(box, 3, 0.1)} for n in (3, 8)]
-    for case in boxes + [cs.cavity_case(n=60, nv=2), cs.cavity_case(n=60, nv=24),
-                         cs.cylinder_case(n_cells=8000, nvx=30, nvy=25, mach=3.0),
-                         cs.sphere_case(n_cells=8000, nv=10, vmax=6.0, mach=2.0)]:
+    for case in (_case("box 3"), _case("box 8"), cs.cavity_case(n=60, nv=2), cs.cavity_case(n=60, nv=24),
+                 _case("cylinder")):
         srv = _lib.Server(1 << 40, 8, 10)
         (m, v, p), keep = _lib.make_structs(case["mesh"], case["vgrid"], case["params"], case["init"], precision,
                                             **tiling)
