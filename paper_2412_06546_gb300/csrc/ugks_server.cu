@@ -57,11 +57,11 @@ struct Request {
     std::vector<double> rho, U, T, q;   // results of a finished request
 };
 
-// Device bytes a case will hold, from its sizes (an upper bound of what
-// ugks_create allocates: f, the flux buffer, which is at most 9/8 of a copy of f, or
-// up to 4 MB or 128 velocities where that is more, with a fixed tiling also the
-// lane sums of stage 1 or as many bytes more of the buffer, FP64 cell / face arrays
-// and records).
+// Device bytes a case will hold, from its sizes, an upper bound of what ugks_create
+// allocates: f and the flux buffer by set_chunks' rules (9/8 of a copy of f, or up to
+// 4 MB or 128 velocities where that is more; with a fixed tiling the fluxes of a group
+// where they exceed that by less than the lane sums of stage 1, else these), and, with
+// an eighth to spare, FP64 cell / face arrays and records.
 size_t footprint_estimate(const Request &r)
 {
     const int D = r.D, M = D + 2, NC = D == 2 ? 2 : 1;
@@ -69,15 +69,20 @@ size_t footprint_estimate(const Request &r)
     const size_t nvp = (size_t)((r.Nv + 127) / 128 * 128);
     const size_t C = (size_t)r.C, F = (size_t)std::max<int64_t>(r.F, 1);
     const size_t f = C * NC * nvp * s, vel = F * NC * s;
-    size_t b = f + std::max({f + f / 8, std::min<size_t>((size_t)4 << 20, vel * nvp), vel * 128});   // f, fluxes
-    if (r.params.patch_cells > 0 || r.params.gather_tile_group > 0) b += C * M * 32 * (s == 8 ? 8 : 16);
-    b += C * (size_t)(M * 2 + D + D * M * 2 + 8) * 8;                  // W, q, prim, gradients, vol
+    const size_t most = std::max(f + f / 8, (size_t)4 << 20);
+    size_t fluxes = std::max(std::min(most, vel * nvp), vel * 128);
+    if (r.params.patch_cells > 0 || r.params.gather_tile_group > 0) {
+        const size_t tile = r.params.vtile > 0 ? r.params.vtile : s == 8 ? 32 : 64;
+        const size_t group = std::min(nvp, r.params.gather_tile_group > 0 ? r.params.gather_tile_group * tile : 1024);
+        fluxes = std::max(fluxes, std::min(vel * group, most + C * M * 32 * (s == 8 ? 8 : 16)));
+    }
+    size_t b = C * (size_t)(M * 2 + D + D * M * 2 + 8) * 8;                  // W, q, prim, gradients, vol
     b += C * 2 * 12 * s + C * (nvp / 32 + 1) * M * s;                  // records, residual partials
     b += F * (size_t)(40 * s + 24 * s + 16 * s + (D * M + D + D + M + M + 5) * 8 + 60 * 8 + 64);
     b += 2 * F * (size_t)(8 * D + 24) + C * 64 + nvp * 64;             // geometry, LSQ, patches
     b += 2 * F * (size_t)(16 + 16 * s);                                // entries
     b += (size_t)64 * 256 * 40;                                        // allocation rounding
-    return b + b / 8;
+    return f + fluxes + b + b / 8;
 }
 
 }  // namespace

@@ -119,3 +119,17 @@ def test_footprint_estimate_bounds_the_device_bytes(precision, tiling):
         g = _lib.Case(case["mesh"], case["vgrid"], case["params"], case["init"], precision=precision, **tiling)
         assert g.info()["device_bytes"] <= estimate
         g.close()
+
+
+@pytest.mark.parametrize("case,fp32,fp64", [
+    (lambda: cs.cavity_case(n=60, nv=2), 26138376, 43120296), (lambda: cs.cavity_case(n=60, nv=24), 56104200, 103015080),
+    (lambda: cs.cylinder_case(n_cells=8000, nvx=30, nvy=25, mach=3.0), 137878443, 260162397)])
+def test_footprint_estimate_admits_what_it_admitted(case, fp32, fp64):
+    """Automatic tilings: no more than when the flux buffer was bounded by a copy of
+    f, so that no budget that held a request refuses it."""
+    c = case()
+    for precision, was in ((_lib.FP32, fp32), (_lib.FP64, fp64)):
+        srv = _lib.Server(1 << 40, 8, 10)
+        estimate = srv.poll(srv.submit(c, 1e-12, 1, precision=precision))["footprint_bytes"]
+        srv.close()
+        assert estimate <= was
